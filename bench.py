@@ -37,12 +37,11 @@ UNIT = "particle-substeps/s"
 FLOPS_PER_UNIT = {1: (447.2, 863.2), 2: (2544.4, 5005.0), 3: (6293.5, 12860.9),
                   4: (11694.7, 24711.2)}
 FP32_LANES = 128                    # FP32 lanes per SM; 1 FMA = 2 FLOP
-# DRAM bytes (read + write) per launch of a rollout kernel (for the reverse
-# sweep: its replay and sweep launches together), from one cold-cache ncu
+# DRAM bytes (read + write) per launch of a rollout kernel, from one cold-cache ncu
 # capture of the workload, valid while the kernel sources are unchanged
 # (sha256 prefix over the rollout sources at capture time).
-TRAFFIC = {("pusher3_h6", "rollout_adj"): ("243c7f35e3b01a4a", 179.97e6)}   # replay + sweep
-ROLLOUT_SOURCES = ("rollout.cuh", "adjoint_time.cu")
+TRAFFIC = {}
+ROLLOUT_SOURCES = ("rollout.cuh", "block_team.cuh", "rollout_kernels.cuh", "adjoint_time.cu")
 
 
 def peaks():
@@ -397,7 +396,7 @@ def secondary_workload(name, seed, flush, stream, steps=5, warmup=3):
     prob = S.Problem(P, init, goal, P["N"], stream.cuda_stream)
     ms = time_solves(prob, P, P["N"], seed, steps, warmup, flush, stream)
     units = P["N"] * P["H"] * P["T"] * P["svgd_iters"]
-    mode = {S.STAMP_ADJ_TIME_PARALLEL: "time-parallel", S.STAMP_ADJ_REPLAY: "segment replay + sequential",
+    mode = {S.STAMP_ADJ_TIME_PARALLEL: "time-parallel", S.STAMP_ADJ_REPLAY: "sequential on the forward's rows",
             S.STAMP_ADJ_SEQUENTIAL: "sequential"}[prob.adjoint_mode(P["N"])]
     prob.close()
     return {"workload": f"{name}: {P['n_blocks']} block(s), H={P['H']}, T={P['T']}, N={P['N']}, "
@@ -560,7 +559,7 @@ def main():
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": dict(workload_config(args, P),
                            reverse_sweep={S.STAMP_ADJ_TIME_PARALLEL: "time-parallel",
-                                          S.STAMP_ADJ_REPLAY: "segment replay + sequential",
+                                          S.STAMP_ADJ_REPLAY: "sequential on the forward's rows",
                                           S.STAMP_ADJ_SEQUENTIAL: "sequential"}.get(adj_mode, str(adj_mode))),
             "roofline": roof, "cpu_baseline": cpu,
             "clocks": clocks, "e2e": e2e,

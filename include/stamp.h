@@ -206,7 +206,7 @@ stamp_status stamp_sync(stamp_problem* prob);
  * totals are gathered at stamp_sync / stamp_solve.  Kernel ids: */
 enum {
     STAMP_K_ROLLOUT_FWD = 0,  /* forward rollout (relaxed or hard) */
-    STAMP_K_ROLLOUT_ADJ = 1,  /* reverse sweep (time-parallel or replay: all its launches together) */
+    STAMP_K_ROLLOUT_ADJ = 1,  /* reverse sweep (time-parallel: all its launches together) */
     STAMP_K_PAIRWISE = 2,     /* pairwise distances + first median digit */
     STAMP_K_MEDIAN = 3,       /* remaining median digits */
     STAMP_K_PHI = 4,          /* Stein direction */
@@ -255,17 +255,14 @@ stamp_status stamp_set_overlap(stamp_problem* prob, int enable);
  * STAMP_ADJ_SEQUENTIAL: each particle's team differentiates substep after
  * substep, recomputing each segment of ckpt_every substeps from its
  * checkpoint on the same serial path.
- * STAMP_ADJ_REPLAY applies to ckpt_every > 1: one launch rebuilds the states
- * before every substep from the checkpoints for all (particle, segment)
- * pairs at once (the segments are independent given their checkpoints),
- * into a scratch tape of interval 1 ((H*T + 1) x N x S floats, allocated at
- * create when at most 4 GiB); then the sequential sweep runs on that tape
- * with nothing to recompute.  The forward still stores only every
- * ckpt_every-th state.
+ * STAMP_ADJ_REPLAY applies to ckpt_every > 1: the sweep reads the state
+ * before every substep from rows that the forward left beside its checkpoint
+ * tape (scratch of (H*T + 1) x N x S floats, allocated at create when at most
+ * 4 GiB) and recomputes nothing.
  * STAMP_ADJ_AUTO (the default): time-parallel where it applies, for up to
  * 3072 particles (beyond that the sequential teams fill the GPU and the
- * Jacobians' extra arithmetic costs more than it saves), else the replay
- * where it applies, else sequential.
+ * Jacobians' extra arithmetic costs more than it saves), else
+ * STAMP_ADJ_REPLAY where it applies, else sequential.
  * All sweeps give the gradient of the same float32 simulation, with sums
  * taken in a different order. */
 enum { STAMP_ADJ_SEQUENTIAL = 0, STAMP_ADJ_TIME_PARALLEL = 1, STAMP_ADJ_AUTO = 2,
@@ -286,11 +283,15 @@ stamp_status stamp_get_adjoint_mode(stamp_problem* prob, int N, int* mode);
  * calls run normally. */
 stamp_status stamp_inject_wait_timeout(stamp_problem* prob);
 
-/* Lanes per particle used by the rollout kernels (1,2,4,8,16,32; 0 = automatic). */
+/* Lanes per particle used by the rollout kernels (one block 1, 2, 4; two
+ * blocks 2..16; three and four blocks 8..32; 0 = automatic, by the number of
+ * particles).  A particle works on 1, 2 or 4 lanes per block; lanes beyond
+ * four per block idle.  The results do not depend on the width, except for the
+ * order in which forces between blocks are summed. */
 stamp_status stamp_set_lanes(stamp_problem* prob, int fwd_lanes, int adj_lanes);
-/* Lanes per (particle, segment) team of the segment replay (STAMP_ADJ_REPLAY):
- * one block 1, 2, 4; two blocks 2..16; three blocks 2..32; four blocks
- * 4..32; 0 = automatic. */
+/* Accepted as before (one block 1, 2, 4; two blocks 2..16; three blocks 2..32;
+ * four blocks 4..32; 0 = automatic) and without effect: STAMP_ADJ_REPLAY has
+ * no launch of its own that rebuilds states. */
 stamp_status stamp_set_replay_lanes(stamp_problem* prob, int lanes);
 
 /* Stein step without any device allocation.  The paper has no counterpart:

@@ -5,8 +5,8 @@
 For each interval C (T % C == 0) and each reverse sweep that applies (the
 automatic choice, and the sequential sweep when that differs) prints one
 JSON line: the checkpoint tape in HBM, (H*T/C + 1) * N * S * 4 bytes; the
-segment replay's scratch, when it runs ((H*T + 1) * N * S floats of states
-plus H*T * N * 2 n_blocks of yaw sines and cosines); and the forward and
+scratch of the forward's per-substep rows, where the sweep reads them
+((H*T + 1) * N * S floats); and the forward and
 reverse-sweep times (CUDA events, mean of 20 launches after 3 warm-up
 launches) on the workload's particles at initialisation.
 """
@@ -22,7 +22,7 @@ from paper_2310_01775_gb300 import workloads as W
 
 
 MODES = {S.STAMP_ADJ_SEQUENTIAL: "sequential", S.STAMP_ADJ_TIME_PARALLEL: "time-parallel",
-         S.STAMP_ADJ_REPLAY: "segment replay"}
+         S.STAMP_ADJ_REPLAY: "stored rows"}
 
 
 def sweep(name: str, intervals):
@@ -60,7 +60,7 @@ def sweep(name: str, intervals):
         HT = P["H"] * P["T"]
         rec = dict(workload=name, ckpt_every=C, reverse_sweep=MODES[used],
                    tape_bytes=(HT // C + 1) * N * prob.S * 4,
-                   replay_scratch_bytes=((HT + 1) * N * prob.S + HT * N * 2 * P["n_blocks"]) * 4
+                   rows_scratch_bytes=(HT + 1) * N * prob.S * 4
                    if used == S.STAMP_ADJ_REPLAY else 0,
                    fwd_ms=t_f / 20, adj_ms=t_a / 20)
         print(json.dumps(rec), flush=True)

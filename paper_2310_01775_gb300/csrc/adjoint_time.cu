@@ -24,6 +24,7 @@
 // reverse per pusher -- the force rows -- and the torque row by linearity,
 // so both sweeps take the same derivatives and differ only in rounding.
 #include "async_copy.cuh"
+#include "block_team.cuh"
 #include "rollout.cuh"
 
 namespace stamp {
@@ -335,15 +336,15 @@ __global__ void __launch_bounds__(128) jac_kernel(const SimConst sc, const Rollo
     const float z[4] = {r[0], r[a.N], r[2 * a.N], r[3 * a.N]};
     const float off = sc.off_max * r[4 * a.N];
     const float dist = sc.dist_max * r[5 * a.N];
-    Slots<1, 1> sl;
-    make_slots<1, 1>(sc, s0, 0, z, off, dist, sl);
-    float cs[1], sn[1];
-    trig(s, cs, sn);
+    Own<4> o;   // the four pushers of the one block
+    place(sc, Quad<1, 1>{}, One{s0.x[0], s0.y[0], s0.ph[0], 0.f, 0.f, 0.f}, off, dist, o);
+    float cs, sn;
+    yaw_sincos(s.ph[0], &sn, &cs);
     float cph0, sph0;
     yaw_sincos(s0.ph[0], &sph0, &cph0);
     const float j1 = (float)(j + 1), step = dist / (float)sc.T;
     float row[kRow];
-    pair_row(sc, s, cs[0], sn[0], sl.p0x, sl.p0y, sl.dx, sl.dy, sl.w, j1, step, cph0, sph0, off, row);
+    pair_row(sc, s, cs, sn, o.p0x, o.p0y, o.dx, o.dy, z, j1, step, cph0, sph0, off, row);
     float4* out = reinterpret_cast<float4*>(coef_row(coef, HT, i, t));
 #pragma unroll
     for (int v = 0; v < kRow / 4; ++v)
@@ -489,7 +490,7 @@ __global__ void __launch_bounds__(32) scan_kernel(const SimConst sc, const Rollo
             const float* r = rel + (size_t)k * kRel * a.N + i;
             const float zl = r[lane * a.N], tu = r[4 * a.N], sg = r[5 * a.N];
             adist += 2.f * sc.w_push * (sc.dist_max * sg);
-            const float zaz = team_sum<4>(zl * az);
+            const float zaz = lanes_sum<4>(zl * az);
             if (on) {
                 float* gr = a.grad + (size_t)i * sc.D + (size_t)k * 6;
                 const float gz = hard ? 0.f : -(zl * (az - zaz) * sc.inv_tau);
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(32) scan_kernel(const SimConst sc, const Rollo
         return;
     }
     // an overflowed reverse sweep gives the particle a zero gradient, and is counted
-    bad = team_sum<4>(bad ? 1.f : 0.f) > 0.f;
+    bad = lanes_sum<4>(bad ? 1.f : 0.f) > 0.f;
     if (on && bad) {
         for (int q = lane; q < sc.D; q += 4) a.grad[(size_t)i * sc.D + q] = 0.f;
         if (lane == 0 && a.dropped) atomicAdd(a.dropped, 1ull);

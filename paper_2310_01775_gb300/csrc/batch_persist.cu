@@ -33,6 +33,7 @@
 // block count); the Stein blocks follow in the order the host expects the
 // instances' rollouts to finish.  Every per-instance buffer starts on a
 // 128-byte boundary, so no cache line is shared by two instances' data.
+#include "block_team.cuh"
 #include "rollout.cuh"
 #include "svgd_bodies.cuh"
 
@@ -99,7 +100,7 @@ __device__ __forceinline__ void cta_signal(unsigned* c) {
 template <int NB>
 __device__ __forceinline__ void roll_warp(const SimConst& sc0, const PersistArgs& p, int g,
                                           int first, float2* wseg, int phase) {
-    constexpr int L = persist_lanes(NB);
+    constexpr int L = persist_lanes(NB), QL = L / rollout::team_groups(NB);
     const BatchInst& in = p.inst[g];
     SimConst sc = sc0;
     sc.H = in.H;
@@ -127,10 +128,10 @@ __device__ __forceinline__ void roll_warp(const SimConst& sc0, const PersistArgs
     const bool on = i < in.N;
     if (!on) i = in.N - 1;   // surplus teams shadow the last particle, store nothing
     if (phase == 0)
-        rollout::fwd_team<NB, L>(sc, a, i, on, lane32 & (L - 1));
+        rollout::fwd_block_team<NB, QL>(sc, a, i, on);
     else
-        rollout::adj_team<NB, L, true>(sc, a, i, on, lane32 & (L - 1),
-                                       wseg + (size_t)(lane32 / L) * rollout::seg_stride<NB>(sc.C));
+        rollout::adj_block_team<NB, QL, true>(sc, a, i, on,
+                                              wseg + (size_t)(lane32 / L) * rollout::seg_stride<NB>(sc.C));
 }
 
 // Adam (Kingma & Ba 2015) on elements [chunk*kPersistAdamChunk, ...) of instance s.

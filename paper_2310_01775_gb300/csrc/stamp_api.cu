@@ -70,16 +70,15 @@ struct stamp_problem {
     int last_n = 0, last_iter = 0, last_hard = 0, last_particle0 = 0;
     unsigned long long last_seed = 0;
     const float* last_theta = nullptr;
-    int fwd_lanes = 0, adj_lanes = 0, replay_lanes = 0;
+    int fwd_lanes = 0, adj_lanes = 0;
     // one-block reverse sweep as a linear recurrence in time (checkpoint
     // interval 1): its scratch exists when the problem qualifies
     int adj_mode = STAMP_ADJ_AUTO;
     float *pit_rel = nullptr, *pit_coef = nullptr;
     bool pit_ok = false;
-    // segment replay (checkpoint interval > 1): the per-substep states of the
-    // last forward, rebuilt in parallel, then swept at interval 1
+    // checkpoint interval > 1: the per-substep states the last forward left
+    // beside its checkpoints, swept at interval 1
     float* full = nullptr;
-    float2* full_trig = nullptr;   // the replayed states' yaw (cos, sin)
     bool replay_ok = false;
     // the bandwidth (pairwise distances + median) depends on theta only: the
     // solves run it on a second stream beside the rollouts
@@ -187,9 +186,9 @@ bool time_parallel(const stamp_problem* p, int N) {
     return p->adj_mode == STAMP_ADJ_TIME_PARALLEL || N <= kTimeParallelMaxN;
 }
 
-// The sweep a call with N particles runs: time-parallel (above), else the
-// segment replay where its scratch exists (checkpoint interval > 1) unless
-// the sequential sweep was asked for, else sequential.
+// The sweep a call with N particles runs: time-parallel (above), else on the
+// forward's rows where they exist (checkpoint interval > 1) unless the
+// sequential sweep was asked for, else sequential.
 int adjoint_kind(const stamp_problem* p, int N) {
     if (time_parallel(p, N)) return STAMP_ADJ_TIME_PARALLEL;
     if (p->replay_ok && p->adj_mode != STAMP_ADJ_SEQUENTIAL) return STAMP_ADJ_REPLAY;
@@ -204,6 +203,7 @@ stamp_status fwd(stamp_problem* p, const float* theta, int N, unsigned long long
     a.tape = p->tape; a.cost = cost; a.final_state = final_state; a.stats_min = stats_word;
     a.init_states = init_states;
     a.particle0 = p->particle0;
+    a.full = p->full;
     const int lanes = lanes_for(p, N, false);
     STAMP_TRY(timed(p, STAMP_K_ROLLOUT_FWD,
                     [&] { return stamp::launch_rollout_fwd(p->sc, a, lanes, p->stream); }));
@@ -224,20 +224,14 @@ stamp_status adj(stamp_problem* p, const float* theta, int N, float* grad) {
             return stamp::launch_adjoint_time(p->sc, a, p->pit_rel, p->pit_coef, p->flag, p->stream);
         });
     const int lanes = lanes_for(p, N, true);
-    if (kind == STAMP_ADJ_REPLAY)
-        return timed(p, STAMP_K_ROLLOUT_ADJ, [&] {
-            stamp::RolloutArgs ar = a;
-            ar.trig = p->full_trig;
-            const int rl = p->replay_lanes ? p->replay_lanes : stamp::replay_lanes(p->sc.nb);
-            cudaError_t e = stamp::launch_replay(p->sc, ar, rl, p->full, p->stream);
-            if (e != cudaSuccess) return e;
-            SimConst sc1 = p->sc;          // the rebuilt tape has interval 1
-            sc1.C = 1;
-            sc1.n_ckpt = sc1.H * sc1.T;
-            stamp::RolloutArgs a1 = ar;
-            a1.tape = p->full;
-            return stamp::launch_rollout_adj(sc1, a1, lanes, p->stream);
-        });
+    if (kind == STAMP_ADJ_REPLAY) {   // the forward's rows: a tape of interval 1
+        SimConst sc1 = p->sc;
+        sc1.C = 1;
+        sc1.n_ckpt = sc1.H * sc1.T;
+        a.tape = p->full;
+        return timed(p, STAMP_K_ROLLOUT_ADJ,
+                     [&] { return stamp::launch_rollout_adj(sc1, a, lanes, p->stream); });
+    }
     return timed(p, STAMP_K_ROLLOUT_ADJ,
                  [&] { return stamp::launch_rollout_adj(p->sc, a, lanes, p->stream); });
 }
@@ -487,17 +481,27 @@ bool lanes_supported(int nb, int lanes) {
     return false;
 }
 
-// Lanes per particle, from sweeps on GB300 at 2048 particles (H = 6, C = 25,
-// segment replay): one block 4/4; two blocks forward 8 (0.28 ms; 0.38 at 4,
-// 0.40 at 16), sweep 8 (0.50 ms; 0.60 at 16); three blocks forward 8
-// (0.75 ms; 0.82 at 16, 0.90 at 32), sweep 8 (1.28 ms; 1.38 at 16, 2.11 at
-// 32); four blocks forward 16 (1.28 ms; 1.39 at 8, 1.46 at 32), sweep 16
-// (2.37 ms; 3.09 at 8, 2.82 at 32).
+// Lanes per particle: 4 per block while that gives each of the SM's four
+// schedulers at most one warp (the serial chain of a substep is the time), 2
+// per block up to two warps a scheduler, then 1 (the instruction count is).
+// One block keeps 4 up to two warps; four blocks keep 4 up to two and never go
+// to 1 (pairs of blocks in contact, frequent there, cost the narrower teams
+// more).  Forward / reverse sweep on GB300, H = 4, T = 100, C = 1, us, at 4, 2
+// and 1 lanes per block:
+//   one block     N = 4096   107/131  125/187  172/281;  N = 16384  176/337  148/269  174/292
+//   two blocks    N = 2048   115/154  121/191  158/266;  N = 4096   134/209  121/195  160/266
+//                 N = 16384  352/601  279/583  238/435
+//   three blocks  N = 1024   101/160  133/191  164/278;  N = 2048   129/221  133/196  166/278
+//                 N = 8192   366/736  319/573  256/452
+//   four blocks   N = 2048   280/402  289/390  396/615;  N = 4096   346/594  362/517  385/594
 int default_lanes(int nb, int N, bool adjoint) {
-    (void)N;
-    if (nb == 1) return 4;
-    if (nb == 2 || nb == 3) return 8;
-    return 16;
+    (void)adjoint;
+    const int groups = nb <= 2 ? nb : 4;
+    const long long schedulers = 4ll * sm_count();
+    const long long w4 = ((long long)N * 4 * groups + 31) / 32;   // warps at 4 lanes per block
+    if (w4 <= schedulers || ((nb == 1 || nb == 4) && w4 <= 2 * schedulers)) return 4 * groups;
+    if (nb == 4 || w4 <= 4 * schedulers) return 2 * groups;
+    return groups;
 }
 
 cudaError_t launch_rollout_fwd(const SimConst& sc, const RolloutArgs& a, int lanes, cudaStream_t st) {
@@ -506,21 +510,6 @@ cudaError_t launch_rollout_fwd(const SimConst& sc, const RolloutArgs& a, int lan
         case 2: return launch_rollout_nb2(sc, a, lanes, false, st);
         case 3: return launch_rollout_nb3(sc, a, lanes, false, st);
         case 4: return launch_rollout_nb4(sc, a, lanes, false, st);
-    }
-    return cudaErrorInvalidValue;
-}
-
-// The fewest lanes each block count supports: the replay is throughput
-// bound, and fewer lanes integrate the state less redundantly.
-int replay_lanes(int nb) { return nb == 1 ? 1 : nb == 2 ? 2 : nb == 3 ? 4 : 8; }
-
-cudaError_t launch_replay(const SimConst& sc, const RolloutArgs& a, int lanes, float* full,
-                          cudaStream_t st) {
-    switch (sc.nb) {
-        case 1: return launch_replay_nb1(sc, a, lanes, full, st);
-        case 2: return launch_replay_nb2(sc, a, lanes, full, st);
-        case 3: return launch_replay_nb3(sc, a, lanes, full, st);
-        case 4: return launch_replay_nb4(sc, a, lanes, full, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -645,7 +634,6 @@ stamp_status stamp_problem_create(const stamp_problem_desc* d, const float* init
         {(void**)&p->pit_rel, pit ? stamp::adjoint_time_rel_floats(max_particles, sc.H) * sizeof(float) : 0},
         {(void**)&p->pit_coef, pit ? pit_coef_bytes : 0},
         {(void**)&p->full, replay ? full_bytes : 0},
-        {(void**)&p->full_trig, replay ? (size_t)sc.H * sc.T * n * sc.nb * sizeof(float2) : 0},
     };
     p->pit_ok = pit;
     p->replay_ok = replay;
@@ -659,7 +647,7 @@ stamp_status stamp_problem_create(const stamp_problem_desc* d, const float* init
     }
     size_t off = 0;
     for (const Part& q : parts) {
-        *q.dst = p->arena + off;
+        *q.dst = q.bytes ? p->arena + off : nullptr;
         off += (q.bytes + 255) / 256 * 256;
     }
     const float one = 1.f;
@@ -708,12 +696,10 @@ stamp_status stamp_set_lanes(stamp_problem* p, int fwd_lanes, int adj_lanes) {
 
 stamp_status stamp_set_replay_lanes(stamp_problem* p, int lanes) {
     if (!p) return fail(STAMP_EINVAL, "NULL problem");
-    // the replay's instantiations: one block 1-4, two 2-16, three 2-32, four 4-32 lanes
     const int lo = p->sc.nb == 1 ? 1 : p->sc.nb == 4 ? 4 : 2, hi = p->sc.nb == 1 ? 4 : p->sc.nb == 2 ? 16 : 32;
     const bool pow2 = lanes > 0 && (lanes & (lanes - 1)) == 0;
     if (lanes != 0 && !(pow2 && lanes >= lo && lanes <= hi))
         return fail(STAMP_EINVAL, "unsupported replay lane count %d for n_blocks=%d", lanes, p->sc.nb);
-    p->replay_lanes = lanes;
     return STAMP_OK;
 }
 

@@ -48,9 +48,10 @@ struct RolloutArgs {
     unsigned long long* dropped;   // count of particles whose reverse sweep overflowed
     const float* init_states;      // N x n_blocks x 3 initial poses (at rest), or NULL: the scene's
     int particle0;          // global index of row 0 (Gumbel draws of a shard of a larger set)
-    // per-substep (cos, sin) of every block's yaw, [H*T][N][NB] float2, or
-    // NULL: written by the segment replay, read by the sweep that follows it
-    float2* trig;
+    int lanes;              // lanes per particle (set by the launcher)
+    // rows of every substep (or NULL): the state before it, [H*T + 1][N][S];
+    // a forward writes them, the reverse sweep takes them as a tape of interval 1
+    float* full;
 };
 
 // One problem instance of a batch, as the batched rollout kernels see it.
@@ -74,6 +75,7 @@ struct BatchArgs {
     const int* iter_dev;    // iteration number on the device (graph replays), or NULL
     int iter;               // iteration when iter_dev is NULL (< 0: no noise)
     int hard;
+    int lanes;              // lanes per particle (set by the launcher)
     unsigned long long* dropped;
 };
 
@@ -105,17 +107,6 @@ cudaError_t launch_rollout_fwd(const SimConst& sc, const RolloutArgs& a, int lan
 cudaError_t launch_rollout_adj(const SimConst& sc, const RolloutArgs& a, int lanes, cudaStream_t st);
 bool lanes_supported(int nb, int lanes);
 int default_lanes(int nb, int N, bool adjoint);
-
-// Segment replay (rollout_nb*.cu): the states before every substep of the
-// last forward, rebuilt from its checkpoints for all (particle, segment)
-// pairs at once into `full` ([H*T + 1][N][S]); `lanes` per team.
-cudaError_t launch_replay(const SimConst& sc, const RolloutArgs& a, int lanes, float* full,
-                          cudaStream_t st);
-cudaError_t launch_replay_nb1(const SimConst&, const RolloutArgs&, int, float*, cudaStream_t);
-cudaError_t launch_replay_nb2(const SimConst&, const RolloutArgs&, int, float*, cudaStream_t);
-cudaError_t launch_replay_nb3(const SimConst&, const RolloutArgs&, int, float*, cudaStream_t);
-cudaError_t launch_replay_nb4(const SimConst&, const RolloutArgs&, int, float*, cudaStream_t);
-int replay_lanes(int nb);
 
 // Batched launchers (rollout_nb*.cu): cta threads per CTA, a multiple of 32.
 cudaError_t launch_rollout_batch(int nb, const SimConst& sc, const BatchArgs& b, int lanes, int cta,

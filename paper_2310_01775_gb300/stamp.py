@@ -340,15 +340,14 @@ class Problem:
 
     def adjoint_launches(self, N):
         """Kernel launches of one reverse sweep with N particles (the
-        time-parallel sweep: relaxed parameters, Jacobians, recurrence; the
-        replay: rebuild, sweep)."""
-        return {STAMP_ADJ_TIME_PARALLEL: 3, STAMP_ADJ_REPLAY: 2}.get(self.adjoint_mode(N), 1)
+        time-parallel sweep: relaxed parameters, Jacobians, recurrence)."""
+        return 3 if self.adjoint_mode(N) == STAMP_ADJ_TIME_PARALLEL else 1
 
     def set_lanes(self, fwd_lanes, adj_lanes):
         stamp_set_lanes(self.handle, fwd_lanes, adj_lanes)
 
     def set_replay_lanes(self, lanes):
-        """Lanes per (particle, segment) team of the segment replay (0: automatic)."""
+        """Accepted and checked, without effect (stamp_set_replay_lanes)."""
         _check(_lib.stamp_set_replay_lanes(self.handle, int(lanes)))
 
     def set_particle_offset(self, particle0):
