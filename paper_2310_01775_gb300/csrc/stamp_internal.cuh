@@ -207,6 +207,18 @@ cudaError_t launch_phi_batch(const SvgdInst* inst, const int4* items, int n_item
 cudaError_t launch_adam_batch(float* theta, float* m, float* v, long long n, const SvgdInst* inst,
                               int n_inst, const int* active, const int* step_dev, const float2* bc,
                               float lr, int* flag, cudaStream_t st);
+// One instance of a batch: its initial draws (key) and its distinct-plan top-k.
+struct InstItem {
+    float* theta;           // N x D
+    const float* cost;      // N
+    int* topk;              // k
+    uint64_t key;           // sm64(seed, kStreamInit)
+    long long elem0;        // first element in the concatenated particles
+    int N, H, M, k;
+};
+// items: device, n of them, ascending elem0; n_elem: elements of the batch.
+cudaError_t launch_init_theta_batch(const InstItem* items, int n, long long n_elem, cudaStream_t st);
+cudaError_t launch_topk_batch(const InstItem* items, int n, int max_n, cudaStream_t st);
 // The single-problem Stein-sum split for N particles, and rows per phi CTA.
 void phi_batch_plan(int N, int* shares, int* j_chunk);
 int phi_rows_per_block();

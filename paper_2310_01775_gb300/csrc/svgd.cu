@@ -182,9 +182,9 @@ __global__ void init_theta_kernel(float* theta, int n, uint64_t key) {
 
 // Distinct-plan top-k: sort (cost bits, index) ascending, then keep the first
 // k distinct argmax sequences (Gamma, Eq. gamma_map; ties to the lowest index).
-__global__ void __launch_bounds__(1024) topk_kernel(const float* __restrict__ theta,
-                                                    const float* __restrict__ cost, int N, int H,
-                                                    int M, int P, int k, int* out) {
+__device__ __forceinline__ void topk_body(const float* __restrict__ theta,
+                                          const float* __restrict__ cost, int N, int H, int M, int P,
+                                          int k, int* out) {
     extern __shared__ unsigned long long sk[];
     int n2 = 1;
     while (n2 < N) n2 <<= 1;
@@ -233,6 +233,30 @@ __global__ void __launch_bounds__(1024) topk_kernel(const float* __restrict__ th
         }
         for (int q = got; q < k; ++q) out[q] = -1;
     }
+}
+
+__global__ void __launch_bounds__(1024) topk_kernel(const float* __restrict__ theta,
+                                                    const float* __restrict__ cost, int N, int H,
+                                                    int M, int P, int k, int* out) {
+    topk_body(theta, cost, N, H, M, P, k, out);
+}
+// One CTA per instance (64 launches of one CTA each took 1.9 ms, one of 64 CTAs 0.05).
+__global__ void __launch_bounds__(1024) topk_batch_kernel(const InstItem* __restrict__ items) {
+    const InstItem& it = items[blockIdx.x];
+    topk_body(it.theta, it.cost, it.N, it.H, it.M, it.M + 2, it.k, it.topk);
+}
+
+__global__ void init_theta_batch_kernel(const InstItem* __restrict__ items, int n, long long n_elem) {
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n_elem) return;
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (__ldg(&items[mid].elem0) <= t) lo = mid; else hi = mid - 1;
+    }
+    const InstItem& it = items[lo];
+    const long long loc = t - it.elem0;
+    if (loc < (long long)it.N * it.H * (it.M + 2)) it.theta[loc] = 2.f * u23(sm64(it.key, (uint64_t)loc)) - 1.f;
 }
 
 template <int DP>
@@ -406,6 +430,24 @@ cudaError_t launch_topk(const float* theta, const float* cost, int N, const SimC
         if (e != cudaSuccess) return e;
     }
     topk_kernel<<<1, 1024, smem, st>>>(theta, cost, N, sc.H, sc.M, sc.P, k, topk_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_topk_batch(const InstItem* items, int n, int max_n, cudaStream_t st) {
+    int n2 = 1;
+    while (n2 < max_n) n2 <<= 1;
+    const size_t smem = (size_t)2 * n2 * sizeof(unsigned long long);
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(topk_batch_kernel,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    topk_batch_kernel<<<n, 1024, smem, st>>>(items);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_init_theta_batch(const InstItem* items, int n, long long n_elem, cudaStream_t st) {
+    init_theta_batch_kernel<<<(unsigned)((n_elem + 255) / 256), 256, 0, st>>>(items, n, n_elem);
     return cudaGetLastError();
 }
 
