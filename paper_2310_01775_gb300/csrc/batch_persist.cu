@@ -324,8 +324,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
 
 size_t persist_smem(int max_D, int seg_warp) {
     const int dp = persist_dp(max_D);
-    const size_t phi = (size_t)4 * phi_stage_floats(max_D, dp) * sizeof(float) +
-                       (size_t)kPersistWarps * kTJ * sizeof(float4) + 2 * sizeof(uint64_t);
+    const size_t phi = phi_smem(max_D, dp, kPersistWarps, kR);
     const size_t pw = 2 * kTile * (size_t)(max_D + 1) * sizeof(float);
     const size_t seg = (size_t)kPersistWarps * seg_warp * sizeof(float2);
     size_t m = phi > pw ? phi : pw;

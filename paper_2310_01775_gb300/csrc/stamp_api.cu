@@ -254,6 +254,12 @@ stamp_status bandwidth(stamp_problem* p, const float* theta, int N, float* h_out
     return STAMP_OK;
 }
 
+// Few particles: the whole step is one CTA's work (timed as STAMP_K_PHI).  A
+// wait made to run out (test hook) needs the Stein-direction kernel.
+bool small_step(const stamp_problem* p, int N) {
+    return N <= stamp::kSmallN && p->kernel_kind == 0 && !p->inject_wait_timeout;
+}
+
 // bw_done: the RBF bandwidth of theta is already in p->h (launched beside the
 // rollouts and waited for).
 stamp_status svgd(stamp_problem* p, float* theta, const float* grad, int N, float* m, float* v,
@@ -284,10 +290,16 @@ stamp_status svgd(stamp_problem* p, float* theta, const float* grad, int N, floa
         }
         if (h_out) STAMP_CUDA(stamp::launch_scale_scalar(p->h, 1.f / (float)H, h_out, p->stream));
         STAMP_TRY(timed(p, STAMP_K_PHI, [&] {
-            return stamp::launch_struct_phi(theta, grad, p->sk_C, p->sk_S, N, H, M, p->h, p->sk_h, wn,
+            return stamp::launch_struct_phi(theta, grad, p->sk_S, N, H, M, p->h, p->sk_h, wn,
                                             p->phi, stamp::kMaxShares, &shares, p->stream);
         }));
         part = p->phi;
+    } else if (!sgd_phase && small_step(p, N)) {
+        stamp::SvgdScratch s{p->d2, p->hist, p->sel, p->counter, p->h, p->flag};
+        return timed(p, STAMP_K_PHI, [&] {
+            return stamp::launch_small_step(theta, grad, N, D, m, v, wn, step, lr, s, h_out, phi_out,
+                                            p->stream);
+        });
     } else if (!sgd_phase) {
         stamp::SvgdScratch s{p->d2, p->hist, p->sel, p->counter, p->h, p->flag};
         if (p->inject_wait_timeout) {
@@ -381,7 +393,7 @@ stamp_status run_solve(stamp_problem* p, const Phases& ph, int N, unsigned long 
         unsigned* sw = stats_out ? p->stats + it : nullptr;
         const bool sgd = it >= (long long)ph.sur + ph.svgd;
         // the bandwidth needs theta only: start it beside this iteration's rollouts
-        const bool side_bw = p->overlap && !sgd && p->kernel_kind == 0 && N >= 2;
+        const bool side_bw = p->overlap && !sgd && p->kernel_kind == 0 && N >= 2 && !small_step(p, N);
         if (side_bw) {
             STAMP_CUDA(cudaEventRecord(p->ev_theta, p->stream));
             STAMP_CUDA(cudaStreamWaitEvent(p->side, p->ev_theta, 0));

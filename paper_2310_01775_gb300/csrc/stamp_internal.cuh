@@ -144,6 +144,11 @@ struct SvgdScratch {
     unsigned wait_limit = 0;
     int skip_first_copy = 0;
 };
+// A whole RBF Stein step (bandwidth, direction, Adam) of N <= kSmallN particles.
+constexpr int kSmallN = 64;
+cudaError_t launch_small_step(float* theta, const float* grad, int N, int D, float* m, float* v,
+                              const float* wn, int step, float lr, const SvgdScratch& s, float* h_out,
+                              float* phi_out, cudaStream_t st);
 cudaError_t launch_pairwise(const float* theta, int N, int D, const SvgdScratch& s, cudaStream_t st);
 cudaError_t launch_median_digit(int N, int digit, const SvgdScratch& s, float* h_out,
                                 cudaStream_t st);
@@ -165,7 +170,7 @@ cudaError_t launch_phi_rows(const float* theta, const float* grad, int N, int D,
 cudaError_t launch_struct_prep(const float* theta, int N, int H, int M, float* C, float* S,
                                cudaStream_t st);
 // Writes `*shares` partial directions (N x D each, consecutive; at most max_shares).
-cudaError_t launch_struct_phi(const float* theta, const float* grad, const float* C, const float* S,
+cudaError_t launch_struct_phi(const float* theta, const float* grad, const float* S,
                               int N, int H, int M, const float* hc_dev, const float* hz_dev,
                               const float* wn, float* phi, int max_shares, int* shares,
                               cudaStream_t st);

@@ -14,14 +14,114 @@
 namespace stamp {
 namespace {
 
-__global__ void __launch_bounds__(256) pairwise_kernel(const float* __restrict__ theta, int N,
-                                                       int D, float* __restrict__ d2,
+// d2 and the first median digit over 64 x 64 tile pairs: each thread owns 4 x 4
+// pairs and walks the columns in chunks of 32, both tiles held column-major in
+// shared memory (two 16-byte loads for 16 pairs, so the subtraction and the
+// multiply-add per pair and column are the bound; one pair row and four pairs
+// a thread, five 4-byte loads, was bound by the loads).  16-byte groups of
+// rows are swizzled by the column so that storing a tile (4 rows x 8 columns
+// a warp) meets no bank twice.  Two pairs per instruction (f32x2).  The sums
+// over the columns run in column order.  GB300: 57 -> 26 us at N = 2048, D = 84,
+// 454 -> 179 us at N = 6001, D = 108; 10 us at N = 1024, D = 16, as before.
+constexpr int kPT = 64, kPC = 32;   // tile edge, columns per chunk
+__device__ __forceinline__ int pw_at(int d, int row) {   // float index in a chunk
+    return d * kPT + ((((row >> 2) ^ (d & 7)) << 2) | (row & 3));
+}
+__global__ void __launch_bounds__(256) pairwise_kernel(const float* __restrict__ theta, int N, int D,
+                                                       float* __restrict__ d2,
                                                        unsigned* __restrict__ hist,
                                                        unsigned* __restrict__ sel,
                                                        unsigned* __restrict__ counter,
-                                                       float* __restrict__ h_dev) {
-    if (blockIdx.y > blockIdx.x) return;
-    pairwise_body(theta, N, D, d2, hist, sel, counter, h_dev, blockIdx.y, blockIdx.x, gridDim.x);
+                                                       float* __restrict__ h_dev, int nt) {
+    // A and B chunks; the finished tile takes their place
+    __shared__ __align__(16) float buf[kPT * (kPT + 1) > 2 * kPC * kPT ? kPT * (kPT + 1) : 2 * kPC * kPT];
+    __shared__ unsigned h0[kBins0];
+    float* A = buf;
+    float* B = buf + kPC * kPT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // tile pair (bi <= bj) number blockIdx.x of the nt (nt + 1) / 2, row by row
+    int bi = 0, left = blockIdx.x;
+    while (left >= nt - bi) left -= nt - bi++;
+    const int bj = bi + left, i0 = bi * kPT, j0 = bj * kPT;
+    for (int t = tid; t < kBins0; t += 256) h0[t] = 0u;
+    const int tx = tid & 15, ty = tid >> 4;
+    f32x2 acc[4][2];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[r][0] = acc[r][1] = 0ull;
+    // this thread's elements of a chunk: column lane & 7 (+ 8 v), row (lane >> 3) + 4 warp (+ 32 u)
+    const int lr = (lane >> 3) + 4 * warp, ld = lane & 7;
+    for (int c0 = 0; c0 < D; c0 += kPC) {
+        float va[2][4], vb[2][4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int d = c0 + ld + 8 * v, ra = i0 + lr + 32 * u, rb = j0 + lr + 32 * u;
+                va[u][v] = d < D && ra < N ? theta[(size_t)ra * D + d] : 0.f;
+                vb[u][v] = d < D && rb < N ? theta[(size_t)rb * D + d] : 0.f;
+            }
+        __syncthreads();   // the previous chunk is read
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                A[pw_at(ld + 8 * v, lr + 32 * u)] = va[u][v];
+                B[pw_at(ld + 8 * v, lr + 32 * u)] = -vb[u][v];   // a - b as a + (-b)
+            }
+        __syncthreads();
+        const int nd = min(kPC, D - c0);
+#pragma unroll 8
+        for (int d = 0; d < nd; ++d) {
+            const float4 a = *reinterpret_cast<const float4*>(A + pw_at(d, 4 * ty));
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(B + pw_at(d, 4 * tx));
+            const f32x2 av[4] = {pack2(a.x, a.x), pack2(a.y, a.y), pack2(a.z, a.z), pack2(a.w, a.w)};
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const f32x2 e0 = add2(av[r], b.x), e1 = add2(av[r], b.y);
+                acc[r][0] = fma2(e0, e0, acc[r][0]);
+                acc[r][1] = fma2(e1, e1, acc[r][1]);
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            float lo, hi;
+            unpack2(acc[r][q], lo, hi);
+            float* p = buf + (4 * ty + r) * (kPT + 1) + 4 * tx + 2 * q;
+            p[0] = lo;
+            p[1] = hi;
+        }
+    __syncthreads();
+    // coalesced rows of the tile and of its mirror; the pairs i < j counted by
+    // digit, equal digits of a warp's 32 pairs at once (the distances of a set
+    // share a few exponents: one atomic a pair would queue on a few counters)
+    for (int t = tid; t < kPT * kPT; t += 256) {
+        const int r = t / kPT, c = t % kPT, i = i0 + r, j = j0 + c;
+        const float v = buf[r * (kPT + 1) + c];
+        if (i < N && j < N) d2[(size_t)i * N + j] = v;
+        const unsigned bin = i < j && j < N ? digit_of(__float_as_uint(v), 0) : 0xffffffffu;
+        const unsigned same = __match_any_sync(0xffffffffu, bin);
+        if (bin != 0xffffffffu && lane == __ffs(same) - 1) atomicAdd(&h0[bin], (unsigned)__popc(same));
+        if (bi != bj) {   // r indexes j, c indexes i
+            const int jm = j0 + r, im = i0 + c;
+            if (jm < N && im < N) d2[(size_t)jm * N + im] = buf[c * (kPT + 1) + r];
+        }
+    }
+    __syncthreads();
+    for (int t = tid; t < kBins0; t += 256)
+        if (h0[t]) atomicAdd(&hist[t], h0[t]);
+    if (last_block(counter, gridDim.x)) {
+        if (N < 2) {
+            if (tid == 0) *h_dev = 1.f;
+            return;
+        }
+        unsigned b0, r0;
+        find_bin<kBins0, 256>(hist, median_rank(N), b0, r0);
+        if (tid == 0) { sel[0] = b0; sel[1] = r0; }
+    }
 }
 
 // Batched: one CTA per work item (instance, tile row bi, tile column bj >= bi).
@@ -57,7 +157,7 @@ __global__ void __launch_bounds__(256) median_digit_batch_kernel(const SvgdInst*
 }
 
 
-template <int DP>
+template <int DP, int R>
 __global__ void __launch_bounds__(kW * 32) phi_kernel(const float* __restrict__ theta,
                                                       const float* __restrict__ grad, int N, int D,
                                                       const float* __restrict__ d2,
@@ -66,8 +166,8 @@ __global__ void __launch_bounds__(kW * 32) phi_kernel(const float* __restrict__ 
                                                       int* err, const float* __restrict__ wn,
                                                       unsigned wait_limit, int skip_first, int row0,
                                                       int rows) {
-    phi_body<DP>(theta, grad, N, D, d2, h_dev, part, j_chunk, err, blockIdx.x, blockIdx.y, wn,
-                 wait_limit, skip_first != 0, row0, rows);
+    phi_body<DP, kW, 8, R>(theta, grad, N, D, d2, h_dev, part, j_chunk, err, blockIdx.x, blockIdx.y, wn,
+                           wait_limit, skip_first != 0, row0, rows);
 }
 
 // Batched: work item (instance, row block, j-share); DP covers the batch's largest D.
@@ -136,6 +236,102 @@ __global__ void adam_batch_kernel(float* __restrict__ theta, float* __restrict__
     v[t] = vt;
     theta[t] = th;
     if (!isfinite(th) || !isfinite(gr)) atomicOr(flag, 1);
+}
+
+// A whole Stein step of at most kSmallN particles in one CTA: distances, their
+// exact lower median (bisection on the float bits), direction and Adam.  The
+// six launches it replaces cost more than their work (N = 32, D = 12: 30 us
+// against 8).
+// Every sum runs in the order of the kernels above with the direct form of the
+// repulsion: 32 particles a share.
+template <int E>   // N <= E (32 or 64)
+__global__ void __launch_bounds__(1024) small_step_kernel(
+    float* __restrict__ theta, const float* __restrict__ grad, int N, int D, float* __restrict__ m,
+    float* __restrict__ v, const float* __restrict__ wn, float lr, float bc1, float bc2,
+    float* __restrict__ h_dev, float* __restrict__ h_out, float* __restrict__ phi_out, int* flag) {
+    extern __shared__ float ssm[];
+    const int ld = D | 1;   // odd row stride: rows fall in different banks
+    float* T = ssm;
+    float* G = T + E * ld;
+    __shared__ float K[E][E + 1];   // d2, then the kernel values
+    __shared__ float h_sh;
+    const int tid = threadIdx.x;
+    for (int t = tid; t < N * D; t += 1024) {
+        T[(t / D) * ld + t % D] = theta[t];
+        G[(t / D) * ld + t % D] = grad[t];
+    }
+    __syncthreads();
+    for (int t = tid; t < N * N; t += 1024) {
+        const int i = t / N, j = t % N;
+        if (i <= j) {
+            float a = 0.f;
+            for (int d = 0; d < D; ++d) {
+                const float e = T[i * ld + d] - T[j * ld + d];
+                a = fmaf(e, e, a);
+            }
+            K[i][j] = K[j][i] = a;
+        }
+    }
+    __syncthreads();
+    // the lower median of the pairs: the smallest value with more than `rank` values <= it
+    const int pairs = N * (N - 1) / 2;
+    constexpr int V = E * E / 1024;
+    unsigned val[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+        const int t = tid + q * 1024, i = t / E, j = t % E;
+        val[q] = i < j && j < N ? __float_as_uint(K[i][j]) : 0xffffffffu;
+    }
+    float h = 1.f;
+    if (N >= 2) {
+        const int rank = (pairs - 1) / 2;
+        unsigned lo = 0u, hi = 0xffffffffu;   // the answer lies in [lo, hi]
+        while (lo < hi) {
+            const unsigned mid = lo + (hi - lo) / 2;
+            int c = 0;
+#pragma unroll
+            for (int q = 0; q < V; ++q) c += __syncthreads_count(val[q] <= mid);
+            if (c > rank) hi = mid; else lo = mid + 1;
+        }
+        h = __uint_as_float(lo) / logf((float)N + 1.f);
+        h = (h >= 1e-12f) ? h : 1.f;
+    }
+    if (tid == 0) {
+        *h_dev = h;
+        if (h_out) *h_out = h;
+    }
+    const float inv_h = 1.f / h, two_h = 2.f * inv_h;
+    for (int t = tid; t < N * N; t += 1024) {
+        const int i = t / N, j = t % N;
+        float k = expf(-K[i][j] * inv_h);
+        if (wn) k *= wn[j];
+        K[i][j] = k;
+    }
+    __syncthreads();
+    const float inv_n = wn ? 1.f : 1.f / (float)N;
+    for (int t = tid; t < N * D; t += 1024) {
+        const int i = t / D, d = t % D;
+        const float ti = T[i * ld + d];
+        float phi = 0.f;
+        for (int j0 = 0; j0 < N; j0 += kTJ) {
+            float ag = 0.f, ar = 0.f;
+            for (int j = j0; j < min(N, j0 + kTJ); ++j) {
+                ag = fmaf(K[i][j], G[j * ld + d], ag);
+                ar = fmaf(K[i][j], ti - T[j * ld + d], ar);
+            }
+            const float part = fmaf(two_h, ar, ag) * inv_n;
+            phi = j0 ? phi + part : part;
+        }
+        if (phi_out) phi_out[t] = phi;
+        const float g = -phi;
+        const float mt = 0.9f * m[t] + 0.1f * g;
+        const float vt = 0.999f * v[t] + 0.001f * g * g;
+        const float th = ti - lr * (mt / bc1) / (sqrtf(vt / bc2) + 1e-8f);
+        m[t] = mt;
+        v[t] = vt;
+        theta[t] = th;
+        if (!isfinite(th) || !isfinite(g)) atomicOr(flag, 1);
+    }
 }
 
 // Eq. dsvgd weights, normalised: w_j = exp(C_j - C~_j - max) / sum, C the hard
@@ -259,43 +455,79 @@ __global__ void init_theta_batch_kernel(const InstItem* __restrict__ items, int 
     if (loc < (long long)it.N * it.H * (it.M + 2)) it.theta[loc] = 2.f * u23(sm64(it.key, (uint64_t)loc)) - 1.f;
 }
 
+template <int DP, int R>
+cudaError_t phi_launch_rows(const float* theta, const float* grad, int N, int D, const float* d2,
+                            const float* h_dev, float* part, int shares, int j_chunk, int* err,
+                            const float* wn, unsigned wait_limit, int skip_first, int row0, int rows,
+                            cudaStream_t st) {
+    const size_t smem = phi_smem(D, DP, kW, R);
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(phi_kernel<DP, R>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    const int per_cta = kW * R;
+    phi_kernel<DP, R><<<dim3((rows + per_cta - 1) / per_cta, shares), kW * 32, smem, st>>>(
+        theta, grad, N, D, d2, h_dev, part, j_chunk, err, wn, wait_limit, skip_first, row0, rows);
+    return cudaGetLastError();
+}
+// The split of the Stein sum of N particles over j-shares and the rows per
+// warp; a function of N alone, so that a shard of the rows sums as all do (a
+// row's sum depends on the shares, not on the rows per warp).  Eight rows per
+// warp (two resident CTAs of 64 rows per SM) once eight shares of them give 1.6
+// CTAs per SM; there the shares are the count, at most max_shares, that fills
+// whole waves best.  Below that four rows per warp and about four CTAs per SM.
+void phi_plan(int N, int max_shares, int* rows_per_warp, int* shares, int* j_chunk) {
+    const int sms = sm_count(), b8 = (N + 8 * kW - 1) / (8 * kW), b4 = (N + 4 * kW - 1) / (4 * kW);
+    int want;
+    if (10 * b8 * kMaxShares >= 16 * sms) {
+        *rows_per_warp = 8;
+        want = 1;
+        double best = 0.0;
+        for (int s = 1; s <= max_shares; ++s) {
+            const int ctas = b8 * s, waves = (ctas + 2 * sms - 1) / (2 * sms);
+            const double fill = (double)ctas / ((double)waves * 2 * sms);
+            if (fill > best + 0.01) {
+                best = fill;
+                want = s;
+            }
+        }
+    } else {
+        *rows_per_warp = 4;
+        want = (4 * sms + b4 - 1) / b4;
+        want = want < 1 ? 1 : (want > max_shares ? max_shares : want);
+    }
+    // the shares start on kTJ-row boundaries (16-byte aligned TMA sources)
+    *j_chunk = ((N + want - 1) / want + kTJ - 1) / kTJ * kTJ;
+    *shares = (N + *j_chunk - 1) / *j_chunk;
+}
 template <int DP>
 cudaError_t phi_launch(const float* theta, const float* grad, int N, int D, const float* d2,
                        const float* h_dev, float* part, int shares, int j_chunk, int* err,
                        const float* wn, unsigned wait_limit, int skip_first, int row0, int rows,
-                       cudaStream_t st) {
-    const size_t smem = (size_t)4 * phi_stage_floats(D, DP) * sizeof(float) +
-                        (size_t)kW * kTJ * sizeof(float4) + 2 * sizeof(uint64_t);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(phi_kernel<DP>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    const int per_cta = kW * kR;
-    phi_kernel<DP><<<dim3((rows + per_cta - 1) / per_cta, shares), kW * 32, smem, st>>>(
-        theta, grad, N, D, d2, h_dev, part, j_chunk, err, wn, wait_limit, skip_first, row0, rows);
-    return cudaGetLastError();
+                       bool r8, cudaStream_t st) {
+    return r8 ? phi_launch_rows<DP, 8>(theta, grad, N, D, d2, h_dev, part, shares, j_chunk, err, wn,
+                                       wait_limit, skip_first, row0, rows, st)
+              : phi_launch_rows<DP, 4>(theta, grad, N, D, d2, h_dev, part, shares, j_chunk, err, wn,
+                                       wait_limit, skip_first, row0, rows, st);
 }
 
 }  // namespace
 
 cudaError_t launch_pairwise(const float* theta, int N, int D, const SvgdScratch& s,
                             cudaStream_t st) {
-    const int nt = (N + kTile - 1) / kTile;
-    const size_t smem = 2 * kTile * (D + 1) * sizeof(float);
-    if (smem + kPairwiseStatic > 48 * 1024) {   // static + dynamic above the default limit
-        cudaError_t e = cudaFuncSetAttribute(pairwise_kernel,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    pairwise_kernel<<<dim3(nt, nt), 256, smem, st>>>(theta, N, D, s.d2, s.hist, s.sel, s.counter,
-                                                     s.h);
+    const int nt = (N + kPT - 1) / kPT;
+    pairwise_kernel<<<nt * (nt + 1) / 2, 256, 0, st>>>(theta, N, D, s.d2, s.hist, s.sel, s.counter,
+                                                       s.h, nt);
     return cudaGetLastError();
 }
 
 cudaError_t launch_median_digit(int N, int digit, const SvgdScratch& s, float* h_out,
                                 cudaStream_t st) {
-    const int cap = 2 * sm_count();
+    // a CTA flushes its bins once: few CTAs for a small matrix (two a SM: 13 us
+    // a digit at N = 2048, 18 with six), more loads in flight for a large one
+    // (N = 6001: 42 + 34 us for the two digits with two, 27 + 21 with six)
+    const int cap = (N >= 4096 ? 6 : 2) * sm_count();
     int grid = N - 1 < cap ? N - 1 : cap;
     if (grid < 1) grid = 1;
     median_digit_kernel<<<grid, 256, 0, st>>>(N, digit, s.d2, s.hist, s.sel, s.counter + digit,
@@ -309,24 +541,20 @@ cudaError_t launch_phi_rows(const float* theta, const float* grad, int N, int D,
     // TMA bulk copies need 16-byte aligned sources
     if ((reinterpret_cast<uintptr_t>(theta) | reinterpret_cast<uintptr_t>(grad)) & 15u)
         return cudaErrorMisalignedAddress;
-    // split the sum over j so that about four CTAs per SM are in flight; the
-    // shares start on kTJ-row boundaries (16-byte aligned TMA sources)
-    const int row_blocks = (N + kW * kR - 1) / (kW * kR);
-    int want = (4 * sm_count() + row_blocks - 1) / row_blocks;
-    want = want < 1 ? 1 : (want > max_shares ? max_shares : want);
-    const int j_chunk = ((N + want - 1) / want + kTJ - 1) / kTJ * kTJ;
-    *shares = (N + j_chunk - 1) / j_chunk;
+    int j_chunk, rpw;
+    phi_plan(N, max_shares, &rpw, shares, &j_chunk);
+    const bool r8 = rpw == 8;
     const unsigned limit = s.wait_limit ? s.wait_limit : kWaitLimit;
     const int dp = (D + 31) / 32;
     switch (dp) {
-        case 1: return phi_launch<1>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, st);
-        case 2: return phi_launch<2>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, st);
-        case 3: return phi_launch<3>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, st);
-        case 4: return phi_launch<4>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, st);
+        case 1: return phi_launch<1>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
+        case 2: return phi_launch<2>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
+        case 3: return phi_launch<3>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
+        case 4: return phi_launch<4>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
         case 5: case 6:
-            return phi_launch<6>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, st);
+            return phi_launch<6>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
         case 7: case 8: case 9:
-            return phi_launch<9>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, st);
+            return phi_launch<9>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -342,6 +570,20 @@ cudaError_t launch_adam(float* theta, const float* part, int shares, float* phi_
     const float bc2 = 1.f - powf(0.999f, (float)step);
     adam_kernel<<<(n + 255) / 256, 256, 0, st>>>(theta, part, shares, phi_out, m, v, n, lr, bc1,
                                                  bc2, flag);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_small_step(float* theta, const float* grad, int N, int D, float* m, float* v,
+                              const float* wn, int step, float lr, const SvgdScratch& s, float* h_out,
+                              float* phi_out, cudaStream_t st) {
+    const int edge = N <= 32 ? 32 : kSmallN;
+    const size_t smem = (size_t)2 * edge * (D | 1) * sizeof(float);   // up to 148 KB
+    auto* kernel = N <= 32 ? small_step_kernel<32> : small_step_kernel<kSmallN>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const float bc1 = 1.f - powf(0.9f, (float)step);
+    const float bc2 = 1.f - powf(0.999f, (float)step);
+    kernel<<<1, 1024, smem, st>>>(theta, grad, N, D, m, v, wn, lr, bc1, bc2, s.h, h_out, phi_out, s.err);
     return cudaGetLastError();
 }
 
@@ -364,19 +606,15 @@ cudaError_t launch_median_digit_batch(const SvgdInst* inst, const int2* items, i
 }
 
 void phi_batch_plan(int N, int* shares, int* j_chunk) {
-    const int row_blocks = (N + kW * kR - 1) / (kW * kR);
-    int want = (4 * sm_count() + row_blocks - 1) / row_blocks;
-    want = want < 1 ? 1 : (want > kMaxShares ? kMaxShares : want);
-    *j_chunk = ((N + want - 1) / want + kTJ - 1) / kTJ * kTJ;
-    *shares = (N + *j_chunk - 1) / *j_chunk;
+    int rpw;
+    phi_plan(N, kMaxShares, &rpw, shares, j_chunk);
 }
 int phi_rows_per_block() { return kW * kR; }
 
 template <int DP>
 cudaError_t phi_batch_launch(const SvgdInst* inst, const int4* items, int n_items, int max_D,
                              const int* active, int* err, cudaStream_t st) {
-    const size_t smem = (size_t)4 * phi_stage_floats(max_D, DP) * sizeof(float) +
-                        (size_t)kW * kTJ * sizeof(float4) + 2 * sizeof(uint64_t);
+    const size_t smem = phi_smem(max_D, DP, kW, kR);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(phi_batch_kernel<DP>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -19,6 +19,28 @@ constexpr int kBins0 = 2048, kBins1 = 2048, kBins2 = 1024;
 // tile, the bin search's scratch), with margin
 constexpr size_t kPairwiseStatic = kBins0 * 4 + kTile * (kTile + 1) * 4 + 256;
 
+// Two float32 lanes in one instruction (each rounded as the scalar one): the
+// loops here are bound by instruction issue, not by the FP32 pipe.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 __device__ __forceinline__ unsigned digit_of(unsigned bits, int d) {
     return d == 0 ? (bits >> 21) : d == 1 ? ((bits >> 10) & 2047u) : (bits & 1023u);
 }
@@ -249,21 +271,39 @@ using async::mbar_try_wait;
 using async::tma_load_1d;
 
 // phi_i = (1/N) sum_j [k_ij g_j + (2/h) k_ij (theta_i - theta_j)], k_ij = exp(-d2_ij/h).
-// A warp owns kR rows; lane l owns columns l, l+32, ...  (DP slots).  The j
+// With u_j = g_j - (2/h) (theta_j - c), c = theta_0, and S_i = sum_{j != i} k_ij,
+//   N phi_i = g_i + sum_{j != i} k_ij u_j + (2/h) (theta_i - c) S_i:
+// one multiply-add per (i, j, column) instead of a subtraction and two.  c is
+// one of the particles, so theta - c is of the size of their distances (no
+// offset common to all particles is multiplied by the kernel), and the term
+// j = i, whose parts would only cancel, is left out of the sums.
+//
+// A warp owns R rows; lane l owns columns l, l+32, ...  (DP slots).  The j
 // range is walked in tiles of kTJ rows of theta and grad, which are
 // contiguous in HBM: one thread streams each tile into one of two shared
 // memory stages with 1-D TMA bulk copies (mbarrier completion), one tile
-// ahead of the compute.  The d2 values of the next tile are prefetched into
-// registers; k_ij for the warp's rows is one float4 per j (a broadcast load).
+// ahead of the compute; the CTA turns the grad tile into u in place.  The d2
+// values of the next tile are prefetched into registers; k_ij for the warp's
+// rows is R/4 float4 per j (broadcast loads).  The shared-memory loads per j
+// (DP + R/4) against R DP multiply-adds, and the instructions around them,
+// bound it: two rows' multiply-adds per instruction (f32x2), R = 8 where that
+// still leaves enough CTAs.  GB300: 72 -> 38 us at N = 2048, D = 84, 672 -> 302 us
+// at N = 6001, D = 108 (FP32 pipe 33% busy).  Error of phi against 64 bits, theta
+// uniform in (-1, 1): 3.0e-7 (direct form 3.2e-7) and 7.0e-7 (7.8e-7).
 constexpr int kR = 4, kW = 8, kTJ = 32;   // rows per warp, warps per CTA, j rows per tile
 __host__ __device__ constexpr int phi_stage_floats(int D, int DP) {
     return ((kTJ * D + 32 * DP) + 3) / 4 * 4;   // per array, 16-byte multiple
+}
+// Dynamic shared memory of a CTA of KW warps with R rows each.
+__host__ __device__ constexpr size_t phi_smem(int D, int DP, int KW, int R) {
+    return (size_t)4 * phi_stage_floats(D, DP) * sizeof(float) +
+           (size_t)KW * kTJ * R * sizeof(float) + 2 * sizeof(uint64_t);
 }
 // KW warps per CTA (kW in the per-piece kernels), the j loop unrolled
 // UNROLL times; false if a copy never
 // landed (error bit 2 set).  A CTA that goes on to other work may reuse the
 // shared memory: the mbarriers are invalidated on the way out.
-template <int DP, int KW = kW, int UNROLL = 4>
+template <int DP, int KW = kW, int UNROLL = 8, int R = kR>
 __device__ __forceinline__ bool phi_body(const float* __restrict__ theta,
                                          const float* __restrict__ grad, int N, int D,
                                          const float* __restrict__ d2,
@@ -272,13 +312,14 @@ __device__ __forceinline__ bool phi_body(const float* __restrict__ theta,
                                          const float* __restrict__ wn, unsigned wait_limit,
                                          bool skip_first, int row0, int rows) {
     extern __shared__ __align__(128) float sm[];
+    constexpr int R4 = R / 4;
     const int sf = phi_stage_floats(D, DP);
     // stage s: theta tile at sm + 2*s*sf, grad tile right after it
-    float4* Ks = reinterpret_cast<float4*>(sm + 4 * sf);             // KW x kTJ
-    uint64_t* bar = reinterpret_cast<uint64_t*>(Ks + KW * kTJ);       // 2 stages
+    float4* Ks = reinterpret_cast<float4*>(sm + 4 * sf);              // KW x kTJ x R4
+    uint64_t* bar = reinterpret_cast<uint64_t*>(Ks + KW * kTJ * R4);   // 2 stages
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // rows [row0, row0 + rows) of phi (all N: row0 = 0, rows = N)
-    const int ib = row0 + (rblock * KW + warp) * kR, re = row0 + rows;
+    const int ib = row0 + (rblock * KW + warp) * R, re = row0 + rows;
     // this CTA's share of the sum over j: rows [jb, je) of theta and grad
     const int jb = share * j_chunk, je = min(N, jb + j_chunk);
     const int ntiles = (je - jb + kTJ - 1) / kTJ;
@@ -311,35 +352,41 @@ __device__ __forceinline__ bool phi_body(const float* __restrict__ theta,
         issue(0);
         if (ntiles > 1) issue(1);
     }
-    float ti[kR][DP], ag[kR][DP], ar[kR][DP], dv[kR];
+    const float two_h = 2.f * inv_h;
+    float c[DP], dv[R], ksum[R];
+    f32x2 acc[R / 2][DP];   // rows 2 p and 2 p + 1
 #pragma unroll
-    for (int r = 0; r < kR; ++r) {
+    for (int q = 0; q < DP; ++q) {
+        const int d = lane + 32 * q;
+        c[q] = d < D ? theta[d] : 0.f;
+    }
 #pragma unroll
-        for (int q = 0; q < DP; ++q) {
-            const int d = lane + 32 * q;
-            ti[r][q] = (ib + r < re && d < D) ? theta[(size_t)(ib + r) * D + d] : 0.f;
-            ag[r][q] = ar[r][q] = 0.f;
-        }
+    for (int r = 0; r < R; ++r) {
+        for (int q = 0; q < DP; ++q) acc[r / 2][q] = 0ull;
+        ksum[r] = 0.f;
         dv[r] = (ib + r < re && jb + lane < je) ? d2[(size_t)(ib + r) * N + jb + lane] : 0.f;
     }
     unsigned phases = 0u;                       // bit s: parity of stage s
     for (int t = 0; t < ntiles; ++t) {
         const int s = t & 1, j0 = jb + t * kTJ, nj = min(kTJ, je - j0);
         {
-            float kv[kR];
+            float kv[R];
+            // Eq. dsvgd: k_ij scaled by w_j / w
+            const float wj = wn && lane < nj ? wn[j0 + lane] : 1.f;
 #pragma unroll
-            for (int r = 0; r < kR; ++r) kv[r] = (ib + r < re && lane < nj) ? expf(-dv[r] * inv_h) : 0.f;
-            if (wn) {   // Eq. dsvgd: k_ij scaled by w_j / w
-                const float wj = lane < nj ? wn[j0 + lane] : 0.f;
-#pragma unroll
-                for (int r = 0; r < kR; ++r) kv[r] *= wj;
+            for (int r = 0; r < R; ++r) {
+                const bool in = ib + r < re && lane < nj && j0 + lane != ib + r;
+                kv[r] = in ? expf(-dv[r] * inv_h) * wj : 0.f;
+                ksum[r] += kv[r];
             }
-            Ks[warp * kTJ + lane] = make_float4(kv[0], kv[1], kv[2], kv[3]);
+#pragma unroll
+            for (int v = 0; v < R4; ++v)
+                Ks[(warp * kTJ + lane) * R4 + v] = make_float4(kv[4 * v], kv[4 * v + 1], kv[4 * v + 2], kv[4 * v + 3]);
         }
         if (t + 1 < ntiles) {   // next tile's distances, consumed one iteration later
             const int jn = j0 + kTJ + lane;
 #pragma unroll
-            for (int r = 0; r < kR; ++r) dv[r] = (ib + r < re && jn < je) ? d2[(size_t)(ib + r) * N + jn] : 0.f;
+            for (int r = 0; r < R; ++r) dv[r] = (ib + r < re && jn < je) ? d2[(size_t)(ib + r) * N + jn] : 0.f;
         }
         const unsigned par = (phases >> s) & 1u;
         unsigned spins = 0;
@@ -361,39 +408,69 @@ __device__ __forceinline__ bool phi_body(const float* __restrict__ theta,
         }
         phases ^= 1u << s;
         const float* Tj = sm + 2 * s * sf;
-        const float* Gj = Tj + sf;
-#pragma unroll (UNROLL)
-        for (int jj = 0; jj < nj; ++jj) {   // several j's shared-memory loads in flight
-            const float4 k4 = Ks[warp * kTJ + jj];
-            const float kk[kR] = {k4.x, k4.y, k4.z, k4.w};
+        float* Uj = sm + (2 * s + 1) * sf;
+        for (int jj = warp; jj < nj; jj += KW)   // u in place of g
 #pragma unroll
             for (int q = 0; q < DP; ++q) {
-                const float g = Gj[jj * D + lane + 32 * q];
-                const float tv = Tj[jj * D + lane + 32 * q];
-#pragma unroll
-                for (int r = 0; r < kR; ++r) {
-                    ag[r][q] = fmaf(kk[r], g, ag[r][q]);
-                    ar[r][q] = fmaf(kk[r], ti[r][q] - tv, ar[r][q]);
-                }
+                const int d = lane + 32 * q;
+                if (d < D) Uj[jj * D + d] = fmaf(-two_h, Tj[jj * D + d] - c[q], Uj[jj * D + d]);
             }
-        }
+        __syncthreads();
+        const float* up = Uj + lane;
+        const ulonglong2* kp = reinterpret_cast<const ulonglong2*>(Ks + warp * kTJ * R4);
+        auto one_j = [&]() {
+            f32x2 kk[R / 2];
+#pragma unroll
+            for (int v = 0; v < R4; ++v) {
+                const ulonglong2 k4 = kp[v];
+                kk[2 * v] = k4.x;
+                kk[2 * v + 1] = k4.y;
+            }
+#pragma unroll
+            for (int q = 0; q < DP; ++q) {
+                const float u = up[32 * q];
+                const f32x2 uu = pack2(u, u);
+#pragma unroll
+                for (int p = 0; p < R / 2; ++p) acc[p][q] = fma2(kk[p], uu, acc[p][q]);
+            }
+            up += D;
+            kp += R4;
+        };
+        int jj = 0;
+        if constexpr (UNROLL > 1)   // several j's shared-memory loads in flight
+            for (; jj + UNROLL <= nj; jj += UNROLL)
+#pragma unroll
+                for (int x = 0; x < UNROLL; ++x) one_j();
+#pragma unroll 1
+        for (; jj < nj; ++jj) one_j();
         __syncthreads();                       // stage s and Ks fully read
         if (tid == 0 && t + 2 < ntiles) {
             fence_async_shared();
             issue(t + 2);
         }
     }
-    // partial phi of this j-share; the Adam kernel sums the shares in order
-    const float inv_n = wn ? 1.f : 1.f / (float)N, two_h = 2.f * inv_h;
+    // partial phi of this j-share (the term j = i in the share that holds it);
+    // the Adam kernel sums the shares in order
+    const float inv_n = wn ? 1.f : 1.f / (float)N;
     float* out = part + (size_t)share * rows * D;
 #pragma unroll
-    for (int r = 0; r < kR; ++r)
+    for (int r = 0; r < R; ++r) {
+        const int i = ib + r;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ksum[r] += __shfl_xor_sync(0xffffffffu, ksum[r], o);
+        const float self = i >= jb && i < je && i < re ? (wn ? wn[i] : 1.f) : 0.f;
 #pragma unroll
         for (int q = 0; q < DP; ++q) {
             const int d = lane + 32 * q;
-            if (ib + r < re && d < D)
-                out[(size_t)(ib - row0 + r) * D + d] = (ag[r][q] + two_h * ar[r][q]) * inv_n;
+            if (i < re && d < D) {
+                float a0, a1;
+                unpack2(acc[r / 2][q], a0, a1);
+                float v = fmaf(two_h * (theta[(size_t)i * D + d] - c[q]), ksum[r], r % 2 ? a1 : a0);
+                if (self != 0.f) v = fmaf(self, grad[(size_t)i * D + d], v);
+                out[(size_t)(i - row0) * D + d] = v * inv_n;
+            }
         }
+    }
     if (tid == 0) {   // every wait has completed and the loop's last barrier passed
         mbar_inval(&bar[0]);
         mbar_inval(&bar[1]);

@@ -19,7 +19,6 @@
 namespace stamp {
 namespace {
 
-constexpr int kRows = 8;        // rows i per CTA (one warp each)
 constexpr int kTJ = 16;         // j per tile
 constexpr int kMaxHs = 16;      // actions per plan
 
@@ -45,98 +44,142 @@ __global__ void struct_prep_kernel(const float* __restrict__ theta, int N, int H
     C[(size_t)i * 2 * H + 2 * k + 1] = a[M + 1];
 }
 
+// A warp owns kRowsPerWarp rows; lane l owns columns l, l + 32, ... of each.  A
+// tile's grad, theta (its offsets and distances) and softmax rows are staged in
+// shared memory once per CTA; each pair and action costs two exponentials and
+// M multiply-adds there, spread over the CTA's threads, and each pair and
+// column four multiply-adds per lane.  The exponentials' weights (w_j, alpha,
+// 2/h) are folded into what is stored: A_ijk = alpha w_j (2/h) e_ijk.  GB300, N =
+// 1024, H = 4, M = 4: 184 -> 68 us (every lane used to read its j's values from
+// global memory, one row per warp).
+constexpr int kRowsPerWarp = 2, kWarps = 8, kRows = kRowsPerWarp * kWarps;
+__host__ __device__ constexpr size_t struct_smem(int D, int H) {
+    return ((size_t)(2 * kTJ + kRows) * D + (size_t)kRows * kTJ * (3 * H + 1)) * sizeof(float);
+}
 template <int DP>
-__global__ void __launch_bounds__(kRows * 32)
+__global__ void __launch_bounds__(kWarps * 32)
 struct_phi_kernel(const float* __restrict__ theta, const float* __restrict__ grad,
-                  const float* __restrict__ C, const float* __restrict__ S, int N, int H, int M,
+                  const float* __restrict__ S, int N, int H, int M,
                   const float* __restrict__ hc_dev, const float* __restrict__ hz_dev,
                   const float* __restrict__ wn, float* __restrict__ phi, int j_chunk) {
-    __shared__ float Ec[kRows][kTJ][kMaxHs + 1], Ez[kRows][kTJ][kMaxHs + 1], Q[kRows][kTJ][kMaxHs + 1];
-    __shared__ float Ks[kRows][kTJ];
+    extern __shared__ float ssm[];
     const int P = M + 2, D = H * P;
+    // per column: softmax(a_k) on the logits, theta on (u_k, v_k)
+    float* Xi = ssm;                   // kRows x D
+    float* Xj = Xi + kRows * D;        // kTJ x D
+    float* Gj = Xj + kTJ * D;          // kTJ x D
+    float* Ac = Gj + kTJ * D;          // kRows x kTJ x H: alpha w_j (2/h_c) e^c
+    float* Az = Ac + kRows * kTJ * H;  // alpha w_j (2/h_z) e^z
+    float* Q = Az + kRows * kTJ * H;   // s_j . (s_i - s_j)
+    float* Ks = Q + kRows * kTJ * H;   // kRows x kTJ: w_j K_ij
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int i0 = blockIdx.x * kRows, i = i0 + warp;
+    const int i0 = blockIdx.x * kRows;
     const float Hf = (float)H;
     const float inv_hc = Hf / __ldg(hc_dev), inv_hz = Hf / __ldg(hz_dev);   // h = h_plain / H
-    const float alpha = 0.5f / Hf;
-    float ti[DP], si[DP], acc[DP];   // theta_i and, on logit slots, softmax(a_ik)
+    const float alpha = 0.5f / Hf, ac = alpha * (2.f * inv_hc), az = alpha * (2.f * inv_hz);
+    auto column = [&](int i, int d) {   // X of particle i
+        const int k = d / P, c = d - k * P;
+        return c < M ? S[(size_t)i * M * H + k * M + c] : theta[(size_t)i * D + d];
+    };
+    for (int t = tid; t < kRows * D; t += kWarps * 32) {
+        const int r = t / D, d = t % D;
+        Xi[t] = i0 + r < N ? column(i0 + r, d) : 0.f;
+    }
+    float xi[kRowsPerWarp][DP], acc[kRowsPerWarp][DP];
+    int kd[DP];
+    bool logit[DP];
 #pragma unroll
     for (int q = 0; q < DP; ++q) {
         const int d = lane + 32 * q;
-        const bool ok = i < N && d < D;
-        ti[q] = ok ? theta[(size_t)i * D + d] : 0.f;
-        si[q] = (ok && d % P < M) ? S[(size_t)i * M * H + (d / P) * M + d % P] : 0.f;
-        acc[q] = 0.f;
+        kd[q] = d < D ? d / P : 0;
+        logit[q] = d < D && d % P < M;
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r) {
+            const int i = i0 + warp * kRowsPerWarp + r;
+            xi[r][q] = i < N && d < D ? column(i, d) : 0.f;
+            acc[r][q] = 0.f;
+        }
     }
     // this CTA's share of the sum over j; partial directions go to share blockIdx.y
     const int jb = blockIdx.y * j_chunk, je = min(N, jb + j_chunk);
     phi += (size_t)blockIdx.y * N * D;
     for (int j0 = jb; j0 < je; j0 += kTJ) {
         const int nj = min(kTJ, je - j0);
-        // per (row, j, action): e^c, e^z and s_j.(s_i - s_j)
-        for (int e = tid; e < kRows * kTJ * H; e += kRows * 32) {
-            const int r = e / (kTJ * H), jj = (e / H) % kTJ, k = e % H;
-            const int ii = i0 + r, j = j0 + jj;
-            float ec = 0.f, ez = 0.f, q = 0.f;
-            if (ii < N && jj < nj) {
-                const float* ci = C + (size_t)ii * 2 * H + 2 * k;
-                const float* cj = C + (size_t)j * 2 * H + 2 * k;
-                const float du = __ldg(ci) - __ldg(cj), dv = __ldg(ci + 1) - __ldg(cj + 1);
-                ec = expf(-(du * du + dv * dv) * inv_hc);
-                const float* s_i = S + (size_t)ii * M * H + k * M;
-                const float* s_j = S + (size_t)j * M * H + k * M;
-                float dz = 0.f;
-                for (int c = 0; c < M; ++c) {
-                    const float a = __ldg(s_i + c), b = __ldg(s_j + c), x = a - b;
-                    dz = fmaf(x, x, dz);
-                    q = fmaf(b, x, q);
-                }
-                ez = expf(-dz * inv_hz);
-            }
-            Ec[r][jj][k] = ec;
-            Ez[r][jj][k] = ez;
-            Q[r][jj][k] = q;
+        for (int t = tid; t < kTJ * D; t += kWarps * 32) {
+            const int jj = t / D, d = t % D;
+            Xj[t] = jj < nj ? column(j0 + jj, d) : 0.f;
+            Gj[t] = jj < nj ? grad[(size_t)j0 * D + t] : 0.f;
         }
         __syncthreads();
-        if (tid < kRows * kTJ) {   // K_ij = alpha sum_k (e^c + e^z), times wn_j (or 1; 1/N at the end)
-            const int r = tid / kTJ, jj = tid % kTJ;
+        // one (row, j) pair per thread: every action's kernels, and their sum K
+        for (int e = tid; e < kRows * kTJ; e += kWarps * 32) {
+            const int r = e / kTJ, jj = e % kTJ;
+            const float w = jj < nj ? (wn ? wn[j0 + jj] : 1.f) : 0.f;
             float ksum = 0.f;
-            for (int k = 0; k < H; ++k) ksum += Ec[r][jj][k] + Ez[r][jj][k];
-            const float w = (jj < nj && wn) ? wn[j0 + jj] : 1.f;
-            Ks[r][jj] = jj < nj ? alpha * ksum * w : 0.f;
+            for (int k = 0; k < H; ++k) {
+                const float* a = Xi + r * D + k * P;
+                const float* b = Xj + jj * D + k * P;
+                float dz = 0.f, q = 0.f;
+                for (int c = 0; c < M; ++c) {
+                    const float bc = b[c], x = a[c] - bc;
+                    dz = fmaf(x, x, dz);
+                    q = fmaf(bc, x, q);
+                }
+                const float du = a[M] - b[M], dv = a[M + 1] - b[M + 1];
+                const float ec = expf(-(du * du + dv * dv) * inv_hc);
+                const float ez = expf(-dz * inv_hz);
+                ksum += ec + ez;
+                const int o = (r * kTJ + jj) * H + k;
+                Ac[o] = ac * w * ec;
+                Az[o] = az * w * ez;
+                Q[o] = q;
+            }
+            Ks[e] = alpha * ksum * w;
         }
         __syncthreads();
-        if (i < N) {
-            for (int jj = 0; jj < nj; ++jj) {
-                const int j = j0 + jj;
-                const float kij = Ks[warp][jj];
-                const float w = wn ? wn[j] : 1.f;
+        for (int jj = 0; jj < nj; ++jj) {
 #pragma unroll
-                for (int q = 0; q < DP; ++q) {
-                    const int d = lane + 32 * q;
-                    if (d >= D) continue;
-                    const int k = d / P, comp = d % P;
-                    const float gj = __ldg(grad + (size_t)j * D + d);
-                    float rep;
-                    if (comp < M) {
-                        const float sj = __ldg(S + (size_t)j * M * H + k * M + comp);
-                        rep = 2.f * inv_hz * Ez[warp][jj][k] * sj * ((si[q] - sj) - Q[warp][jj][k]);
-                    } else {
-                        rep = 2.f * inv_hc * Ec[warp][jj][k] * (ti[q] - __ldg(theta + (size_t)j * D + d));
-                    }
-                    acc[q] = fmaf(kij, gj, fmaf(alpha * w, rep, acc[q]));
+            for (int q = 0; q < DP; ++q) {
+                const int d = lane + 32 * q;
+                if (d >= D) continue;
+                const float g = Gj[jj * D + d], x = Xj[jj * D + d];
+#pragma unroll
+                for (int r = 0; r < kRowsPerWarp; ++r) {
+                    const int rj = (warp * kRowsPerWarp + r) * kTJ + jj, o = rj * H + kd[q];
+                    // logits: A^z s_j ((s_i - s_j) - q); offset, distance: A^c (c_i - c_j)
+                    const float rep = logit[q] ? Az[o] * (x * ((xi[r][q] - x) - Q[o]))
+                                               : Ac[o] * (xi[r][q] - x);
+                    acc[r][q] = fmaf(Ks[rj], g, acc[r][q] + rep);
                 }
             }
         }
         __syncthreads();
     }
     const float scale = wn ? 1.f : 1.f / (float)N;
-    if (i < N)
 #pragma unroll
-        for (int q = 0; q < DP; ++q) {
-            const int d = lane + 32 * q;
-            if (d < D) phi[(size_t)i * D + d] = acc[q] * scale;
-        }
+    for (int r = 0; r < kRowsPerWarp; ++r) {
+        const int i = i0 + warp * kRowsPerWarp + r;
+        if (i < N)
+#pragma unroll
+            for (int q = 0; q < DP; ++q) {
+                const int d = lane + 32 * q;
+                if (d < D) phi[(size_t)i * D + d] = acc[r][q] * scale;
+            }
+    }
+}
+
+template <int DP>
+cudaError_t struct_launch(dim3 grid, const float* theta, const float* grad, const float* S, int N, int H,
+                          int M, const float* hc, const float* hz, const float* wn, float* phi,
+                          int j_chunk, cudaStream_t st) {
+    const size_t smem = struct_smem(H * (M + 2), H);
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(struct_phi_kernel<DP>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    struct_phi_kernel<DP><<<grid, kWarps * 32, smem, st>>>(theta, grad, S, N, H, M, hc, hz, wn, phi, j_chunk);
+    return cudaGetLastError();
 }
 
 __global__ void scale_scalar_kernel(const float* src, float s, float* dst) { *dst = *src * s; }
@@ -154,7 +197,7 @@ cudaError_t launch_struct_prep(const float* theta, int N, int H, int M, float* C
     return cudaGetLastError();
 }
 
-cudaError_t launch_struct_phi(const float* theta, const float* grad, const float* C, const float* S,
+cudaError_t launch_struct_phi(const float* theta, const float* grad, const float* S,
                               int N, int H, int M, const float* hc_dev, const float* hz_dev,
                               const float* wn, float* phi, int max_shares, int* shares,
                               cudaStream_t st) {
@@ -167,15 +210,14 @@ cudaError_t launch_struct_phi(const float* theta, const float* grad, const float
     *shares = (N + j_chunk - 1) / j_chunk;
     const dim3 grid(rows, *shares);
     switch ((D + 31) / 32) {
-        case 1: struct_phi_kernel<1><<<grid, kRows * 32, 0, st>>>(theta, grad, C, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk); break;
-        case 2: struct_phi_kernel<2><<<grid, kRows * 32, 0, st>>>(theta, grad, C, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk); break;
-        case 3: struct_phi_kernel<3><<<grid, kRows * 32, 0, st>>>(theta, grad, C, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk); break;
-        case 4: struct_phi_kernel<4><<<grid, kRows * 32, 0, st>>>(theta, grad, C, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk); break;
-        case 5: case 6: struct_phi_kernel<6><<<grid, kRows * 32, 0, st>>>(theta, grad, C, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk); break;
-        case 7: case 8: case 9: struct_phi_kernel<9><<<grid, kRows * 32, 0, st>>>(theta, grad, C, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk); break;
-        default: return cudaErrorInvalidValue;
+        case 1: return struct_launch<1>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
+        case 2: return struct_launch<2>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
+        case 3: return struct_launch<3>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
+        case 4: return struct_launch<4>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
+        case 5: case 6: return struct_launch<6>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
+        case 7: case 8: case 9: return struct_launch<9>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace stamp
