@@ -18,6 +18,8 @@
 
 #include "mlp.cuh"
 #include "rollout.cuh"
+#include "surrogate_mlp.cuh"
+#include "svgd_bodies.cuh"
 #include "stamp.h"
 #include "stamp_internal.cuh"
 
@@ -28,7 +30,6 @@ constexpr uint64_t kStreamPoses = 2, kStreamActions = 3;
 constexpr int kChunk = 4096;         // transitions per chunk (one key each)
 constexpr int kTrainRows = 16384;    // largest training minibatch
 constexpr int kAttempts = 32;        // rejection-sampling attempts per start scene
-constexpr int kSelectChunk = 8192;   // keys sorted by one CTA of the screening selection
 
 // Features of push k (and the stored relaxation).  Pose source: the scene's
 // start poses (src NULL), else src (+ delta when given); the pose used is
@@ -103,42 +104,6 @@ cost_kernel(const SimConst sc, int N, const float* __restrict__ src, const float
     if (stats_min) atomicMin(stats_min, __float_as_uint(c));
 }
 
-// Reverse of push k's features: dx (N x F, dC/df_k) is added into the pose
-// adjoint (which holds dC/dq_{k+1} on entry and dC/dq_k on exit) and gives
-// grad log rho = -dC/dtheta for push k's parameters (with the w_push term).
-template <int NB>
-__global__ void __launch_bounds__(128)
-features_bwd_kernel(const SimConst sc, int N, int k, const float* __restrict__ pose,
-                    const float* __restrict__ relax, const float* __restrict__ dx,
-                    float* __restrict__ apose, float* __restrict__ grad) {
-    constexpr int M = rollout::Dims<NB>::M, P = M + 2, IN = 8 * NB + 2;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const float* di = dx + (size_t)i * IN;
-    const float* pi = pose + (size_t)i * 3 * NB;
-    float* ai = apose + (size_t)i * 3 * NB;
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        float sn, cs;
-        sincosf(pi[3 * b + 2], &sn, &cs);
-        ai[3 * b] += di[4 * b];
-        ai[3 * b + 1] += di[4 * b + 1];
-        ai[3 * b + 2] += cs * di[4 * b + 3] - sn * di[4 * b + 2];
-    }
-    const float* ri = relax + ((size_t)i * sc.H + k) * P;
-    float zg = 0.f;
-#pragma unroll
-    for (int c = 0; c < M; ++c) zg += ri[c] * di[4 * NB + c];
-    float* gi = grad + (size_t)i * sc.D + k * P;
-    // softmax((a+g)/tau): dC/da_j = z_j (dC/dz_j - sum_c z_c dC/dz_c) / tau
-#pragma unroll
-    for (int c = 0; c < M; ++c) gi[c] = -(ri[c] * (di[4 * NB + c] - zg) * sc.inv_tau);
-    const float tu = ri[M], sv = ri[M + 1];
-    gi[M] = -(di[4 * NB + M] * (1.f - tu * tu));
-    const float dist = sc.dist_max * sv;
-    gi[M + 1] = -((di[4 * NB + M + 1] + 2.f * sc.w_push * dist * sc.dist_max) * sv * (1.f - sv));
-}
-
 // Random start scenes: the first of kAttempts counter-based draws whose block
 // centres are all more than 0.16 m apart; products and sums in float32 with
 // explicit rounding so that the accept decision is reproducible.
@@ -195,46 +160,89 @@ __global__ void delta_kernel(int m, int nb, const float* __restrict__ start,
     y[t] = final_state[(size_t)i * 6 * nb + 6 * b + q] - start[t];
 }
 
-// Sort keys (cost bits << 32 | index; a negative or NaN cost sorts last).
-__global__ void keys_kernel(const float* __restrict__ cost, int n, unsigned long long* __restrict__ keys) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    unsigned cb = __float_as_uint(cost[t]);
-    if (cb >= 0x7F800001u) cb = 0xFFFFFFFFu;
-    keys[t] = ((unsigned long long)cb << 32) | (unsigned)t;
+// Selection of the N lowest (cost, index) pairs.  Five digit passes find the
+// N-th pair exactly -- the cost's bits (11 + 11 + 10), then the index (10 + 10)
+// among equal costs -- each counting the pairs that match the digits so far;
+// the last CTA of a pass picks the next digit.  The N pairs up to it are then
+// gathered in any order, and each one's place is the number of smaller ones.
+// 131072 candidates to 2048 on GB300: 50 us; sorting 8192-key chunks in three
+// passes took 215.
+constexpr int kSelBins = 2048, kSelPasses = 5;
+constexpr size_t kSelBytes = (kSelPasses * kSelBins + 24) * sizeof(unsigned);
+struct Select {
+    unsigned* hist;      // kSelPasses x kSelBins, zeroed
+    unsigned* state;     // [0, 5): counters of finished CTAs, [5]: pairs gathered (zeroed);
+                         // [8 + 2 p]: pass p's digit, [9 + 2 p]: rank inside it
+};
+// The digit of pass p, and whether the pair matches the digits before it.
+__device__ __forceinline__ bool sel_digit(unsigned v, unsigned idx, int p, const unsigned* st, unsigned& d) {
+    switch (p) {
+        case 0: d = v >> 21; return true;
+        case 1: d = (v >> 10) & 2047u; return v >> 21 == st[8];
+        case 2: d = v & 1023u; return v >> 10 == (st[8] << 11 | st[10]);
+    }
+    const bool eq = v == (st[8] << 21 | st[10] << 10 | st[12]);
+    if (p == 3) { d = idx >> 10; return eq; }
+    d = idx & 1023u;
+    return eq && idx >> 10 == st[14];
 }
-
-// Each CTA bitonic-sorts one chunk of kSelectChunk keys in shared memory
-// (missing keys padded with the largest key) and writes its `keep` smallest.
-__global__ void __launch_bounds__(1024)
-select_kernel(const unsigned long long* __restrict__ in, int n, int keep,
-              unsigned long long* __restrict__ out) {
-    extern __shared__ unsigned long long key[];
-    const int c0 = blockIdx.x * kSelectChunk, m = min(kSelectChunk, n - c0);
-    for (int t = threadIdx.x; t < kSelectChunk; t += blockDim.x) key[t] = t < m ? in[c0 + t] : ~0ull;
+__device__ __forceinline__ unsigned cost_key(float cost) {   // a negative or NaN cost sorts last
+    const unsigned cb = __float_as_uint(cost);
+    return cb >= 0x7F800001u ? 0xFFFFFFFFu : cb;
+}
+__global__ void __launch_bounds__(256) select_pass_kernel(const float* __restrict__ cost, int n, int N,
+                                                          int p, Select s) {
+    __shared__ unsigned h[kSelBins], st[24];
+    for (int t = threadIdx.x; t < kSelBins; t += 256) h[t] = 0u;
+    if (threadIdx.x < 24) st[threadIdx.x] = __ldcg(s.state + threadIdx.x);
     __syncthreads();
-    for (int size = 2; size <= kSelectChunk; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = threadIdx.x; t < kSelectChunk / 2; t += blockDim.x) {
-                const int lo = 2 * t - (t & (stride - 1)), hi = lo + stride;
-                const bool up = (lo & size) == 0;
-                const unsigned long long a = key[lo], b = key[hi];
-                if ((a > b) == up) { key[lo] = b; key[hi] = a; }
-            }
-            __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int t0 = blockIdx.x * 256; t0 < n; t0 += gridDim.x * 256) {
+        const int t = t0 + (int)threadIdx.x;
+        unsigned d = 0;
+        const bool in = t < n && sel_digit(cost_key(cost[t]), (unsigned)t, p, st, d);
+        // equal digits of the warp at once (costs share a few exponents)
+        const unsigned same = __match_any_sync(0xffffffffu, in ? d : 0xffffffffu);
+        if (in && lane == __ffs(same) - 1) atomicAdd(&h[d], (unsigned)__popc(same));
+    }
+    __syncthreads();
+    unsigned* out = s.hist + p * kSelBins;
+    for (int t = threadIdx.x; t < kSelBins; t += 256)
+        if (h[t]) atomicAdd(&out[t], h[t]);
+    if (last_block(s.state + p, gridDim.x)) {
+        unsigned bin, rem;
+        find_bin<kSelBins, 256>(out, p == 0 ? (unsigned)(N - 1) : st[7 + 2 * p], bin, rem);
+        if (threadIdx.x == 0) {
+            s.state[8 + 2 * p] = bin;
+            s.state[9 + 2 * p] = rem;
         }
-    for (int t = threadIdx.x; t < keep; t += blockDim.x) out[(size_t)blockIdx.x * keep + t] = key[t];
+    }
 }
-
-__global__ void gather_kernel(const unsigned long long* __restrict__ keys, int N, int D,
-                              const float* __restrict__ cand, float* __restrict__ theta,
-                              int* __restrict__ index) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= N * D) return;
-    const int i = t / D, d = t % D;
-    const int src = (int)(keys[i] & 0xFFFFFFFFull);
-    theta[t] = cand[(size_t)src * D + d];
-    if (index && d == 0) index[i] = src;
+__global__ void __launch_bounds__(256) select_gather_kernel(const float* __restrict__ cost, int n, Select s,
+                                                            unsigned long long* __restrict__ out) {
+    const unsigned* st = s.state;
+    const unsigned long long last = (unsigned long long)(st[8] << 21 | st[10] << 10 | st[12]) << 32 |
+                                    (st[14] << 10 | st[16]);
+    const int t = blockIdx.x * 256 + threadIdx.x;
+    if (t >= n) return;
+    const unsigned long long key = (unsigned long long)cost_key(cost[t]) << 32 | (unsigned)t;
+    if (key <= last) out[atomicAdd(s.state + 5, 1u)] = key;
+}
+// Places of 8 of the N pairs per CTA (a warp each), and their candidates' copies.
+__global__ void __launch_bounds__(256) select_place_kernel(const unsigned long long* __restrict__ keys,
+                                                           int N, int D, const float* __restrict__ cand,
+                                                           float* __restrict__ theta,
+                                                           int* __restrict__ index) {
+    const int lane = threadIdx.x & 31, q = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (q >= N) return;
+    const unsigned long long key = keys[q];
+    unsigned below = 0;
+    for (int t = lane; t < N; t += 32) below += keys[t] < key;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
+    const int src = (int)(key & 0xFFFFFFFFull);
+    for (int d = lane; d < D; d += 32) theta[(size_t)below * D + d] = cand[(size_t)src * D + d];
+    if (index && lane == 0) index[below] = src;
 }
 
 // Uniform(-1/sqrt(fan_in), 1/sqrt(fan_in)) parameters; draw t of key `seed`.
@@ -357,13 +365,6 @@ cudaError_t cost(const SimConst& sc, int N, const float* src, const float* delta
     cost_kernel<NB><<<(N + 127) / 128, 128, 0, st>>>(sc, N, src, delta, relax, c, apose, stats);
     return cudaGetLastError();
 }
-template <int NB>
-cudaError_t features_bwd(const SimConst& sc, int N, int k, const float* pose, const float* relax,
-                         const float* dx, float* apose, float* grad, cudaStream_t st) {
-    features_bwd_kernel<NB><<<(N + 127) / 128, 128, 0, st>>>(sc, N, k, pose, relax, dx, apose, grad);
-    return cudaGetLastError();
-}
-
 cudaError_t features_nb(const SimConst& sc, const float* theta, int N, int k, uint64_t seed, int iter,
                         const float* src, const float* delta, float* pose_out, float* x, float* relax,
                         cudaStream_t st) {
@@ -383,15 +384,6 @@ cudaError_t cost_nb(const SimConst& sc, int N, const float* src, const float* de
     }
     return cudaErrorInvalidValue;
 }
-cudaError_t features_bwd_nb(const SimConst& sc, int N, int k, const float* pose, const float* relax,
-                            const float* dx, float* apose, float* grad, cudaStream_t st) {
-    switch (sc.nb) {
-        case 1: return features_bwd<1>(sc, N, k, pose, relax, dx, apose, grad, st);
-        case 2: return features_bwd<2>(sc, N, k, pose, relax, dx, apose, grad, st);
-        case 3: return features_bwd<3>(sc, N, k, pose, relax, dx, apose, grad, st);
-    }
-    return cudaErrorInvalidValue;
-}
 
 }  // namespace surrogate
 }  // namespace stamp
@@ -405,10 +397,11 @@ struct stamp_surrogate {
     stamp_mlp* mlp = nullptr;
     stamp_problem* trans = nullptr;   // one-push simulator (H = 1) for transitions
     char* arena = nullptr;
-    float *params = nullptr, *pose = nullptr, *x = nullptr, *y = nullptr, *relax = nullptr,
-          *apose = nullptr, *dx = nullptr, *cost = nullptr, *cand = nullptr, *tstart = nullptr,
+    float *params = nullptr, *pose = nullptr, *y = nullptr, *relax = nullptr,
+          *apose = nullptr, *cost = nullptr, *cand = nullptr, *tstart = nullptr,
           *tfinal = nullptr, *taction = nullptr, *tcost = nullptr;
-    unsigned long long *keys = nullptr, *keys2 = nullptr;
+    unsigned long long* keys = nullptr;   // the screened (cost, index) pairs
+    unsigned* sel = nullptr;              // selection histograms and state
 };
 
 namespace {
@@ -458,29 +451,25 @@ stamp_status surrogate_rollout(stamp_surrogate* s, const SimConst& sc, const flo
     const bool rev = grad != nullptr;
     if (N < 1 || N > (rev ? s->max_n : s->max_rows))
         return sur_fail(STAMP_EINVAL, "N outside the surrogate's capacity");
-    const int S3 = 3 * s->nb, tiles = (N + 127) / 128;
+    const int S3 = 3 * s->nb;
     cudaStream_t st = s->stream;
-    for (int k = 0; k < sc.H; ++k) {
-        const float* prev = k ? s->pose + (size_t)(k - 1) * N * S3 : nullptr;
-        SUR_CUDA(surrogate::features_nb(sc, theta, N, k, seed, iter, prev, k ? s->y : nullptr,
-                                        s->pose + (size_t)k * N * S3, s->x, s->relax, st),
-                 "feature launch failed");
-        SUR_TRY(rev ? stamp_mlp_forward_saved(s->mlp, s->x, N, s->y, k * tiles)
-                    : stamp_mlp_forward(s->mlp, s->x, N, s->y));
-    }
+    const mlp::View net = mlp::view(s->mlp);
+    mlp::SurArgs a{};
+    a.theta = theta; a.N = N; a.n_tiles = (N + 127) / 128; a.seed = seed; a.iter = iter;
+    a.w_tiled = net.w_tiled; a.wt_tiled = net.wt_tiled; a.bias = net.bias;
+    a.pose = s->pose; a.y = s->y; a.relax = s->relax;
+    a.zsave = rev ? net.zsave : nullptr; a.tile_cap = net.tile_cap;
+    a.apose = s->apose; a.grad = grad; a.err = net.err;
+    SUR_CUDA(mlp::surrogate_pass(sc, a, false, net.sm_count, st), "surrogate rollout launch failed");
     SUR_CUDA(surrogate::cost_nb(sc, N, s->pose + (size_t)(sc.H - 1) * N * S3, s->y, s->relax, cost,
                                 rev ? s->apose : nullptr, stats_word, st),
              "cost launch failed");
-    if (!rev) return STAMP_OK;
-    for (int k = sc.H - 1; k >= 0; --k) {
-        // q_{k+1} = q_k + y_k: dC/dy_k = dC/dq_{k+1}
-        SUR_TRY(stamp_mlp_backward(s->mlp, s->apose, N, k * tiles, s->dx, nullptr));
-        SUR_CUDA(surrogate::features_bwd_nb(sc, N, k, s->pose + (size_t)k * N * S3, s->relax, s->dx,
-                                            s->apose, grad, st),
-                 "feature backward failed");
-    }
+    // q_{k+1} = q_k + y_k: dC/dy_k = dC/dq_{k+1}
+    if (rev) SUR_CUDA(mlp::surrogate_pass(sc, a, true, net.sm_count, st), "surrogate reverse launch failed");
     return STAMP_OK;
 }
+
+static int net_sms(const stamp_surrogate* s) { return mlp::view(s->mlp).sm_count; }
 
 stamp_status surrogate_screen(stamp_surrogate* s, const SimConst& sc, const float* cand, int n_cand,
                               int N, float* theta_out, int* index_out) {
@@ -488,22 +477,15 @@ stamp_status surrogate_screen(stamp_surrogate* s, const SimConst& sc, const floa
     if (N < 1 || N > n_cand || N > kMaxScreenN || n_cand > s->max_rows)
         return sur_fail(STAMP_EINVAL, "need 1 <= N <= min(n_candidates, 4096) and n_candidates <= max_rows");
     SUR_TRY(surrogate_rollout(s, sc, cand, n_cand, 0, -1, s->cost, nullptr, nullptr));
-    using surrogate::kSelectChunk;
-    const size_t smem = kSelectChunk * sizeof(unsigned long long);
-    SUR_CUDA(cudaFuncSetAttribute(surrogate::select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem), "shared-memory opt-in failed");
-    surrogate::keys_kernel<<<(n_cand + 255) / 256, 256, 0, s->stream>>>(s->cost, n_cand, s->keys);
-    unsigned long long *a = s->keys, *b = s->keys2;
-    int n = n_cand;
-    while (n > kSelectChunk) {   // N <= 4096 keeps at most half of every full chunk: n shrinks
-        const int chunks = (n + kSelectChunk - 1) / kSelectChunk;
-        surrogate::select_kernel<<<chunks, 1024, smem, s->stream>>>(a, n, N, b);
-        n = chunks * N;
-        std::swap(a, b);
-    }
-    surrogate::select_kernel<<<1, 1024, smem, s->stream>>>(a, n, N, b);
-    const int D = sc.D;
-    surrogate::gather_kernel<<<(N * D + 255) / 256, 256, 0, s->stream>>>(b, N, D, cand, theta_out, index_out);
+    const surrogate::Select sel{s->sel, s->sel + surrogate::kSelPasses * surrogate::kSelBins};
+    SUR_CUDA(cudaMemsetAsync(s->sel, 0, surrogate::kSelBytes, s->stream), "clearing the selection failed");
+    // four candidates a thread: enough CTAs to fill the GPU, few flushes of the bins
+    const int grid = std::min(2 * net_sms(s), (n_cand + 1023) / 1024);
+    for (int p = 0; p < surrogate::kSelPasses; ++p)
+        surrogate::select_pass_kernel<<<grid, 256, 0, s->stream>>>(s->cost, n_cand, N, p, sel);
+    surrogate::select_gather_kernel<<<(n_cand + 255) / 256, 256, 0, s->stream>>>(s->cost, n_cand, sel, s->keys);
+    surrogate::select_place_kernel<<<(N + 7) / 8, 256, 0, s->stream>>>(s->keys, N, sc.D, cand, theta_out,
+                                                                       index_out);
     SUR_CUDA(cudaGetLastError(), "selection launch failed");
     return STAMP_OK;
 }
@@ -545,14 +527,15 @@ stamp_status stamp_surrogate_create(const stamp_problem_desc* desc, int max_rows
     stamp_status r = stamp_mlp_create(s->in_dim, s->out_dim, (int)R, train_rows, cuda_stream, &s->mlp);
     if (r != STAMP_OK) { stamp_problem_destroy(trans); delete s; return r; }
     const size_t C = stamp::surrogate::kChunk;
-    const size_t bytes[] = {s->n_params * 4, (size_t)s->max_H * R * S3 * 4, R * s->in_dim * 4,
+    const size_t bytes[] = {s->n_params * 4, (size_t)s->max_H * R * S3 * 4,
                             R * s->out_dim * 4, R * s->max_H * P * 4, (size_t)max_particles * S3 * 4,
-                            (size_t)max_particles * s->in_dim * 4, R * 4, R * s->max_H * P * 4,
-                            C * S3 * 4, C * 6 * s->nb * 4, C * P * 4, C * 4, R * 8, R * 8};
-    void** dst[] = {(void**)&s->params, (void**)&s->pose, (void**)&s->x, (void**)&s->y,
-                    (void**)&s->relax, (void**)&s->apose, (void**)&s->dx, (void**)&s->cost,
+                            R * 4, R * s->max_H * P * 4,
+                            C * S3 * 4, C * 6 * s->nb * 4, C * P * 4, C * 4, (size_t)stamp::kMaxScreenN * 8,
+                            stamp::surrogate::kSelBytes};
+    void** dst[] = {(void**)&s->params, (void**)&s->pose, (void**)&s->y,
+                    (void**)&s->relax, (void**)&s->apose, (void**)&s->cost,
                     (void**)&s->cand, (void**)&s->tstart, (void**)&s->tfinal, (void**)&s->taction,
-                    (void**)&s->tcost, (void**)&s->keys, (void**)&s->keys2};
+                    (void**)&s->tcost, (void**)&s->keys, (void**)&s->sel};
     size_t total = 0;
     for (size_t b : bytes) total += (b + 255) / 256 * 256;
     cudaError_t e = cudaMalloc(&s->arena, total);
