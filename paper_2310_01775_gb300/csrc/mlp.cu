@@ -26,16 +26,20 @@ namespace stamp {
 namespace mlp {
 namespace {
 
-// Forward of all four layers for 128-row tiles; y: rows x kOut FP32.
-// Optionally stores, for the backward pass, the input activations a_1..a_3 and
-// the pre-activations z_0..z_2 (BF16 tiles): slot (l, tile_base + tile) of
-// buffers holding tile_cap tiles per layer.
+// Forward of all four layers for 128-row tiles: x (rows x in_dim FP32) becomes
+// layer 0's operand, rounded to BF16 and zero-padded, on the way in, and the
+// head writes the out_dim columns of y (row stride ldy).  Optionally stores,
+// for the backward pass, the input tile a_0 (x_tiled), the input activations
+// a_1..a_3 and the pre-activations z_0..z_2 (BF16 tiles): slot (l, tile_base +
+// tile) of buffers holding tile_cap tiles per layer.  Packing the input and
+// unpacking a padded output in launches of their own cost 3.8 + 3.0 us at 16384
+// rows beside the 18.2 of this kernel (GB300).
 __global__ void __launch_bounds__(kThreads, 1)
-mlp_fwd_kernel(const unsigned char* __restrict__ x_tiled, int n_tiles,
+mlp_fwd_kernel(const float* __restrict__ x, int in_dim, unsigned char* __restrict__ x_tiled, int n_tiles,
                const unsigned char* __restrict__ w_tiled, const float* __restrict__ bias,
-               float* __restrict__ y, int rows, unsigned char* __restrict__ saved,
-               unsigned char* __restrict__ zsave, int tile_base, int tile_cap,
-               int* __restrict__ err) {
+               float* __restrict__ y, int ldy, int out_dim, int rows,
+               unsigned char* __restrict__ saved, unsigned char* __restrict__ zsave, int tile_base,
+               int tile_cap, int* __restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     FwdSmem& sm = *reinterpret_cast<FwdSmem*>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -51,16 +55,33 @@ mlp_fwd_kernel(const unsigned char* __restrict__ x_tiled, int n_tiles,
     const unsigned tmem = sm.tmem_slot;
     unsigned tma_phase = 0, mma_phase = 0;
     bool failed = false, tma_pending = false, mma_pending = false;
-    // weights of layer l (and, for l = 0, the tile's input) into shared memory
-    auto issue_load = [&](int l, int tile) {
+    auto issue_load = [&](int l) {   // layer l's weights into shared memory
         const unsigned wbytes = (unsigned)(layer_n(l) * layer_k(l) * 2);
-        mbar_expect_tx(&sm.tma_bar, wbytes + (l == 0 ? kInBytes : 0u));
+        mbar_expect_tx(&sm.tma_bar, wbytes);
         tma_load_1d(sm.w, w_tiled + layer_w_offset(l), wbytes, &sm.tma_bar);
-        if (l == 0) tma_load_1d(sm.act, x_tiled + (size_t)tile * kInBytes, kInBytes, &sm.tma_bar);
+    };
+    // a tile's input: thread -> row tid % 128, columns 8 (tid / 128) ...
+    const int xr = tid % kRows, xc = tid / kRows * 8;
+    float xv[8];
+    auto read_x = [&](int tile) {
+        const int r = tile * kRows + xr;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            xv[c] = r < rows && xc + c < in_dim ? __ldg(x + (size_t)r * in_dim + xc + c) : 0.f;
+    };
+    auto put_x = [&](int tile) {
+        const uint4 pk = make_uint4(pack_bf16(xv[0], xv[1]), pack_bf16(xv[2], xv[3]),
+                                    pack_bf16(xv[4], xv[5]), pack_bf16(xv[6], xv[7]));
+        const unsigned off = tile_off(xr, xc, kIn);
+        *reinterpret_cast<uint4*>(sm.act + off) = pk;
+        if (saved) *reinterpret_cast<uint4*>(x_tiled + (size_t)(tile_base + tile) * kInBytes + off) = pk;
     };
     if (blockIdx.x < n_tiles) {
-        if (tid == 0) issue_load(0, blockIdx.x);
+        if (tid == 0) issue_load(0);
         tma_pending = true;
+        read_x(blockIdx.x);
+        put_x(blockIdx.x);
+        fence_async_shared();
     }
     for (int tile = blockIdx.x; tile < n_tiles && !failed; tile += gridDim.x) {
         for (int l = 0; l < 4 && !failed; ++l) {
@@ -81,6 +102,7 @@ mlp_fwd_kernel(const unsigned char* __restrict__ x_tiled, int n_tiles,
                 mma_commit(&sm.mma_bar);
             }
             mma_pending = true;
+            if (l == 3 && tile + (int)gridDim.x < n_tiles) read_x(tile + gridDim.x);
             if (saved && l > 0) {   // this layer's input activation, for the backward pass
                 // (read beside the MMA, which only reads it too)
                 unsigned char* dst = saved + ((size_t)l * tile_cap + tile_base + tile) * kActBytes;
@@ -94,14 +116,12 @@ mlp_fwd_kernel(const unsigned char* __restrict__ x_tiled, int n_tiles,
             mma_phase ^= 1u;
             mma_pending = false;
             tc_fence_after();
-            // the weight buffer is free (and, after the last layer, the input
-            // buffer): start the next layer's (or next tile's) copy now, so it
-            // runs beside this epilogue
-            const int next_l = l < 3 ? l + 1 : 0, next_tile = l < 3 ? tile : tile + gridDim.x;
-            if (next_tile < n_tiles) {
+            // the weight buffer is free: start the next layer's (or next tile's)
+            // copy now, so it runs beside this epilogue
+            if (l < 3 || tile + (int)gridDim.x < n_tiles) {
                 if (tid == 0) {
                     fence_async_shared();
-                    issue_load(next_l, next_tile);
+                    issue_load(l < 3 ? l + 1 : 0);
                 }
                 tma_pending = true;
             }
@@ -135,17 +155,18 @@ mlp_fwd_kernel(const unsigned char* __restrict__ x_tiled, int n_tiles,
                                 zsave + ((size_t)l * tile_cap + tile_base + tile) * kActBytes + off) = pz;
                     }
                 }
-            } else if (half == 0) {
-                float v[16];
-                tmem_ld16(lane_base, v);
-                const int r = tile * kRows + row;
-                if (r < rows) {
-                    float4* dst = reinterpret_cast<float4*>(y + (size_t)r * kOut);
+            } else {
+                if (tile + (int)gridDim.x < n_tiles) put_x(tile + gridDim.x);   // act is free too
+                if (half == 0) {
+                    float v[16];
+                    tmem_ld16(lane_base, v);
+                    const int r = tile * kRows + row;
+                    if (r < rows) {
+                        float* dst = y + (size_t)r * ldy;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        dst[q] = make_float4(v[4 * q] + __ldg(bl + 4 * q), v[4 * q + 1] + __ldg(bl + 4 * q + 1),
-                                             v[4 * q + 2] + __ldg(bl + 4 * q + 2),
-                                             v[4 * q + 3] + __ldg(bl + 4 * q + 3));
+                        for (int c = 0; c < kOut; ++c)
+                            if (c < out_dim) dst[c] = v[c] + __ldg(bl + c);
+                    }
                 }
             }
             // the next MMA reads act (written here) and overwrites TMEM (read here)
@@ -167,20 +188,6 @@ mlp_fwd_kernel(const unsigned char* __restrict__ x_tiled, int n_tiles,
     }
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
-}
-
-// x (rows x in_dim FP32) -> zero-padded BF16 K-major tiles of 128 x kIn.
-__global__ void pack_input_kernel(const float* __restrict__ x, int rows, int in_dim,
-                                  unsigned char* __restrict__ out, int n_tiles) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int total = n_tiles * kRows * kIn;
-    if (t >= total) return;
-    const int tile = t / (kRows * kIn), rem = t % (kRows * kIn);
-    const int r = rem / kIn, c = rem % kIn;
-    const int gr = tile * kRows + r;
-    const float v = (gr < rows && c < in_dim) ? x[(size_t)gr * in_dim + c] : 0.f;
-    *reinterpret_cast<__nv_bfloat16*>(out + (size_t)tile * kInBytes + tile_off(r, c, kIn)) =
-        __float2bfloat16_rn(v);
 }
 
 // Master FP32 parameters (W_l as (n_l, k_l) real sizes, then b_l) -> packed BF16
@@ -346,44 +353,66 @@ mlp_bwd_kernel(const float* __restrict__ dy, int rows, int out_dim, int n_tiles,
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
-// 8x8 transpose of 16-bit elements across a warp: thread t holds row t/4,
-// columns 2(t%4) and 2(t%4)+1 before and after.
-__device__ __forceinline__ unsigned transpose8x8(unsigned x) {
-    unsigned y;
-    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
-    return y;
-}
-
-// Weight gradient of one layer on the tensor cores: the sum over rows of
-// outer products is an MMA whose reduction dimension K is the rows.  The
-// saved activations and dz tiles are K-major with K = units (a 128-byte core
-// matrix = 8 rows x 8 units); for this MMA the units become M and N and the
-// rows become K, so each core matrix is transposed (movmatrix) into the
-// K-major operand layout in shared memory:
-//   D (M = 128 units of P per blockIdx.x) x (N = NQ units of Q)
+// Weight gradients of all four layers in one launch: the sum over rows of
+// outer products is an MMA whose reduction dimension K is the rows.  The saved
+// activations and dz tiles hold, per 8 x 8 core matrix, 8 rows of 8 units:
+// units contiguous, so as operands over rows they are M/N-major as they lie
+// (descriptor: unit groups 128 B apart, row groups (units / 8) * 128 B apart;
+// the transpose bits of the instruction descriptor), and their tiles go to
+// shared memory by TMA as they are:
+//   D (M = 128 units of P, half mb) x (N = NQ units of Q)
 //     += P^T (M x 128 rows) . Q (128 rows x N)      per 128-row tile,
-// accumulated in TMEM over the tiles of this CTA's row split (blockIdx.y),
-// then stored as the split's partial; a second kernel sums the splits in
-// order (deterministic: no atomics).  The bias gradient of the dz operand's
-// units is summed from the transposed operand, rows in order, per split.
-constexpr int kDwMaxSplits = 128;
+// accumulated in TMEM over the tiles of the CTA's row split, two tiles in
+// flight; then stored as the split's partial, which a second launch sums in
+// split order (deterministic: no atomics).  The bias gradient of the dz
+// operand's units is summed beside the MMA, in a fixed order, per split.  The
+// splits give each SM one CTA with about the same bytes (the hidden layers'
+// 96 KB a tile, the outer ones' 40 and 36).  GB300, 16384 rows, cold caches: 19.5
+// us (52 MB from DRAM) and 10 us for the reduction; a launch per layer that
+// transposed every core matrix through registers (movmatrix), and its
+// reduction, took 80 + 44.
+constexpr int kDwMaxSplits = 32;     // of a layer
+constexpr unsigned kDwStage = 96 * 1024;   // P half (32 KB) and Q (up to 64 KB) of a tile
 struct DwSmem {
-    alignas(128) unsigned char A[kRows * kRows * 2];     // 32 KB: 128 units x 128 rows
-    alignas(128) unsigned char B[kHidden * kRows * 2];   // 64 KB: up to 256 units x 128 rows
-    uint64_t mma_bar;
+    alignas(128) unsigned char stage[2][kDwStage];
+    uint64_t full[2], mma_bar;
     unsigned tmem_slot;
 };
+struct DwLayer {
+    const unsigned char *P, *Q;   // first tile; P: 256 units, Q: NQ units
+    size_t p_stride, q_stride;    // bytes per tile
+    int NQ, dz_is_P, splits, per; // per: tiles per split
+    size_t part, bias;            // first float of the splits' partials
+    int out_r, in_r;              // real sizes of W
+    size_t w;                     // offset of W in the packed gradient
+    int cta0;                     // first CTA: (split, half) pairs, split-major
+    int e0;                       // first element of the reduction
+};
+struct DwArgs {
+    DwLayer l[kLayers];   // in order of their CTAs and elements
+    int n_tiles;
+    float *part, *grad;
+    int* err;
+};
 
-__global__ void __launch_bounds__(kThreads, 1)
-mlp_dw_tc_kernel(const unsigned char* __restrict__ P, int KP, size_t p_stride,
-                 const unsigned char* __restrict__ Q, int NQ, size_t q_stride, int n_tiles,
-                 int tiles_per_split, float* __restrict__ part, float* __restrict__ dbp,
-                 int dz_is_P, int* __restrict__ err) {
+__device__ __forceinline__ uint32_t idesc_bf16_mn(int M, int N) {   // both operands M/N-major
+    return idesc_bf16(M, N) | (1u << 15) | (1u << 16);
+}
+
+__global__ void __launch_bounds__(kThreads, 1) mlp_dw_kernel(const DwArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     DwSmem& sm = *reinterpret_cast<DwSmem*>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const unsigned cols = NQ <= 32 ? 32u : NQ <= 64 ? 64u : NQ <= 128 ? 128u : 256u;
+    int li = 0;
+#pragma unroll
+    for (int q = 1; q < kLayers; ++q)
+        if ((int)blockIdx.x >= a.l[q].cta0) li = q;
+    const DwLayer& L = a.l[li];
+    const int NQ = L.NQ, c = blockIdx.x - L.cta0, mb = c & 1, split = c >> 1;
+    const unsigned cols = NQ <= 32 ? 32u : 256u;
     if (tid == 0) {
+        mbar_init(&sm.full[0], 1);
+        mbar_init(&sm.full[1], 1);
         mbar_init(&sm.mma_bar, 1);
         fence_async_shared();
     }
@@ -392,81 +421,78 @@ mlp_dw_tc_kernel(const unsigned char* __restrict__ P, int KP, size_t p_stride,
     __syncthreads();
     tc_fence_after();
     const unsigned tmem = sm.tmem_slot;
-    const int mb = blockIdx.x, split = blockIdx.y;
-    const int t0 = split * tiles_per_split, t1 = min(n_tiles, t0 + tiles_per_split);
-    // the dz operand's units whose bias gradient this CTA sums (thread u: unit u)
-    const int n_bias = dz_is_P ? kRows : (mb == 0 ? NQ : 0);
-    const unsigned char* bias_src = dz_is_P ? sm.A : sm.B;
-    float bsum = 0.f;
-    unsigned mma_phase = 0;
+    const int t0 = split * L.per, t1 = min(a.n_tiles, t0 + L.per);
+    constexpr unsigned kPHalf = kRows * kRows * 2;   // 32 KB: 16 row groups of 2 KB
+    auto issue = [&](int t) {
+        unsigned char* st = sm.stage[(t - t0) & 1];
+        uint64_t* bar = &sm.full[(t - t0) & 1];
+        const unsigned q_bytes = (unsigned)(kRows * NQ * 2);
+        mbar_expect_tx(bar, kPHalf + q_bytes);
+        const unsigned char* p = L.P + (size_t)t * L.p_stride + mb * 2048;
+        for (int g = 0; g < kRows / 8; ++g) tma_load_1d(st + g * 2048, p + g * 4096, 2048, bar);
+        tma_load_1d(st + kPHalf, L.Q + (size_t)t * L.q_stride, q_bytes, bar);
+    };
+    if (tid == 0)
+        for (int t = t0; t < t1 && t < t0 + 2; ++t) issue(t);
+    // the dz operand's units whose bias gradient this CTA sums: warp g takes unit
+    // group g, a lane every 32nd row (16 bytes of it: no bank conflicts)
+    const int n_bias = L.dz_is_P ? kRows : (mb == 0 ? NQ : 0);
+    const bool biased = warp < n_bias / 8;
+    const unsigned bias_at = (L.dz_is_P ? 0u : kPHalf) + warp * 128 + (lane & 7) * 16;
+    const unsigned bias_rg = L.dz_is_P ? 2048u : (unsigned)(NQ / 8) * 128u;
+    float bsum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    unsigned full_phase = 0, mma_phase = 0;   // bit s: parity of stage s
     bool failed = false, mma_pending = false;
-    const int nA = 16 * 16, nB = 16 * (NQ / 8);
-    for (int t = t0; t < t1 && !failed; ++t) {
-        const unsigned char* Pt = P + (size_t)t * p_stride;
-        const unsigned char* Qt = Q + (size_t)t * q_stride;
-        // core matrix c: row group gs (8 rows) of unit group gu, transposed;
-        // each warp first issues the loads of kBatch core matrices, so that
-        // many are in flight, then transposes and stores them
-        constexpr int kBatch = 8, kWarps = kThreads / 32;
-        const int off = (lane >> 2) * 16 + (lane & 3) * 4;
-        for (int c0 = warp; c0 < nA + nB; c0 += kBatch * kWarps) {
-            unsigned w[kBatch];
-            unsigned char* dst[kBatch];
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) {
-                const int c = c0 + u * kWarps;
-                dst[u] = nullptr;
-                if (c < nA + nB) {
-                    const bool isA = c < nA;
-                    const int cc = isA ? c : c - nA, gs = cc & 15, gu = cc >> 4;
-                    const unsigned char* src = isA ? Pt + gs * (KP / 8) * 128 + (mb * 16 + gu) * 128
-                                                   : Qt + gs * (NQ / 8) * 128 + gu * 128;
-                    dst[u] = (isA ? sm.A : sm.B) + gu * 2048 + gs * 128 + off;
-                    w[u] = __ldg(reinterpret_cast<const unsigned*>(src + off));
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u)
-                if (c0 + u * kWarps < nA + nB)   // warp-uniform: movmatrix needs the whole warp
-                    *reinterpret_cast<unsigned*>(dst[u]) = transpose8x8(w[u]);
+    int t = t0;
+    for (; t < t1 && !failed; ++t) {
+        const int s = (t - t0) & 1;
+        unsigned char* st = sm.stage[s];
+        unsigned spins = 0;
+        bool ok = true;
+        while (!(ok = mbar_try_wait(&sm.full[s], (full_phase >> s) & 1u)) && ++spins < kWaitLimit) {
         }
-        fence_async_shared();
-        tc_fence_before();
-        __syncthreads();
+        if (__syncthreads_or(!ok)) { failed = true; break; }   // the copies stay pending
+        full_phase ^= 1u << s;
         if (tid == 0) {
-            tc_fence_after();
-            const uint32_t idesc = idesc_bf16(kRows, NQ);
+            const uint32_t idesc = idesc_bf16_mn(kRows, NQ);
+            const unsigned q_rg = (unsigned)(NQ / 8) * 128u;   // bytes per row group of Q
             for (int kk = 0; kk < kRows / 16; ++kk)
-                mma_bf16(tmem, smem_desc(sm.A + kk * 256, 128, 2048),
-                         smem_desc(sm.B + kk * 256, 128, 2048), idesc, (t > t0 || kk > 0) ? 1u : 0u);
+                mma_bf16(tmem, smem_desc(st + kk * 4096, 2048, 128),
+                         smem_desc(st + kPHalf + kk * 2 * q_rg, q_rg, 128), idesc, (t > t0 || kk > 0) ? 1u : 0u);
             mma_commit(&sm.mma_bar);
         }
         mma_pending = true;
-        if (tid < n_bias) {   // bias gradient: this unit's row of the operand, rows in order
-            const unsigned char* rowp = bias_src + (tid >> 3) * 2048 + (tid & 7) * 16;
-            for (int g = 0; g < kRows / 8; ++g) {
-                const uint4 q = *reinterpret_cast<const uint4*>(rowp + g * 128);
-                const unsigned w[4] = {q.x, q.y, q.z, q.w};
+        if (biased) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) bsum += bf_lo(w[e]) + bf_hi(w[e]);
+            for (int q = 0; q < 4; ++q) {
+                const uint4 w = *reinterpret_cast<const uint4*>(st + bias_at + (4 * q + (lane >> 3)) * bias_rg);
+                const unsigned e[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    bsum[2 * u] += bf_lo(e[u]);
+                    bsum[2 * u + 1] += bf_hi(e[u]);
+                }
             }
         }
-        unsigned spins = 0;
-        bool ok = true;
+        spins = 0;
         while (!(ok = mbar_try_wait(&sm.mma_bar, mma_phase)) && ++spins < kWaitLimit) {
         }
         if (__syncthreads_or(!ok)) { failed = true; break; }   // the MMA stays pending
         mma_phase ^= 1u;
         mma_pending = false;
-        tc_fence_after();
+        if (tid == 0 && t + 2 < t1) {
+            fence_async_shared();
+            issue(t + 2);
+        }
     }
+    tc_fence_after();
     if (!failed) {
         // epilogue: TMEM lane = unit of P (row of D), column = unit of Q
         const int quarter = warp & 3, cpart = warp >> 2, row = quarter * 32 + lane;
         const unsigned lane_base = tmem + ((unsigned)(quarter * 32) << 16);
-        float* out = part + ((size_t)split * gridDim.x * kRows + mb * kRows + row) * NQ;
-        if (NQ >= 128) {
-            for (int c0 = cpart * (NQ / 4); c0 < (cpart + 1) * (NQ / 4); c0 += 32) {
+        float* out = a.part + L.part + ((size_t)(split * 2 + mb) * kRows + row) * NQ;
+        if (NQ == kHidden) {
+            for (int c0 = cpart * (kHidden / 4); c0 < (cpart + 1) * (kHidden / 4); c0 += 32) {
                 float v[32];
                 tmem_ld32(lane_base + c0, v);
 #pragma unroll
@@ -474,23 +500,40 @@ mlp_dw_tc_kernel(const unsigned char* __restrict__ P, int KP, size_t p_stride,
                     reinterpret_cast<float4*>(out + c0)[q] =
                         make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
             }
-        } else if (cpart == 0 && NQ == 32) {
+        } else if (cpart == 0 && NQ == kIn) {
             float v[32];
             tmem_ld32(lane_base, v);
 #pragma unroll
             for (int q = 0; q < 8; ++q)
                 reinterpret_cast<float4*>(out)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-        } else if (cpart == 0) {   // NQ == 16
+        } else if (cpart == 0) {   // NQ == kOut
             float v[16];
             tmem_ld16(lane_base, v);
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 reinterpret_cast<float4*>(out)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         }
-        if (tid < n_bias) dbp[(size_t)split * kHidden + (dz_is_P ? mb * kRows : 0) + tid] = bsum;
+        if (biased) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) bsum[u] += __shfl_xor_sync(~0u, bsum[u], o);
+                if (lane == 0)
+                    a.part[L.bias + (size_t)split * kHidden + (L.dz_is_P ? mb * kRows : 0) + warp * 8 + u] = bsum[u];
+            }
+        }
     }
     if (failed && tid == 0) {
-        atomicOr(err, 2);
+        atomicOr(a.err, 2);
+        // a last bounded wait for the copies and the MMA still in flight
+        for (int q = 0; q < 2; ++q)
+            if (t + q < t1) {
+                const int s = (t + q - t0) & 1;
+                const bool waited = q == 0 && mma_pending;   // this tile's copies have landed
+                if (!waited)
+                    for (unsigned w = 0; w < kWaitLimit && !mbar_try_wait(&sm.full[s], (full_phase >> s) & 1u); ++w) {
+                    }
+            }
         if (mma_pending)
             for (unsigned w = 0; w < kWaitLimit && !mbar_try_wait(&sm.mma_bar, mma_phase); ++w) {
             }
@@ -500,24 +543,29 @@ mlp_dw_tc_kernel(const unsigned char* __restrict__ P, int KP, size_t p_stride,
     if (warp == 0) tmem_dealloc(tmem, cols);
 }
 
-// dW (real sizes out_r x in_r, added to) and db (out_r, added to) from the
-// splits' partials, summed in split order.  part: [split][M][NQ] with
-// M = units of P; transpose: P holds the layer's inputs (D = dW^T).
-__global__ void mlp_dw_reduce_kernel(const float* __restrict__ part, const float* __restrict__ dbp,
-                                     int splits, int M, int NQ, int transpose, int out_r, int in_r,
-                                     float* __restrict__ dW, float* __restrict__ db) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < M * NQ) {
+// dW and db of every layer from the splits' partials, summed in split order.
+// part: [split][256 units of P][NQ]; where P holds the layer's inputs, D = dW^T.
+__global__ void __launch_bounds__(256) mlp_dw_reduce_kernel(const DwArgs a) {
+    const int e = blockIdx.x * 256 + threadIdx.x;
+    int li = 0;
+#pragma unroll
+    for (int q = 1; q < kLayers; ++q)
+        if (e >= a.l[q].e0) li = q;
+    const DwLayer& L = a.l[li];
+    const int r = e - L.e0, n = kHidden * L.NQ;
+    if (r < n) {
+        const float* p = a.part + L.part + r;
         float s = 0.f;
-        for (int q = 0; q < splits; ++q) s += part[(size_t)q * M * NQ + e];
-        const int m = e / NQ, n = e % NQ;
-        const int o = transpose ? n : m, i = transpose ? m : n;
-        if (o < out_r && i < in_r) dW[(size_t)o * in_r + i] += s;
+#pragma unroll 8
+        for (int q = 0; q < L.splits; ++q) s += p[(size_t)q * n];
+        const int m = r / L.NQ, u = r % L.NQ;
+        const int o = L.dz_is_P ? m : u, i = L.dz_is_P ? u : m;
+        if (o < L.out_r && i < L.in_r) a.grad[L.w + (size_t)o * L.in_r + i] = s;
     }
-    if (e < out_r) {
+    if (r < L.out_r) {
         float s = 0.f;
-        for (int q = 0; q < splits; ++q) s += dbp[(size_t)q * kHidden + e];
-        db[e] += s;
+        for (int q = 0; q < L.splits; ++q) s += a.part[L.bias + (size_t)q * kHidden + r];
+        a.grad[L.w + (size_t)L.out_r * L.in_r + r] = s;
     }
 }
 
@@ -565,19 +613,18 @@ cudaError_t forward(const float* x, int rows, int in_dim, int out_dim, const uns
                     unsigned char* saved, unsigned char* zsave, int tile_base, int tile_cap,
                     int* err, int sm_count, cudaStream_t st) {
     const int n_tiles = (rows + kRows - 1) / kRows;
-    unsigned char* xt = x_tiled + (size_t)tile_base * kInBytes;
-    const int total = n_tiles * kRows * kIn;
-    pack_input_kernel<<<(total + 255) / 256, 256, 0, st>>>(x, rows, in_dim, xt, n_tiles);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     const size_t smem = fwd_smem_bytes();
-    e = cudaFuncSetAttribute(mlp_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(mlp_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
     const int grid = n_tiles < sm_count ? n_tiles : sm_count;
-    mlp_fwd_kernel<<<grid, kThreads, smem, st>>>(xt, n_tiles, w_tiled, bias, ypad, rows, saved,
-                                                 zsave, tile_base, tile_cap, err);
+    // a y that shares storage with x is written after every row of x has been read
+    const bool overlap = x < y + (size_t)rows * out_dim && y < x + (size_t)rows * in_dim;
+    mlp_fwd_kernel<<<grid, kThreads, smem, st>>>(x, in_dim, x_tiled, n_tiles, w_tiled, bias,
+                                                 overlap ? ypad : y, overlap ? kOut : out_dim, out_dim,
+                                                 rows, saved, zsave, tile_base, tile_cap, err);
     e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || !overlap) return e;
     unpack_output_kernel<<<(rows * out_dim + 255) / 256, 256, 0, st>>>(ypad, rows, out_dim, y);
     return cudaGetLastError();
 }
@@ -597,7 +644,9 @@ cudaError_t backward(const float* dy, int rows, int in_dim, int out_dim,
     return cudaGetLastError();
 }
 
-size_t dw_part_floats() { return (size_t)kDwMaxSplits * (kHidden * kHidden + kHidden); }
+size_t dw_part_floats() {   // a layer: 256 x NQ and 256 bias sums per split
+    return (size_t)kDwMaxSplits * kHidden * (2 * kHidden + kIn + kOut + kLayers);
+}
 
 cudaError_t weight_grads(const unsigned char* x_tiled, const unsigned char* saved,
                          const unsigned char* dzsave, int tile_base, int tile_cap, int rows,
@@ -605,39 +654,56 @@ cudaError_t weight_grads(const unsigned char* x_tiled, const unsigned char* save
                          cudaStream_t st) {
     const int n_tiles = (rows + kRows - 1) / kRows;
     const size_t smem = sizeof(DwSmem) + 1024;
-    cudaError_t e = cudaFuncSetAttribute(mlp_dw_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(mlp_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    float* dbp = part + (size_t)kDwMaxSplits * kHidden * kHidden;
-    for (int l = 0; l < kLayers; ++l) {
-        const int in_r = l == 0 ? in_dim : kHidden, out_r = l == 3 ? out_dim : kHidden;
-        const unsigned char* a = l == 0 ? x_tiled + (size_t)tile_base * kInBytes
-                                        : saved + ((size_t)l * tile_cap + tile_base) * kActBytes;
-        const size_t a_stride = l == 0 ? kInBytes : kActBytes;
+    DwArgs a{};
+    a.n_tiles = n_tiles;
+    a.part = part;
+    a.grad = grad;
+    a.err = err;
+    // one CTA per SM in all, the splits by a tile's bytes: 27 and 11 of the
+    // hidden and the outer layers on 152 SMs (two halves of P each)
+    const int order[kLayers] = {1, 2, 0, 3};   // the longest CTAs first
+    size_t at = 0;
+    int cta = 0, elem = 0;
+    for (int q = 0; q < kLayers; ++q) {
+        const int l = order[q];
+        DwLayer& L = a.l[q];
+        const unsigned char* act = l == 0 ? x_tiled + (size_t)tile_base * kInBytes
+                                          : saved + ((size_t)l * tile_cap + tile_base) * kActBytes;
+        const size_t act_stride = l == 0 ? kInBytes : kActBytes;
         const unsigned char* dz = dzsave + ((size_t)l * tile_cap + tile_base) * kActBytes;
-        // P: the operand of 256 units (M in 128-unit blocks); Q: the other one
+        // P: the operand of 256 units; Q: the other one
         const bool dz_is_P = layer_n(l) == kHidden;
-        const unsigned char* P = dz_is_P ? dz : a;
-        const unsigned char* Q = dz_is_P ? a : dz;
-        const int KP = dz_is_P ? layer_n(l) : layer_k(l), NQ = dz_is_P ? layer_k(l) : layer_n(l);
-        const size_t p_stride = dz_is_P ? kActBytes : a_stride, q_stride = dz_is_P ? a_stride : kActBytes;
-        const int mblocks = KP / kRows;
-        int splits = sm_count / mblocks;
+        L.P = dz_is_P ? dz : act;
+        L.Q = dz_is_P ? act : dz;
+        L.p_stride = dz_is_P ? kActBytes : act_stride;
+        L.q_stride = dz_is_P ? act_stride : kActBytes;
+        L.NQ = dz_is_P ? layer_k(l) : layer_n(l);
+        L.dz_is_P = dz_is_P ? 1 : 0;
+        int splits = L.NQ == kHidden ? sm_count * 27 / 152 : sm_count * 11 / 152;
         splits = splits < 1 ? 1 : splits > kDwMaxSplits ? kDwMaxSplits : splits;
         splits = splits > n_tiles ? n_tiles : splits;
-        const int per = (n_tiles + splits - 1) / splits;
-        splits = (n_tiles + per - 1) / per;
-        mlp_dw_tc_kernel<<<dim3(mblocks, splits), kThreads, smem, st>>>(
-            P, KP, p_stride, Q, NQ, q_stride, n_tiles, per, part, dbp, dz_is_P ? 1 : 0, err);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        float* dW = grad + param_offset(l, in_dim, out_dim);
-        mlp_dw_reduce_kernel<<<(KP * NQ + 255) / 256, 256, 0, st>>>(
-            part, dbp, splits, KP, NQ, dz_is_P ? 0 : 1, out_r, in_r, dW, dW + (size_t)out_r * in_r);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        L.per = (n_tiles + splits - 1) / splits;
+        L.splits = (n_tiles + L.per - 1) / L.per;
+        L.part = at;
+        at += (size_t)L.splits * kHidden * L.NQ;
+        L.bias = at;
+        at += (size_t)L.splits * kHidden;
+        L.in_r = l == 0 ? in_dim : kHidden;
+        L.out_r = l == 3 ? out_dim : kHidden;
+        L.w = param_offset(l, in_dim, out_dim);
+        L.cta0 = cta;
+        cta += 2 * L.splits;
+        L.e0 = elem;
+        elem += kHidden * L.NQ;
     }
-    return cudaSuccess;
+    mlp_dw_kernel<<<cta, kThreads, smem, st>>>(a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    mlp_dw_reduce_kernel<<<(elem + 255) / 256, 256, 0, st>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t mse(const float* y, const float* t, int n, float* dy, float* loss, cudaStream_t st) {
@@ -800,7 +866,6 @@ extern "C" stamp_status stamp_mlp_backward(stamp_mlp* m, const float* dy, int ro
                                  tile_base, m->tile_cap, dx, m->err, m->sm_count, m->stream),
             "MLP backward launch failed");
     if (dparams) {
-        MLP_TRY(cudaMemsetAsync(dparams, 0, m->n_params * 4, m->stream), "memset failed");
         MLP_TRY(stamp::mlp::weight_grads(m->x_tiled, m->saved, m->dzsave, tile_base, m->tile_cap,
                                          rows, m->in_dim, m->out_dim, dparams, m->dw_part, m->err,
                                          m->sm_count, m->stream),
@@ -832,7 +897,6 @@ extern "C" stamp_status stamp_mlp_train(stamp_mlp* m, float* params, const float
             MLP_TRY(stamp::mlp::backward(m->dy, batch, m->in_dim, m->out_dim, m->wt_tiled, m->zsave,
                                          m->dzsave, 0, m->tile_cap, nullptr, m->err, m->sm_count,
                                          m->stream), "MLP backward launch failed");
-            MLP_TRY(cudaMemsetAsync(m->grad, 0, m->n_params * 4, m->stream), "memset failed");
             MLP_TRY(stamp::mlp::weight_grads(m->x_tiled, m->saved, m->dzsave, 0, m->tile_cap, batch,
                                              m->in_dim, m->out_dim, m->grad, m->dw_part, m->err,
                                              m->sm_count, m->stream),

@@ -39,9 +39,9 @@ size_t fwd_smem_bytes();
 // input-gradient backward (W_l^T: N = in, K = out), plus FP32 biases.
 cudaError_t pack_weights(const float* params, int in_dim, int out_dim, unsigned char* w_tiled,
                          unsigned char* wt_tiled, float* bias, cudaStream_t st);
-// y (rows x out_dim FP32) = MLP(x (rows x in_dim FP32)).  x_tiled: input
-// tiles (8 KB each, written at tile_base); ypad: rows x 16 FP32 scratch.
-// saved / zsave (NULL or buffers of tile_cap 64 KB tiles per layer) receive
+// y (rows x out_dim FP32) = MLP(x (rows x in_dim FP32)).  ypad: rows x 16 FP32
+// scratch, for a y that overlaps x.  saved / zsave (NULL or buffers of tile_cap
+// 64 KB tiles per layer) and x_tiled (8 KB tiles, written with saved) receive
 // the activations for the backward pass at tiles tile_base...
 cudaError_t forward(const float* x, int rows, int in_dim, int out_dim, const unsigned char* w_tiled,
                     const float* bias, unsigned char* x_tiled, float* ypad, float* y,
@@ -53,7 +53,7 @@ cudaError_t backward(const float* dy, int rows, int in_dim, int out_dim,
                      const unsigned char* wt_tiled, const unsigned char* zsave,
                      unsigned char* dzsave, int tile_base, int tile_cap, float* dx, int* err,
                      int sm_count, cudaStream_t st);
-// grad (packed like the parameters) += dL/dW_l, dL/db_l, on the tensor
+// grad (packed like the parameters) = dL/dW_l, dL/db_l, on the tensor
 // cores (BF16 operands, FP32 accumulation in TMEM), reduced over row splits
 // in a fixed order; part: dw_part_floats() floats of scratch; err: bit 2 if
 // a bounded wait gave up.
