@@ -47,6 +47,35 @@ __device__ __forceinline__ void tma_load_1d(void* dst, const void* src, unsigned
 __device__ __forceinline__ void fence_async_shared() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
+// ---------------- thread-block clusters ------------------------------------
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// barrier initialisations visible to the cluster's other CTAs (before cluster_sync)
+__device__ __forceinline__ void fence_mbar_init() {
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync() {   // every thread of every CTA of the cluster
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// CTA `rank`'s address of what lies at shared address `addr` here
+__device__ __forceinline__ unsigned peer_addr(unsigned addr, unsigned rank) {
+    unsigned d;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
+    return d;
+}
+// Shared memory to the same place of CTA `rank`, completing on that CTA's copy of
+// `bar`; address and bytes must be multiples of 16
+__device__ __forceinline__ void bulk_to_peer(void* p, unsigned bytes, uint64_t* bar, unsigned rank) {
+    const unsigned src = smem_u32(p);
+    asm volatile(
+        "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+        ::"r"(peer_addr(src, rank)), "r"(src), "r"(bytes), "r"(peer_addr(smem_u32(bar), rank))
+        : "memory");
+}
 constexpr unsigned kWaitLimit = 1u << 22;   // try_wait polls before a wait gives up
 
 }  // namespace async

@@ -95,10 +95,7 @@ mlp_fwd_kernel(const float* __restrict__ x, int in_dim, unsigned char* __restric
             tma_pending = false;
             if (tid == 0) {
                 tc_fence_after();
-                const uint32_t idesc = idesc_bf16(kRows, N);
-                for (int kk = 0; kk < K / 16; ++kk)
-                    mma_bf16(tmem, smem_desc(sm.act + kk * 256, 128, (K / 8) * 128),
-                             smem_desc(sm.w + kk * 256, 128, (K / 8) * 128), idesc, kk > 0);
+                mma_tile(tmem, sm.act, sm.w, K, N);
                 mma_commit(&sm.mma_bar);
             }
             mma_pending = true;
@@ -284,10 +281,7 @@ mlp_bwd_kernel(const float* __restrict__ dy, int rows, int out_dim, int n_tiles,
             tma_pending = false;
             if (tid == 0) {
                 tc_fence_after();
-                const uint32_t idesc = idesc_bf16(kRows, Nb);
-                for (int kk = 0; kk < Kb / 16; ++kk)
-                    mma_bf16(tmem, smem_desc(sm.act + kk * 256, 128, (Kb / 8) * 128),
-                             smem_desc(sm.w + kk * 256, 128, (Kb / 8) * 128), idesc, kk > 0);
+                mma_tile(tmem, sm.act, sm.w, Kb, Nb);
                 mma_commit(&sm.mma_bar);
             }
             mma_pending = true;

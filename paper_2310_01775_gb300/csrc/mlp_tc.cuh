@@ -95,6 +95,18 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+__device__ __forceinline__ void tmem_ld8(unsigned taddr, float (&v)[8]) {
+    unsigned r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                   "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 __device__ __forceinline__ unsigned pack_bf16(float a, float b) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const unsigned*>(&h);
@@ -109,6 +121,19 @@ __host__ __device__ __forceinline__ unsigned tile_off(int row, int col, int K) {
 }
 
 constexpr int kRows = 128;                        // rows per tile (MMA M)
+
+// D (128 x N) = A (128 x K) . B (N x K)^T, K-major operands; K is 16, 32 or 256.
+// A slice of 16 columns is 256 bytes on in both: 16 in a descriptor's address.
+__device__ __forceinline__ void mma_tile(unsigned tmem, const unsigned char* A, const unsigned char* B,
+                                         int K, int N) {
+    const uint32_t idesc = idesc_bf16(kRows, N);
+    const uint64_t da = smem_desc(A, 128, (K / 8) * 128), db = smem_desc(B, 128, (K / 8) * 128);
+    mma_bf16(tmem, da, db, idesc, 0u);
+    if (K >= 32) mma_bf16(tmem, da + 16, db + 16, idesc, 1u);
+    if (K >= 256)
+#pragma unroll
+        for (int kk = 2; kk < 16; ++kk) mma_bf16(tmem, da + 16 * kk, db + 16 * kk, idesc, 1u);
+}
 // 16 warps: warp w reads TMEM lane quarter w % 4 (rows 32 (w % 4) ...) and
 // takes part w / 4 of the four column parts in the epilogues
 constexpr int kThreads = 512;

@@ -8,8 +8,9 @@
 // not depend on the poses: four warps compute the next push's beside the
 // layer-1 MMA.  What it replaces, per push at 131072 rows on GB300: features
 // 40 us, packing 13.5, MLP 88, unpacking 6; at 2048 rows 8 + 3 + 18 + 3, and
-// the launches between them; six pushes of 131072 rows take 548 us here, of 2048
-// rows 95 (and 97 in reverse, where the 12 launches took 155).
+// the launches between them; six pushes of 131072 rows take 530 us here.  Few
+// plans would leave most SMs idle (2048 rows: 16 tiles, 95 us, and 97 in reverse):
+// they go to the cluster kernels below (33 and 30 us).
 // Reverse, per push: the pose adjoints (in registers) are the head's dy; the
 // input-gradient chain of mlp_bwd_kernel; the features' reverse on the row.
 //
@@ -61,6 +62,34 @@ __device__ __forceinline__ void action_features(const SimConst& sc, const SurArg
     }
 #pragma unroll
     for (int c = 0; c < P; ++c) put_bf16(tile, row, 4 * NB + c, f[c]);
+}
+
+// All pushes' action features of plans i0 ... i0 + rows - 1 to a.relax, by all
+// threads of a cluster: (push, plan) pairs n0, n0 + step, ...
+template <int NB>
+__device__ __forceinline__ void all_action_features(const SimConst& sc, const SurArgs& a, int i0, int rows,
+                                                    uint64_t gkey, int n0, int step) {
+    constexpr int M = rollout::Dims<NB>::M, P = M + 2;
+    for (int n = n0; n < sc.H * rows; n += step) {
+        const int k = n / rows, i = i0 + n % rows;
+        if (i >= a.N) continue;
+        float z[M], uu, vv;
+        rollout::relax_action<NB>(sc, a.theta + (size_t)i * sc.D, k, i, gkey, a.iter >= 0, false, z, uu, vv);
+        float* r = a.relax + ((size_t)i * sc.H + k) * P;
+#pragma unroll
+        for (int c = 0; c < M; ++c) r[c] = z[c];
+        r[M] = tanhf(uu);
+        r[M + 1] = rollout::sigmoidf_(vv);
+    }
+}
+// Push k's, from there, into row `row` of the tile.
+template <int NB>
+__device__ __forceinline__ void stored_features(const SimConst& sc, const SurArgs& a, int i, bool on, int k,
+                                                unsigned char* tile, int row) {
+    constexpr int P = rollout::Dims<NB>::M + 2;
+    const float* r = a.relax + ((size_t)i * sc.H + k) * P;
+#pragma unroll
+    for (int c = 0; c < P; ++c) put_bf16(tile, row, 4 * NB + c, on ? r[c] : 0.f);
 }
 
 template <int NB>
@@ -139,11 +168,7 @@ __global__ void __launch_bounds__(kThreads, 1) sur_fwd_kernel(const SimConst sc,
                 tma_pending = false;
                 if (tid == 0) {
                     tc_fence_after();
-                    const uint32_t idesc = idesc_bf16(kRows, N);
-                    const unsigned char* A = l == 0 ? sm.x : sm.act;
-                    for (int kk = 0; kk < K / 16; ++kk)
-                        mma_bf16(tmem, smem_desc(A + kk * 256, 128, (K / 8) * 128),
-                                 smem_desc(sm.w + kk * 256, 128, (K / 8) * 128), idesc, kk > 0);
+                    mma_tile(tmem, l == 0 ? sm.x : sm.act, sm.w, K, N);
                     mma_commit(&sm.mma_bar);
                 }
                 mma_pending = true;
@@ -232,35 +257,41 @@ __global__ void __launch_bounds__(kThreads, 1) sur_fwd_kernel(const SimConst sc,
 
 // Reverse of one push's features on row i: di = dC/df, the pose adjoint is
 // advanced from q_{k+1} to q_k, and grad log rho of the push's parameters
-// written (with the push-length term).
+// written (with the push-length term).  load() reads what it needs, beside an MMA.
 template <int NB>
-__device__ __forceinline__ void features_reverse(const SimConst& sc, const SurArgs& a, int i, int k,
-                                                 const float* di, float (&ai)[3 * NB]) {
-    constexpr int M = rollout::Dims<NB>::M, P = M + 2;
-    const float* pi = a.pose + ((size_t)k * a.N + i) * 3 * NB;
+struct FeaturesReverse {
+    static constexpr int M = rollout::Dims<NB>::M, P = M + 2;
+    float sn[NB], cs[NB], r[P];
+    __device__ __forceinline__ void load(const SimConst& sc, const SurArgs& a, int i, int k) {
+        const float* pi = a.pose + ((size_t)k * a.N + i) * 3 * NB;
+        const float* ri = a.relax + ((size_t)i * sc.H + k) * P;
 #pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        float sn, cs;
-        sincosf(pi[3 * b + 2], &sn, &cs);
-        ai[3 * b] += di[4 * b];
-        ai[3 * b + 1] += di[4 * b + 1];
-        ai[3 * b + 2] += cs * di[4 * b + 3] - sn * di[4 * b + 2];
+        for (int c = 0; c < P; ++c) r[c] = ri[c];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) sincosf(pi[3 * b + 2], &sn[b], &cs[b]);
     }
-    const float* ri = a.relax + ((size_t)i * sc.H + k) * P;
-    float r[P], zg = 0.f;
+    __device__ __forceinline__ void apply(const SimConst& sc, const SurArgs& a, int i, int k, const float* di,
+                                          float (&ai)[3 * NB], bool store) const {
 #pragma unroll
-    for (int c = 0; c < P; ++c) r[c] = ri[c];
+        for (int b = 0; b < NB; ++b) {
+            ai[3 * b] += di[4 * b];
+            ai[3 * b + 1] += di[4 * b + 1];
+            ai[3 * b + 2] += cs[b] * di[4 * b + 3] - sn[b] * di[4 * b + 2];
+        }
+        if (!store) return;
+        float zg = 0.f;
 #pragma unroll
-    for (int c = 0; c < M; ++c) zg += r[c] * di[4 * NB + c];
-    float* gi = a.grad + (size_t)i * sc.D + k * P;
-    // softmax((a+g)/tau): dC/da_j = z_j (dC/dz_j - sum_c z_c dC/dz_c) / tau
+        for (int c = 0; c < M; ++c) zg += r[c] * di[4 * NB + c];
+        float* gi = a.grad + (size_t)i * sc.D + k * P;
+        // softmax((a+g)/tau): dC/da_j = z_j (dC/dz_j - sum_c z_c dC/dz_c) / tau
 #pragma unroll
-    for (int c = 0; c < M; ++c) gi[c] = -(r[c] * (di[4 * NB + c] - zg) * sc.inv_tau);
-    const float tu = r[M], sv = r[M + 1];
-    gi[M] = -(di[4 * NB + M] * (1.f - tu * tu));
-    const float dist = sc.dist_max * sv;
-    gi[M + 1] = -((di[4 * NB + M + 1] + 2.f * sc.w_push * dist * sc.dist_max) * sv * (1.f - sv));
-}
+        for (int c = 0; c < M; ++c) gi[c] = -(r[c] * (di[4 * NB + c] - zg) * sc.inv_tau);
+        const float tu = r[M], sv = r[M + 1];
+        gi[M] = -(di[4 * NB + M] * (1.f - tu * tu));
+        const float dist = sc.dist_max * sv;
+        gi[M + 1] = -((di[4 * NB + M + 1] + 2.f * sc.w_push * dist * sc.dist_max) * sv * (1.f - sv));
+    }
+};
 
 template <int NB>
 __global__ void __launch_bounds__(kThreads, 1) sur_bwd_kernel(const SimConst sc, const SurArgs a) {
@@ -325,10 +356,7 @@ __global__ void __launch_bounds__(kThreads, 1) sur_bwd_kernel(const SimConst sc,
                 tma_pending = false;
                 if (tid == 0) {
                     tc_fence_after();
-                    const uint32_t idesc = idesc_bf16(kRows, Nb);
-                    for (int kk = 0; kk < Kb / 16; ++kk)
-                        mma_bf16(tmem, smem_desc(sm.act + kk * 256, 128, (Kb / 8) * 128),
-                                 smem_desc(sm.w + kk * 256, 128, (Kb / 8) * 128), idesc, kk > 0);
+                    mma_tile(tmem, sm.act, sm.w, Kb, Nb);
                     mma_commit(&sm.mma_bar);
                 }
                 mma_pending = true;
@@ -368,7 +396,11 @@ __global__ void __launch_bounds__(kThreads, 1) sur_bwd_kernel(const SimConst sc,
                 } else if (part == 0) {
                     float v[32];
                     tmem_ld32(lane_base, v);
-                    if (on) features_reverse<NB>(sc, a, i, k, v, ap);
+                    if (on) {
+                        FeaturesReverse<NB> f;
+                        f.load(sc, a, i, k);
+                        f.apply(sc, a, i, k, v, ap, true);
+                    }
                 }
                 fence_async_shared();
                 tc_fence_before();
@@ -389,8 +421,346 @@ __global__ void __launch_bounds__(kThreads, 1) sur_bwd_kernel(const SimConst sc,
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
+// Few plans: two CTAs of a cluster take TR (32 or 64) rows, so that 2048 rows use
+// 128 SMs where 128-row tiles use 16, and the weights stay in shared memory.
+// The roles of the operands are swapped: M = 128 of a hidden layer's units per
+// CTA, N = the rows, so a narrow N costs less and nothing is computed for
+// padding.  A hidden output is stored as the N-major operand it comes out as
+// (TMEM lane = unit, column = row: a thread holds 8 rows of a unit, 16 bytes of
+// an 8 x 8 core matrix; row groups 128 B apart, unit groups TR * 16 B): the CTA's
+// 128 units are contiguous and go to the peer by bulk copies between the shared
+// memories that complete on the receiver's barrier.  The head (and the reverse's
+// input gradient) takes the rows as M instead, a thread per row; both CTAs
+// compute it, the poses and the features, so nothing else is exchanged.  Two
+// output buffers in turn: who has the peer's half of an output knows that the
+// peer has read the one before, which is what the next write replaces.
+template <int TR>
+struct SurClSmem {
+    alignas(128) unsigned char act[2][kHidden * TR * 2];
+    alignas(128) unsigned char x[TR * kIn * 2];             // features, or dz_3: K-major
+    alignas(128) unsigned char w_in[kIn * kHidden * 2];     // forward: half of layer 0; reverse: W_0^T
+    alignas(128) unsigned char w_out[kOut * kHidden * 2];   // forward: the head; reverse: half of W_3^T
+    alignas(128) unsigned char w_mid[2][kHidden / 2 * kHidden * 2];
+    uint64_t w_bar, mma_bar, in_bar[2];
+    unsigned tmem_slot;
+};
+constexpr int kUnits = kHidden / 2;   // of a CTA
+constexpr unsigned kClCols = 64;
+
+// One CTA's side of the cluster.
+template <int TR>
+struct ClusterSide {
+    static constexpr int kGroups = TR / 8 / kParts;          // row groups of a thread
+    static constexpr unsigned kUnitGroup = TR / 8 * 128;     // bytes of 8 units
+    static constexpr unsigned kHalf = kUnits / 8 * kUnitGroup;
+    SurClSmem<TR>& sm;
+    const unsigned rank = async::cluster_rank();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // hidden layers: unit `unit` of this CTA, row groups part * kGroups ...
+    const int quarter = warp & 3, part = warp >> 2, unit = quarter * 32 + lane;
+    unsigned tmem = 0, out = 0, mma_phase = 0;   // out: hidden outputs so far
+    bool w_ready = false, in_pending = false, mma_pending = false;
+
+    __device__ explicit ClusterSide(SurClSmem<TR>& s) : sm(s) {
+        if (tid == 0) {
+            mbar_init(&sm.w_bar, 1);
+            mbar_init(&sm.mma_bar, 1);
+            mbar_init(&sm.in_bar[0], 1);
+            mbar_init(&sm.in_bar[1], 1);
+            async::fence_mbar_init();
+            fence_async_shared();
+        }
+        if (warp == 0) tmem_alloc(&sm.tmem_slot, kClCols);
+        // the features' unused columns stay zero, and so do the rows past TR that the
+        // row-major products read (their results are not used)
+        for (int t = tid * 16; t < (int)(sizeof sm.act + sizeof sm.x); t += kThreads * 16)
+            *reinterpret_cast<uint4*>(sm.act[0] + t) = make_uint4(0, 0, 0, 0);
+        tc_fence_before();
+        async::cluster_sync();
+        tc_fence_after();
+        tmem = sm.tmem_slot;
+    }
+    __device__ unsigned lane_base() const { return tmem + ((unsigned)(quarter * 32) << 16); }
+    __device__ static bool wait(uint64_t* bar, unsigned parity) {
+        for (unsigned w = 0; w < kWaitLimit; ++w)
+            if (mbar_try_wait(bar, parity)) return true;
+        return false;
+    }
+    // units x rows: W (128 units, K-major) times x (K columns) or the last output.
+    // rows x N: the last output times W (N units, K-major), when rows_first.
+    // False (in every thread): a wait gave up.
+    __device__ bool multiply(const unsigned char* W, int from_x_columns, int rows_first_units) {
+        bool ok = w_ready || wait(&sm.w_bar, 0);
+        if (!from_x_columns) ok = ok && wait(&sm.in_bar[(out - 1) & 1], ((out - 1) >> 1) & 1);
+        if (__syncthreads_or(!ok)) return false;   // the copies stay pending
+        w_ready = true;
+        in_pending = false;
+        if (tid == 0) {
+            tc_fence_after();
+            if (from_x_columns) {
+                mma_tile(tmem, W, sm.x, from_x_columns, TR);
+            } else {
+                const uint64_t dw = smem_desc(W, 128, (kHidden / 8) * 128);
+                const uint64_t da = smem_desc(sm.act[(out - 1) & 1], kUnitGroup, 128);
+                if (rows_first_units) {
+                    const uint32_t idesc = idesc_bf16(kRows, rows_first_units) | (1u << 15);   // A: M-major
+#pragma unroll
+                    for (int kk = 0; kk < kHidden / 16; ++kk)
+                        mma_bf16(tmem, da + kk * (2 * kUnitGroup >> 4), dw + kk * 16, idesc, kk > 0);
+                } else {
+                    const uint32_t idesc = idesc_bf16(kRows, TR) | (1u << 16);   // B: N-major
+#pragma unroll
+                    for (int kk = 0; kk < kHidden / 16; ++kk)
+                        mma_bf16(tmem, dw + kk * 16, da + kk * (2 * kUnitGroup >> 4), idesc, kk > 0);
+                }
+            }
+            mma_commit(&sm.mma_bar);
+        }
+        mma_pending = true;
+        return true;
+    }
+    __device__ bool product_done() {
+        const bool ok = wait(&sm.mma_bar, mma_phase);
+        if (__syncthreads_or(!ok)) return false;   // the MMA stays pending
+        mma_phase ^= 1u;
+        mma_pending = false;
+        tc_fence_after();
+        return true;
+    }
+    // this thread's rows of its unit, from the product
+    __device__ void read(float (&v)[8 * kGroups]) const {
+        if constexpr (kGroups == 1) tmem_ld8(lane_base() + part * 8, v);
+        else tmem_ld16(lane_base() + part * 16, v);
+    }
+    // before this layer's epilogue: the bytes that the peer will send; where this thread writes
+    __device__ unsigned char* begin_output() {
+        if (tid == 0) mbar_expect_tx(&sm.in_bar[out & 1], kHalf);
+        in_pending = true;
+        return sm.act[out & 1] + rank * kHalf + (unit >> 3) * kUnitGroup + part * kGroups * 128 + (unit & 7) * 16;
+    }
+    // after it: the four warps of 32 units are done, and one thread sends these to the peer
+    __device__ void send_output() {
+        fence_async_shared();
+        tc_fence_before();
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + quarter) : "memory");
+        if (part == 0 && lane == 0)
+            async::bulk_to_peer(sm.act[out & 1] + rank * kHalf + quarter * 4 * kUnitGroup, 4 * kUnitGroup,
+                                &sm.in_bar[out & 1], rank ^ 1u);
+        ++out;
+    }
+    // pre-activations of layer l, push k: 16 bytes for 8 rows of a unit
+    __device__ unsigned char* z_slot(const SurArgs& a, int l, int k, int tile) const {
+        return a.zsave + ((size_t)l * a.tile_cap + (size_t)k * a.n_tiles) * kActBytes +
+               (size_t)tile * (kHidden * TR * 2) + ((size_t)(part * kGroups) * kHidden + rank * kUnits + unit) * 16;
+    }
+    __device__ void finish(bool failed, int* err) {
+        if (failed && tid == 0) {
+            atomicOr(err, 2);
+            // a last bounded wait for what is still in flight before the memory is given up
+            if (!w_ready) wait(&sm.w_bar, 0);
+            if (in_pending) wait(&sm.in_bar[(out - 1) & 1], ((out - 1) >> 1) & 1);
+            if (mma_pending) wait(&sm.mma_bar, mma_phase);
+        }
+        async::cluster_sync();   // no CTA leaves while the peer's copy reads or writes its memory
+        if (warp == 0) tmem_dealloc(tmem, kClCols);
+    }
+};
+
+template <int NB, int TR>
+__global__ void __launch_bounds__(kThreads, 1) sur_fwd_cluster_kernel(const SimConst sc, const SurArgs a) {
+    constexpr int S3 = 3 * NB, kG = ClusterSide<TR>::kGroups;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    SurClSmem<TR>& sm = *reinterpret_cast<SurClSmem<TR>*>(smem_raw);
+    ClusterSide<TR> s(sm);
+    const int tile = blockIdx.x / 2;
+    // a thread per row: warps 0 .. hold the poses, warps 4 .. fetch the action's features
+    const int row = s.tid % 128, i = tile * TR + row;
+    const bool posed = s.tid < TR, acted = s.tid >= 128 && s.tid < 128 + TR;
+    const bool on = i < a.N, first = s.rank == 0;
+    const uint64_t gkey = a.iter >= 0 ? sm64(sm64(a.seed, kStreamGumbel), (uint64_t)a.iter) : 0ull;
+    if (s.tid == 0) {   // this CTA's units of the weights (K-major: contiguous), the whole head
+        constexpr unsigned w0 = kUnits * kIn * 2, w1 = kUnits * kHidden * 2, w3 = kOut * kHidden * 2;
+        mbar_expect_tx(&sm.w_bar, w0 + 2 * w1 + w3);
+        fence_async_shared();
+        tma_load_1d(sm.w_in, a.w_tiled + layer_w_offset(0) + s.rank * w0, w0, &sm.w_bar);
+        tma_load_1d(sm.w_mid[0], a.w_tiled + layer_w_offset(1) + s.rank * w1, w1, &sm.w_bar);
+        tma_load_1d(sm.w_mid[1], a.w_tiled + layer_w_offset(2) + s.rank * w1, w1, &sm.w_bar);
+        tma_load_1d(sm.w_out, a.w_tiled + layer_w_offset(3), w3, &sm.w_bar);
+    }
+    float bias[3];
+#pragma unroll
+    for (int l = 0; l < 3; ++l) bias[l] = __ldg(a.bias + l * kHidden + s.rank * kUnits + s.unit);
+    float q[S3];
+#pragma unroll
+    for (int t = 0; t < S3; ++t) q[t] = sc.init[t / 3][t % 3];
+    if (posed) {
+        pose_features<NB>(q, on, sm.x, row);
+        if (on && first && (a.zsave || sc.H == 1))
+#pragma unroll
+            for (int t = 0; t < S3; ++t) a.pose[(size_t)i * S3 + t] = q[t];
+    }
+    all_action_features<NB>(sc, a, tile * TR, TR, gkey, s.tid * 2 + s.rank, 2 * kThreads);
+    async::cluster_sync();   // the cluster's stores to a.relax are there
+    if (acted) stored_features<NB>(sc, a, i, on, 0, sm.x, row);
+    fence_async_shared();
+    bool failed = false;
+    for (int k = 0; k < sc.H && !failed; ++k) {
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            if (!s.multiply(l == 0 ? sm.w_in : sm.w_mid[l ? l - 1 : 0], l == 0 ? kIn : 0, 0)) { failed = true; break; }
+            // layer 0 has read the push's features: the next push's, beside this MMA
+            if (l == 1 && acted && k + 1 < sc.H) stored_features<NB>(sc, a, i, on, k + 1, sm.x, row);
+            if (!s.product_done()) { failed = true; break; }
+            unsigned char* dst = s.begin_output();
+            float v[8 * kG];
+            s.read(v);
+#pragma unroll
+            for (int g = 0; g < kG; ++g) {
+                uint4 pk, pz;
+                unsigned* pw = reinterpret_cast<unsigned*>(&pk);
+                unsigned* pzw = reinterpret_cast<unsigned*>(&pz);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float z0 = v[g * 8 + 2 * e] + bias[l], z1 = v[g * 8 + 2 * e + 1] + bias[l];
+                    pw[e] = pack_bf16(silu(z0), silu(z1));
+                    pzw[e] = pack_bf16(z0, z1);
+                }
+                *reinterpret_cast<uint4*>(dst + g * 128) = pk;
+                if (a.zsave)   // pre-activation of layer l, for the reverse sweep
+                    *reinterpret_cast<uint4*>(s.z_slot(a, l, k, tile) + g * kHidden * 16) = pz;
+            }
+            s.send_output();
+        }
+        if (failed || !s.multiply(sm.w_out, 0, kOut) || !s.product_done()) { failed = true; break; }
+        if (posed) {
+            float v[16];
+            tmem_ld16(s.lane_base(), v);
+            const float* bl = a.bias + 3 * kHidden;
+            float d[S3];
+#pragma unroll
+            for (int t = 0; t < S3; ++t) d[t] = v[t] + __ldg(bl + t);
+            if (k + 1 == sc.H) {   // the cost adds the last pose change itself
+                if (on && first)
+#pragma unroll
+                    for (int t = 0; t < S3; ++t) a.y[(size_t)i * S3 + t] = d[t];
+            } else {
+#pragma unroll
+                for (int t = 0; t < S3; ++t) q[t] += d[t];
+                if (on && first && (a.zsave || k + 2 == sc.H))
+#pragma unroll
+                    for (int t = 0; t < S3; ++t) a.pose[((size_t)(k + 1) * a.N + i) * S3 + t] = q[t];
+                pose_features<NB>(q, on, sm.x, row);
+            }
+        }
+        fence_async_shared();
+        tc_fence_before();
+    }
+    s.finish(failed, a.err);
+}
+
+template <int NB, int TR>
+__global__ void __launch_bounds__(kThreads, 1) sur_bwd_cluster_kernel(const SimConst sc, const SurArgs a) {
+    constexpr int S3 = 3 * NB, kG = ClusterSide<TR>::kGroups;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    SurClSmem<TR>& sm = *reinterpret_cast<SurClSmem<TR>*>(smem_raw);
+    ClusterSide<TR> s(sm);
+    const int tile = blockIdx.x / 2, row = s.tid % 128, i = tile * TR + row;
+    const bool posed = s.tid < TR, on = posed && i < a.N;   // a thread per row
+    if (s.tid == 0) {   // this CTA's rows of the transposed weights, all of W_0^T
+        constexpr unsigned w0 = kIn * kHidden * 2, w1 = kUnits * kHidden * 2, w3 = kOut * kUnits * 2;
+        mbar_expect_tx(&sm.w_bar, w0 + 2 * w1 + w3);
+        fence_async_shared();
+        tma_load_1d(sm.w_out, a.wt_tiled + layer_w_offset(3) + s.rank * w3, w3, &sm.w_bar);
+        tma_load_1d(sm.w_mid[1], a.wt_tiled + layer_w_offset(2) + s.rank * w1, w1, &sm.w_bar);
+        tma_load_1d(sm.w_mid[0], a.wt_tiled + layer_w_offset(1) + s.rank * w1, w1, &sm.w_bar);
+        tma_load_1d(sm.w_in, a.wt_tiled + layer_w_offset(0), w0, &sm.w_bar);
+    }
+    float ap[S3];   // dC/dq_{k+1}
+#pragma unroll
+    for (int t = 0; t < S3; ++t) ap[t] = on ? a.apose[(size_t)i * S3 + t] : 0.f;
+    bool failed = false;
+    for (int k = sc.H - 1; k >= 0 && !failed; --k) {
+        if (posed) {   // dz_3 = dy = dC/dq_{k+1}: a BF16 K-major tile of 16 columns
+            float d[kOut];
+#pragma unroll
+            for (int c = 0; c < kOut; ++c) d[c] = c < S3 ? ap[c < S3 ? c : 0] : 0.f;
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                uint4 pk;
+                unsigned* pw = reinterpret_cast<unsigned*>(&pk);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) pw[e] = pack_bf16(d[g * 8 + 2 * e], d[g * 8 + 2 * e + 1]);
+                *reinterpret_cast<uint4*>(sm.x + tile_off(row, g * 8, kOut)) = pk;
+            }
+        }
+        fence_async_shared();
+        FeaturesReverse<NB> f;
+#pragma unroll
+        for (int m = 3; m > 0; --m) {   // da_m = dz_m W_m
+            if (!s.multiply(m == 3 ? sm.w_out : sm.w_mid[m < 3 ? m - 1 : 0], m == 3 ? kOut : 0, 0)) {
+                failed = true;
+                break;
+            }
+            uint4 z[kG];   // beside the MMA
+#pragma unroll
+            for (int g = 0; g < kG; ++g)
+                z[g] = *reinterpret_cast<const uint4*>(s.z_slot(a, m - 1, k, tile) + g * kHidden * 16);
+            if (m == 2 && on) f.load(sc, a, i, k);
+            if (!s.product_done()) { failed = true; break; }
+            unsigned char* dst = s.begin_output();
+            float v[8 * kG];
+            s.read(v);
+#pragma unroll
+            for (int g = 0; g < kG; ++g) {
+                const unsigned zw[4] = {z[g].x, z[g].y, z[g].z, z[g].w};
+                uint4 pk;
+                unsigned* pw = reinterpret_cast<unsigned*>(&pk);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    pw[e] = pack_bf16(v[g * 8 + 2 * e] * silu_grad(bf_lo(zw[e])),
+                                      v[g * 8 + 2 * e + 1] * silu_grad(bf_hi(zw[e])));
+                *reinterpret_cast<uint4*>(dst + g * 128) = pk;
+            }
+            s.send_output();
+        }
+        if (failed || !s.multiply(sm.w_in, 0, kIn) || !s.product_done()) { failed = true; break; }
+        if (posed) {
+            float v[32];
+            tmem_ld32(s.lane_base(), v);
+            if (on) f.apply(sc, a, i, k, v, ap, s.rank == 0);
+        }
+        tc_fence_before();
+    }
+    s.finish(failed, a.err);
+}
+
+template <int NB, int TR>
+cudaError_t launch_cluster(const SimConst& sc, const SurArgs& a, bool reverse, cudaStream_t st) {
+    auto* kernel = reverse ? sur_bwd_cluster_kernel<NB, TR> : sur_fwd_cluster_kernel<NB, TR>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((a.N + TR - 1) / TR * 2);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = sizeof(SurClSmem<TR>);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)cfg.dynamicSmemBytes);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchKernelEx(&cfg, kernel, sc, a);
+}
+
 template <int NB>
 cudaError_t launch(const SimConst& sc, const SurArgs& a, bool reverse, int sms, cudaStream_t st) {
+    // The narrowest tile whose clusters all run at once: its time does not depend on
+    // N (GB300, 6 pushes with the gradient: 78 us on 32 rows, 96 on 64, 181 on
+    // 128-row tiles; a second wave would double it).  The outputs' bits are the same.
+    if (a.N <= sms / 2 * 32) return launch_cluster<NB, 32>(sc, a, reverse, st);
+    if (a.N <= sms / 2 * 64) return launch_cluster<NB, 64>(sc, a, reverse, st);
     const size_t smem = (reverse ? sizeof(FwdSmem) : sizeof(SurSmem)) + 1024;
     auto* kernel = reverse ? sur_bwd_kernel<NB> : sur_fwd_kernel<NB>;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
