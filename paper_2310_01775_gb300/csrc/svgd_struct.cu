@@ -19,7 +19,7 @@
 namespace stamp {
 namespace {
 
-constexpr int kTJ = 16;         // j per tile
+constexpr int kTJ = 32;         // j per tile
 constexpr int kMaxHs = 16;      // actions per plan
 
 // C (N x 2H): (u_k, v_k); S (N x M H): softmax(a_k).
@@ -44,60 +44,47 @@ __global__ void struct_prep_kernel(const float* __restrict__ theta, int N, int H
     C[(size_t)i * 2 * H + 2 * k + 1] = a[M + 1];
 }
 
-// A warp owns kRowsPerWarp rows; lane l owns columns l, l + 32, ... of each.  A
-// tile's grad, theta (its offsets and distances) and softmax rows are staged in
-// shared memory once per CTA; each pair and action costs two exponentials and
-// M multiply-adds there, spread over the CTA's threads, and each pair and
-// column four multiply-adds per lane.  The exponentials' weights (w_j, alpha,
-// 2/h) are folded into what is stored: A_ijk = alpha w_j (2/h) e_ijk.  GB300, N =
-// 1024, H = 4, M = 4: 184 -> 68 us (every lane used to read its j's values from
-// global memory, one row per warp).
-constexpr int kRowsPerWarp = 2, kWarps = 8, kRows = kRowsPerWarp * kWarps;
-__host__ __device__ constexpr size_t struct_smem(int D, int H) {
-    return ((size_t)(2 * kTJ + kRows) * D + (size_t)kRows * kTJ * (3 * H + 1)) * sizeof(float);
-}
-template <int DP>
+// HP lanes (H rounded up to a power of two) own kRows rows of the plan, a lane an
+// action of each: its softmax row, its (u, v) and the accumulators of its M + 2
+// columns stay in registers, a pair's exponentials are computed once, and K is
+// their sum over the lanes.  Tiles of theta's, the softmax's and grad's columns
+// are staged in shared memory, where the lanes of an action read the same
+// address.  What bounds it is arithmetic, about 10 + 7 (M + 2) operations per
+// pair and action; kSplit warps share the rows of a tile's j to keep enough of
+// them in flight, and are summed in order at the end.  GB300, N = 1024, H = 4, M =
+// 4: 68 -> 19.8 us (a lane per column read the pair's exponentials, computed by
+// other threads, from shared memory: five reads per pair and column).
+constexpr int kRows = 2, kSplit = 4, kWarps = 8;
+template <int HP>
+constexpr int kCtaRows = kWarps / kSplit * (32 / HP) * kRows;
+
+template <int M, int HP>
 __global__ void __launch_bounds__(kWarps * 32)
 struct_phi_kernel(const float* __restrict__ theta, const float* __restrict__ grad,
-                  const float* __restrict__ S, int N, int H, int M,
+                  const float* __restrict__ S, int N, int H,
                   const float* __restrict__ hc_dev, const float* __restrict__ hz_dev,
                   const float* __restrict__ wn, float* __restrict__ phi, int j_chunk) {
     extern __shared__ float ssm[];
-    const int P = M + 2, D = H * P;
-    // per column: softmax(a_k) on the logits, theta on (u_k, v_k)
-    float* Xi = ssm;                   // kRows x D
-    float* Xj = Xi + kRows * D;        // kTJ x D
-    float* Gj = Xj + kTJ * D;          // kTJ x D
-    float* Ac = Gj + kTJ * D;          // kRows x kTJ x H: alpha w_j (2/h_c) e^c
-    float* Az = Ac + kRows * kTJ * H;  // alpha w_j (2/h_z) e^z
-    float* Q = Az + kRows * kTJ * H;   // s_j . (s_i - s_j)
-    float* Ks = Q + kRows * kTJ * H;   // kRows x kTJ: w_j K_ij
+    constexpr int P = M + 2, kGroups = 32 / HP;
+    const int D = H * P;
+    float* Xj = ssm;               // kTJ x D: softmax(a_k) on the logits, theta on (u_k, v_k)
+    float* Gj = Xj + kTJ * D;      // kTJ x D
+    float* Wj = Gj + kTJ * D;      // kTJ
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int i0 = blockIdx.x * kRows;
+    const int split = warp % kSplit, k = lane % HP, ks = k < H ? k : 0;
+    const int row0 = (warp / kSplit * kGroups + lane / HP) * kRows, i0 = blockIdx.x * kCtaRows<HP>;
     const float Hf = (float)H;
     const float inv_hc = Hf / __ldg(hc_dev), inv_hz = Hf / __ldg(hz_dev);   // h = h_plain / H
     const float alpha = 0.5f / Hf, ac = alpha * (2.f * inv_hc), az = alpha * (2.f * inv_hz);
-    auto column = [&](int i, int d) {   // X of particle i
-        const int k = d / P, c = d - k * P;
-        return c < M ? S[(size_t)i * M * H + k * M + c] : theta[(size_t)i * D + d];
-    };
-    for (int t = tid; t < kRows * D; t += kWarps * 32) {
-        const int r = t / D, d = t % D;
-        Xi[t] = i0 + r < N ? column(i0 + r, d) : 0.f;
-    }
-    float xi[kRowsPerWarp][DP], acc[kRowsPerWarp][DP];
-    int kd[DP];
-    bool logit[DP];
+    float xi[kRows][P], acc[kRows][P];
 #pragma unroll
-    for (int q = 0; q < DP; ++q) {
-        const int d = lane + 32 * q;
-        kd[q] = d < D ? d / P : 0;
-        logit[q] = d < D && d % P < M;
+    for (int r = 0; r < kRows; ++r) {
+        const int i = i0 + row0 + r;
 #pragma unroll
-        for (int r = 0; r < kRowsPerWarp; ++r) {
-            const int i = i0 + warp * kRowsPerWarp + r;
-            xi[r][q] = i < N && d < D ? column(i, d) : 0.f;
-            acc[r][q] = 0.f;
+        for (int c = 0; c < P; ++c) {
+            xi[r][c] = i >= N ? 0.f
+                       : c < M ? S[(size_t)i * M * H + ks * M + c] : theta[(size_t)i * D + ks * P + c];
+            acc[r][c] = 0.f;
         }
     }
     // this CTA's share of the sum over j; partial directions go to share blockIdx.y
@@ -105,80 +92,94 @@ struct_phi_kernel(const float* __restrict__ theta, const float* __restrict__ gra
     phi += (size_t)blockIdx.y * N * D;
     for (int j0 = jb; j0 < je; j0 += kTJ) {
         const int nj = min(kTJ, je - j0);
-        for (int t = tid; t < kTJ * D; t += kWarps * 32) {
-            const int jj = t / D, d = t % D;
-            Xj[t] = jj < nj ? column(j0 + jj, d) : 0.f;
-            Gj[t] = jj < nj ? grad[(size_t)j0 * D + t] : 0.f;
+        for (int t = tid; t < nj * H; t += kWarps * 32) {
+            const int jj = t / H, q = t - jj * H;
+            const float* s = S + (size_t)(j0 + jj) * M * H + q * M;
+            const float* th = theta + (size_t)(j0 + jj) * D + q * P;
+            float* x = Xj + t * P;
+#pragma unroll
+            for (int c = 0; c < P; ++c) x[c] = c < M ? s[c] : th[c];
         }
+        for (int t = tid; t < nj * D; t += kWarps * 32) Gj[t] = grad[(size_t)j0 * D + t];
+        if (tid < nj) Wj[tid] = wn ? wn[j0 + tid] : 1.f;
         __syncthreads();
-        // one (row, j) pair per thread: every action's kernels, and their sum K
-        for (int e = tid; e < kRows * kTJ; e += kWarps * 32) {
-            const int r = e / kTJ, jj = e % kTJ;
-            const float w = jj < nj ? (wn ? wn[j0 + jj] : 1.f) : 0.f;
-            float ksum = 0.f;
-            for (int k = 0; k < H; ++k) {
-                const float* a = Xi + r * D + k * P;
-                const float* b = Xj + jj * D + k * P;
-                float dz = 0.f, q = 0.f;
-                for (int c = 0; c < M; ++c) {
-                    const float bc = b[c], x = a[c] - bc;
-                    dz = fmaf(x, x, dz);
-                    q = fmaf(bc, x, q);
-                }
-                const float du = a[M] - b[M], dv = a[M + 1] - b[M + 1];
-                const float ec = expf(-(du * du + dv * dv) * inv_hc);
-                const float ez = expf(-dz * inv_hz);
-                ksum += ec + ez;
-                const int o = (r * kTJ + jj) * H + k;
-                Ac[o] = ac * w * ec;
-                Az[o] = az * w * ez;
-                Q[o] = q;
+#pragma unroll 2
+        for (int jj = split; jj < nj; jj += kSplit) {
+            const float2* xp = reinterpret_cast<const float2*>(Xj + jj * D + ks * P);
+            const float2* gp = reinterpret_cast<const float2*>(Gj + jj * D + ks * P);
+            const float w = Wj[jj];
+            float x[P], g[P];
+#pragma unroll
+            for (int c = 0; c < P / 2; ++c) {
+                const float2 xv = xp[c], gv = gp[c];
+                x[2 * c] = xv.x; x[2 * c + 1] = xv.y;
+                g[2 * c] = gv.x; g[2 * c + 1] = gv.y;
             }
-            Ks[e] = alpha * ksum * w;
-        }
-        __syncthreads();
-        for (int jj = 0; jj < nj; ++jj) {
 #pragma unroll
-            for (int q = 0; q < DP; ++q) {
-                const int d = lane + 32 * q;
-                if (d >= D) continue;
-                const float g = Gj[jj * D + d], x = Xj[jj * D + d];
+            for (int r = 0; r < kRows; ++r) {
+                float dz = 0.f, q = 0.f, df[P];
 #pragma unroll
-                for (int r = 0; r < kRowsPerWarp; ++r) {
-                    const int rj = (warp * kRowsPerWarp + r) * kTJ + jj, o = rj * H + kd[q];
-                    // logits: A^z s_j ((s_i - s_j) - q); offset, distance: A^c (c_i - c_j)
-                    const float rep = logit[q] ? Az[o] * (x * ((xi[r][q] - x) - Q[o]))
-                                               : Ac[o] * (xi[r][q] - x);
-                    acc[r][q] = fmaf(Ks[rj], g, acc[r][q] + rep);
+                for (int c = 0; c < P; ++c) df[c] = xi[r][c] - x[c];
+#pragma unroll
+                for (int c = 0; c < M; ++c) {
+                    dz = fmaf(df[c], df[c], dz);
+                    q = fmaf(x[c], df[c], q);
+                }
+                const float ec = expf(-(df[M] * df[M] + df[M + 1] * df[M + 1]) * inv_hc);
+                const float ez = expf(-dz * inv_hz);
+                float sum = k < H ? ec + ez : 0.f;
+#pragma unroll
+                for (int o = 1; o < HP; o <<= 1) sum += __shfl_xor_sync(~0u, sum, o);
+                const float K = alpha * sum * w, Az = az * w * ez, Ac = ac * w * ec;
+                // logits: A^z s_j ((s_i - s_j) - q); offset, distance: A^c (c_i - c_j)
+#pragma unroll
+                for (int c = 0; c < P; ++c) {
+                    const float rep = c < M ? Az * (x[c] * (df[c] - q)) : Ac * df[c];
+                    acc[r][c] = fmaf(K, g[c], acc[r][c] + rep);
                 }
             }
         }
         __syncthreads();
     }
+    // the splits' sums, in order: split x row x column
+    float* sums = ssm;
+    if (k < H)
+#pragma unroll
+        for (int r = 0; r < kRows; ++r)
+#pragma unroll
+            for (int c = 0; c < P; ++c)
+                sums[((size_t)split * kCtaRows<HP> + row0 + r) * D + k * P + c] = acc[r][c];
+    __syncthreads();
     const float scale = wn ? 1.f : 1.f / (float)N;
+    const int n = min(kCtaRows<HP>, N - i0) * D;
+    for (int t = tid; t < n; t += kWarps * 32) {
+        float v = sums[t];
 #pragma unroll
-    for (int r = 0; r < kRowsPerWarp; ++r) {
-        const int i = i0 + warp * kRowsPerWarp + r;
-        if (i < N)
-#pragma unroll
-            for (int q = 0; q < DP; ++q) {
-                const int d = lane + 32 * q;
-                if (d < D) phi[(size_t)i * D + d] = acc[r][q] * scale;
-            }
+        for (int q = 1; q < kSplit; ++q) v += sums[q * kCtaRows<HP> * D + t];
+        phi[(size_t)i0 * D + t] = v * scale;
     }
 }
 
-template <int DP>
-cudaError_t struct_launch(dim3 grid, const float* theta, const float* grad, const float* S, int N, int H,
-                          int M, const float* hc, const float* hz, const float* wn, float* phi,
-                          int j_chunk, cudaStream_t st) {
-    const size_t smem = struct_smem(H * (M + 2), H);
+template <int M, int HP>
+cudaError_t struct_launch(const float* theta, const float* grad, const float* S, int N, int H,
+                          const float* hc, const float* hz, const float* wn, float* phi, int max_shares,
+                          int* shares, cudaStream_t st) {
+    const int D = H * (M + 2), rows = (N + kCtaRows<HP> - 1) / kCtaRows<HP>;
+    // split the sum over j so that about two CTAs (16 warps) per SM are in flight
+    int want = (2 * sm_count() + rows - 1) / rows;
+    want = want < 1 ? 1 : (want > max_shares ? max_shares : want);
+    const int j_chunk = ((N + want - 1) / want + kTJ - 1) / kTJ * kTJ;
+    *shares = (N + j_chunk - 1) / j_chunk;
+    const size_t tile = (2 * (size_t)kTJ * D + kTJ) * sizeof(float);
+    const size_t sums = (size_t)kSplit * kCtaRows<HP> * D * sizeof(float);
+    const size_t smem = tile > sums ? tile : sums;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(struct_phi_kernel<DP>,
+        cudaError_t e = cudaFuncSetAttribute(struct_phi_kernel<M, HP>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    struct_phi_kernel<DP><<<grid, kWarps * 32, smem, st>>>(theta, grad, S, N, H, M, hc, hz, wn, phi, j_chunk);
+    struct_phi_kernel<M, HP><<<dim3(rows, *shares), kWarps * 32, smem, st>>>(theta, grad, S, N, H, hc, hz, wn,
+                                                                             phi, j_chunk);
     return cudaGetLastError();
 }
 
@@ -201,22 +202,23 @@ cudaError_t launch_struct_phi(const float* theta, const float* grad, const float
                               int N, int H, int M, const float* hc_dev, const float* hz_dev,
                               const float* wn, float* phi, int max_shares, int* shares,
                               cudaStream_t st) {
-    if (H > kMaxHs) return cudaErrorInvalidValue;
-    const int D = H * (M + 2), rows = (N + kRows - 1) / kRows;
-    // split the sum over j so that about four CTAs per SM are in flight
-    int want = (4 * sm_count() + rows - 1) / rows;
-    want = want < 1 ? 1 : (want > max_shares ? max_shares : want);
-    const int j_chunk = ((N + want - 1) / want + kTJ - 1) / kTJ * kTJ;
-    *shares = (N + j_chunk - 1) / j_chunk;
-    const dim3 grid(rows, *shares);
-    switch ((D + 31) / 32) {
-        case 1: return struct_launch<1>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
-        case 2: return struct_launch<2>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
-        case 3: return struct_launch<3>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
-        case 4: return struct_launch<4>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
-        case 5: case 6: return struct_launch<6>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
-        case 7: case 8: case 9: return struct_launch<9>(grid, theta, grad, S, N, H, M, hc_dev, hz_dev, wn, phi, j_chunk, st);
+    if (H < 1 || H > kMaxHs) return cudaErrorInvalidValue;
+#define STRUCT_HP(M_, HP_) \
+    return struct_launch<M_, HP_>(theta, grad, S, N, H, hc_dev, hz_dev, wn, phi, max_shares, shares, st)
+#define STRUCT_M(M_)                    \
+    if (H == 1) STRUCT_HP(M_, 1);       \
+    if (H == 2) STRUCT_HP(M_, 2);       \
+    if (H <= 4) STRUCT_HP(M_, 4);       \
+    if (H <= 8) STRUCT_HP(M_, 8);       \
+    STRUCT_HP(M_, 16)
+    switch (M) {
+        case 4: STRUCT_M(4);
+        case 8: STRUCT_M(8);
+        case 12: STRUCT_M(12);
+        case 16: STRUCT_M(16);
     }
+#undef STRUCT_M
+#undef STRUCT_HP
     return cudaErrorInvalidValue;
 }
 
