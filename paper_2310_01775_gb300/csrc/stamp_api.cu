@@ -274,20 +274,16 @@ stamp_status svgd(stamp_problem* p, float* theta, const float* grad, int N, floa
         STAMP_CUDA(stamp::launch_struct_prep(theta, N, H, M, p->sk_C, p->sk_S, p->stream));
         stamp::SvgdScratch a{p->d2, p->hist, p->sel, p->counter, p->h, p->flag};
         stamp::SvgdScratch b{p->sk_d2, p->sk_hist, p->sk_sel, p->sk_counter, p->sk_h, p->flag};
-        const stamp::SvgdScratch* ss[2] = {&a, &b};
-        const float* comp[2] = {p->sk_C, p->sk_S};
-        const int width[2] = {2 * H, M * H};
-        for (int q = 0; q < 2; ++q) {
-            STAMP_CUDA(cudaMemsetAsync(ss[q]->hist, 0, (2048 + 2048 + 1024) * sizeof(unsigned), p->stream));
-            STAMP_TRY(timed(p, STAMP_K_PAIRWISE, [&] {
-                return stamp::launch_pairwise(comp[q], N, width[q], *ss[q], p->stream);
-            }));
-            if (N >= 2)
-                for (int dg = 1; dg <= 2; ++dg)
-                    STAMP_TRY(timed(p, STAMP_K_MEDIAN, [&] {
-                        return stamp::launch_median_digit(N, dg, *ss[q], nullptr, p->stream);
-                    }));
-        }
+        for (unsigned* hist : {a.hist, b.hist})
+            STAMP_CUDA(cudaMemsetAsync(hist, 0, (2048 + 2048 + 1024) * sizeof(unsigned), p->stream));
+        STAMP_TRY(timed(p, STAMP_K_PAIRWISE, [&] {
+            return stamp::launch_pairwise2(p->sk_C, 2 * H, a, p->sk_S, M * H, b, N, p->stream);
+        }));
+        if (N >= 2)
+            for (int dg = 1; dg <= 2; ++dg)
+                STAMP_TRY(timed(p, STAMP_K_MEDIAN, [&] {
+                    return stamp::launch_median_digit2(N, dg, a, b, p->stream);
+                }));
         if (h_out) STAMP_CUDA(stamp::launch_scale_scalar(p->h, 1.f / (float)H, h_out, p->stream));
         STAMP_TRY(timed(p, STAMP_K_PHI, [&] {
             return stamp::launch_struct_phi(theta, grad, p->sk_S, N, H, M, p->h, p->sk_h, wn,

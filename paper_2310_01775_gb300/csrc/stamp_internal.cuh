@@ -152,6 +152,11 @@ cudaError_t launch_small_step(float* theta, const float* grad, int N, int D, flo
 cudaError_t launch_pairwise(const float* theta, int N, int D, const SvgdScratch& s, cudaStream_t st);
 cudaError_t launch_median_digit(int N, int digit, const SvgdScratch& s, float* h_out,
                                 cudaStream_t st);
+// the same of two matrices of N rows, side by side
+cudaError_t launch_pairwise2(const float* x0, int D0, const SvgdScratch& s0, const float* x1, int D1,
+                             const SvgdScratch& s1, int N, cudaStream_t st);
+cudaError_t launch_median_digit2(int N, int digit, const SvgdScratch& s0, const SvgdScratch& s1,
+                                 cudaStream_t st);
 // Writes `*shares` partial Stein directions (N x D each, consecutive) to part;
 // at most max_shares.
 // wn: normalised importance weights of Eq. dsvgd (device N), or NULL: 1/N.

@@ -27,12 +27,23 @@ constexpr int kPT = 64, kPC = 32;   // tile edge, columns per chunk
 __device__ __forceinline__ int pw_at(int d, int row) {   // float index in a chunk
     return d * kPT + ((((row >> 2) ^ (d & 7)) << 2) | (row & 3));
 }
-__global__ void __launch_bounds__(256) pairwise_kernel(const float* __restrict__ theta, int N, int D,
-                                                       float* __restrict__ d2,
-                                                       unsigned* __restrict__ hist,
-                                                       unsigned* __restrict__ sel,
-                                                       unsigned* __restrict__ counter,
-                                                       float* __restrict__ h_dev, int nt) {
+// blockIdx.y: the matrix, of one or two side by side (the structured kernel's two
+// bandwidths: too few CTAs each to fill the chip.  GB300, N = 1024: distances and
+// the median's two passes 52 us one after the other, 29 side by side).
+struct Matrix {
+    const float* x;   // N x D
+    int D;
+    float* d2;
+    unsigned *hist, *sel, *counter;
+    float *h, *h_out;
+};
+struct Matrices { Matrix m[2]; };
+__global__ void __launch_bounds__(256) pairwise_kernel(const __grid_constant__ Matrices ms, int N, int nt) {
+    const Matrix& m = ms.m[blockIdx.y];
+    const float* __restrict__ theta = m.x;
+    float* __restrict__ d2 = m.d2;
+    unsigned* __restrict__ hist = m.hist;
+    const int D = m.D;
     // A and B chunks; the finished tile takes their place
     __shared__ __align__(16) float buf[kPT * (kPT + 1) > 2 * kPC * kPT ? kPT * (kPT + 1) : 2 * kPC * kPT];
     __shared__ unsigned h0[kBins0];
@@ -113,14 +124,14 @@ __global__ void __launch_bounds__(256) pairwise_kernel(const float* __restrict__
     __syncthreads();
     for (int t = tid; t < kBins0; t += 256)
         if (h0[t]) atomicAdd(&hist[t], h0[t]);
-    if (last_block(counter, gridDim.x)) {
+    if (last_block(m.counter, gridDim.x)) {
         if (N < 2) {
-            if (tid == 0) *h_dev = 1.f;
+            if (tid == 0) *m.h = 1.f;
             return;
         }
         unsigned b0, r0;
         find_bin<kBins0, 256>(hist, median_rank(N), b0, r0);
-        if (tid == 0) { sel[0] = b0; sel[1] = r0; }
+        if (tid == 0) { m.sel[0] = b0; m.sel[1] = r0; }
     }
 }
 
@@ -135,14 +146,9 @@ __global__ void __launch_bounds__(256) pairwise_batch_kernel(const SvgdInst* __r
 }
 
 
-__global__ void __launch_bounds__(256) median_digit_kernel(int N, int dg,
-                                                           const float* __restrict__ d2,
-                                                           unsigned* __restrict__ hist,
-                                                           unsigned* __restrict__ sel,
-                                                           unsigned* __restrict__ counter,
-                                                           float* __restrict__ h_dev,
-                                                           float* __restrict__ h_out) {
-    median_digit_body(N, dg, d2, hist, sel, counter, h_dev, h_out, blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(256) median_digit_kernel(const __grid_constant__ Matrices ms, int N, int dg) {
+    const Matrix& m = ms.m[blockIdx.y];
+    median_digit_body(N, dg, m.d2, m.hist, m.sel, m.counter + dg, m.h, m.h_out, blockIdx.x, gridDim.x);
 }
 
 // Batched: work item (instance, CTA index) of the instance's med_ctas CTAs.
@@ -514,25 +520,40 @@ cudaError_t phi_launch(const float* theta, const float* grad, int N, int D, cons
 
 }  // namespace
 
-cudaError_t launch_pairwise(const float* theta, int N, int D, const SvgdScratch& s,
-                            cudaStream_t st) {
+static Matrix matrix(const float* x, int D, const SvgdScratch& s, float* h_out) {
+    return Matrix{x, D, s.d2, s.hist, s.sel, s.counter, s.h, h_out};
+}
+static cudaError_t pairwise(const Matrices& ms, int n, int N, cudaStream_t st) {
     const int nt = (N + kPT - 1) / kPT;
-    pairwise_kernel<<<nt * (nt + 1) / 2, 256, 0, st>>>(theta, N, D, s.d2, s.hist, s.sel, s.counter,
-                                                       s.h, nt);
+    pairwise_kernel<<<dim3(nt * (nt + 1) / 2, n), 256, 0, st>>>(ms, N, nt);
     return cudaGetLastError();
 }
-
-cudaError_t launch_median_digit(int N, int digit, const SvgdScratch& s, float* h_out,
-                                cudaStream_t st) {
+static cudaError_t median_digit(const Matrices& ms, int n, int N, int digit, cudaStream_t st) {
     // a CTA flushes its bins once: few CTAs for a small matrix (two a SM: 13 us
     // a digit at N = 2048, 18 with six), more loads in flight for a large one
     // (N = 6001: 42 + 34 us for the two digits with two, 27 + 21 with six)
     const int cap = (N >= 4096 ? 6 : 2) * sm_count();
     int grid = N - 1 < cap ? N - 1 : cap;
     if (grid < 1) grid = 1;
-    median_digit_kernel<<<grid, 256, 0, st>>>(N, digit, s.d2, s.hist, s.sel, s.counter + digit,
-                                              s.h, h_out);
+    median_digit_kernel<<<dim3(grid, n), 256, 0, st>>>(ms, N, digit);
     return cudaGetLastError();
+}
+cudaError_t launch_pairwise(const float* theta, int N, int D, const SvgdScratch& s,
+                            cudaStream_t st) {
+    return pairwise(Matrices{{matrix(theta, D, s, nullptr)}}, 1, N, st);
+}
+cudaError_t launch_median_digit(int N, int digit, const SvgdScratch& s, float* h_out,
+                                cudaStream_t st) {
+    return median_digit(Matrices{{matrix(nullptr, 0, s, h_out)}}, 1, N, digit, st);
+}
+cudaError_t launch_pairwise2(const float* x0, int D0, const SvgdScratch& s0, const float* x1, int D1,
+                             const SvgdScratch& s1, int N, cudaStream_t st) {
+    return pairwise(Matrices{{matrix(x0, D0, s0, nullptr), matrix(x1, D1, s1, nullptr)}}, 2, N, st);
+}
+cudaError_t launch_median_digit2(int N, int digit, const SvgdScratch& s0, const SvgdScratch& s1,
+                                 cudaStream_t st) {
+    return median_digit(Matrices{{matrix(nullptr, 0, s0, nullptr), matrix(nullptr, 0, s1, nullptr)}}, 2, N,
+                        digit, st);
 }
 
 cudaError_t launch_phi_rows(const float* theta, const float* grad, int N, int D, int row0,
