@@ -260,7 +260,7 @@ stamp_status stamp_set_overlap(stamp_problem* prob, int enable);
  * tape (scratch of (H*T + 1) x N x S floats, allocated at create when at most
  * 4 GiB) and recomputes nothing.
  * STAMP_ADJ_AUTO (the default): time-parallel where it applies, for up to
- * 3072 particles (beyond that the sequential teams fill the GPU and the
+ * 2048 particles (beyond that the sequential teams fill the GPU and the
  * Jacobians' extra arithmetic costs more than it saves), else
  * STAMP_ADJ_REPLAY where it applies, else sequential.
  * All sweeps give the gradient of the same float32 simulation, with sums

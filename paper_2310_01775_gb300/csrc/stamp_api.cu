@@ -38,7 +38,7 @@ constexpr long long kMaxStatsIters = 1 << 20;
 // the time-parallel reverse sweep keeps 39 coefficients per particle and
 // substep; above this it is not set up (the sequential sweep runs)
 constexpr size_t kMaxTimeParallelBytes = (size_t)4 << 30;
-constexpr int kTimeParallelMaxN = 3072;   // the automatic mode's crossover (see time_parallel)
+constexpr int kTimeParallelMaxN = 2048;   // the automatic mode's crossover (see time_parallel)
 constexpr unsigned kInjectedWaitLimit = 4096;   // polls of a wait made to run out (test hook)
 
 bool is_device_ptr(const void* p) {
@@ -176,10 +176,11 @@ stamp_status check_dev(const void* ptr, const char* name, bool allow_null = fals
 
 // The reverse sweep a call with N particles uses: time-parallel where its
 // scratch exists and, in the automatic mode, up to kTimeParallelMaxN
-// particles -- measured on GB300 (one block, H = 4, T = 100): the
-// time-parallel sweep takes half the sequential one's time at 1024
-// particles and breaks even near 4096, where the sequential teams fill the
-// GPU and the Jacobians' extra arithmetic no longer comes for free.
+// particles -- measured on GB300 (one block, H = 4, T = 100): the sequential
+// teams take 121 us at any N up to 4096 (a warp per scheduler or less, bound by
+// the serial chain), the time-parallel sweep 39 at 128 particles, 67 at 1024,
+// 105 at 2048 and 163 at 3072, where the Jacobians' extra arithmetic no longer
+// comes for free (H = 1 or 2: 33 to 35 us against 34 at 1600, 37 at 2048, 52 at 3072).
 bool time_parallel(const stamp_problem* p, int N) {
     if (!p->pit_ok || p->adj_mode == STAMP_ADJ_SEQUENTIAL || p->adj_mode == STAMP_ADJ_REPLAY)
         return false;
