@@ -247,9 +247,9 @@ __global__ void adam_batch_kernel(float* __restrict__ theta, float* __restrict__
 // A whole Stein step of at most kSmallN particles in one CTA: distances, their
 // exact lower median (bisection on the float bits), direction and Adam.  The
 // six launches it replaces cost more than their work (N = 32, D = 12: 30 us
-// against 8).
-// Every sum runs in the order of the kernels above with the direct form of the
-// repulsion: 32 particles a share.
+// against 9).
+// Every sum has the terms and the order of the kernels above and of phi_body, 32
+// particles a share, so an instance of a batch moves as one solved alone does.
 template <int E>   // N <= E (32 or 64)
 __global__ void __launch_bounds__(1024) small_step_kernel(
     float* __restrict__ theta, const float* __restrict__ grad, int N, int D, float* __restrict__ m,
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(1024) small_step_kernel(
     float* T = ssm;
     float* G = T + E * ld;
     __shared__ float K[E][E + 1];   // d2, then the kernel values
-    __shared__ float h_sh;
+    __shared__ float S[E][E / 32];  // a share's kernel values summed
     const int tid = threadIdx.x;
     for (int t = tid; t < N * D; t += 1024) {
         T[(t / D) * ld + t % D] = theta[t];
@@ -307,26 +307,34 @@ __global__ void __launch_bounds__(1024) small_step_kernel(
         if (h_out) *h_out = h;
     }
     const float inv_h = 1.f / h, two_h = 2.f * inv_h;
-    for (int t = tid; t < N * N; t += 1024) {
-        const int i = t / N, j = t % N;
-        float k = expf(-K[i][j] * inv_h);
-        if (wn) k *= wn[j];
+    for (int t = tid; t < E * E; t += 1024) {   // a warp: a row and share
+        const int i = t / E, j = t % E;
+        float k = 0.f;
+        if (i < N && j < N && i != j) {
+            k = expf(-K[i][j] * inv_h);
+            if (wn) k *= wn[j];
+        }
         K[i][j] = k;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(~0u, k, o);
+        if (tid % 32 == 0) S[i][j / 32] = k;
+    }
+    for (int t = tid; t < N * D; t += 1024) {   // u in place of g
+        const int j = t / D, d = t % D;
+        G[j * ld + d] = fmaf(-two_h, T[j * ld + d] - T[d], G[j * ld + d]);
     }
     __syncthreads();
     const float inv_n = wn ? 1.f : 1.f / (float)N;
     for (int t = tid; t < N * D; t += 1024) {
         const int i = t / D, d = t % D;
-        const float ti = T[i * ld + d];
+        const float ti = T[i * ld + d], self = wn ? wn[i] : 1.f;
         float phi = 0.f;
         for (int j0 = 0; j0 < N; j0 += kTJ) {
-            float ag = 0.f, ar = 0.f;
-            for (int j = j0; j < min(N, j0 + kTJ); ++j) {
-                ag = fmaf(K[i][j], G[j * ld + d], ag);
-                ar = fmaf(K[i][j], ti - T[j * ld + d], ar);
-            }
-            const float part = fmaf(two_h, ar, ag) * inv_n;
-            phi = j0 ? phi + part : part;
+            float a = 0.f;
+            for (int j = j0; j < min(N, j0 + kTJ); ++j) a = fmaf(K[i][j], G[j * ld + d], a);
+            a = fmaf(two_h * (ti - T[d]), S[i][j0 / kTJ], a);
+            if (self != 0.f && i / kTJ == j0 / kTJ) a = fmaf(self, grad[t], a);
+            phi = j0 ? phi + a * inv_n : a * inv_n;
         }
         if (phi_out) phi_out[t] = phi;
         const float g = -phi;

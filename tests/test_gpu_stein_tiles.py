@@ -63,3 +63,25 @@ def test_structured_step(N, nb, H):
     ref = O.stein_direction_structured(theta.astype(np.float64), g.astype(np.float64), P)
     ref = ref[0] if isinstance(ref, tuple) else ref
     assert np.abs(phi.cpu().numpy() - ref).max() <= 1e-4 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("N,nb,H", [(1921, 1, 6), (2113, 4, 7), (1921, 4, 16)])   # D = 36, 126, 288
+def test_many_particles(N, nb, H):
+    """Eight rows per warp; a shard of the rows (ragged, not at a tile's edge) sums
+    as all rows do."""
+    prob, _ = make_problem(N, n_blocks=nb, H=H)
+    theta, g = W.random_theta(N, prob.D, N + H), W.random_normal((N, prob.D), N + H + 1)
+    th, gr = torch.tensor(theta, device="cuda"), torch.tensor(g, device="cuda")
+    h, phi = torch.zeros(1, device="cuda"), torch.zeros_like(th)
+    m, v = torch.zeros_like(th), torch.zeros_like(th)
+    a = th.clone()
+    prob.svgd_step(a, gr, N, m, v, 1, 1e-2, 0, h, phi)
+    prob.sync()
+    check(theta, g, float(h), phi.cpu().numpy())
+    row0, rows = 130, N - 161
+    part = th[row0:row0 + rows].clone()
+    m, v = torch.zeros_like(part), torch.zeros_like(part)
+    prob.svgd_step_rows(th, gr, N, row0, rows, part, m, v, 1, 1e-2, 0)
+    prob.sync()
+    prob.close()
+    assert torch.equal(part, a[row0:row0 + rows])
