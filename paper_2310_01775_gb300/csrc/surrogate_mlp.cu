@@ -10,7 +10,7 @@
 // 40 us, packing 13.5, MLP 88, unpacking 6; at 2048 rows 8 + 3 + 18 + 3, and
 // the launches between them; six pushes of 131072 rows take 530 us here.  Few
 // plans would leave most SMs idle (2048 rows: 16 tiles, 95 us, and 97 in reverse):
-// they go to the cluster kernels below (33 and 30 us).
+// they go to the cluster kernels below (36 and 37 us).
 // Reverse, per push: the pose adjoints (in registers) are the head's dy; the
 // input-gradient chain of mlp_bwd_kernel; the features' reverse on the row.
 //
