@@ -241,6 +241,7 @@ mlp_bwd_kernel(const float* __restrict__ dy, int rows, int out_dim, int n_tiles,
     const int row = quarter * 32 + lane;
     unsigned tma_phase = 0, mma_phase = 0;
     bool failed = false, tma_pending = false, mma_pending = false;
+    after_previous();
     auto issue_load = [&](int m) {   // W_m^T into shared memory
         const unsigned wbytes = (unsigned)(layer_k(m) * layer_n(m) * 2);
         mbar_expect_tx(&sm.tma_bar, wbytes);
@@ -415,6 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_dw_kernel(const DwArgs a) {
     __syncthreads();
     tc_fence_after();
     const unsigned tmem = sm.tmem_slot;
+    after_previous();
     const int t0 = split * L.per, t1 = min(a.n_tiles, t0 + L.per);
     constexpr unsigned kPHalf = kRows * kRows * 2;   // 32 KB: 16 row groups of 2 KB
     auto issue = [&](int t) {
@@ -540,6 +542,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_dw_kernel(const DwArgs a) {
 // dW and db of every layer from the splits' partials, summed in split order.
 // part: [split][256 units of P][NQ]; where P holds the layer's inputs, D = dW^T.
 __global__ void __launch_bounds__(256) mlp_dw_reduce_kernel(const DwArgs a) {
+    after_previous();
     const int e = blockIdx.x * 256 + threadIdx.x;
     int li = 0;
 #pragma unroll
@@ -633,9 +636,8 @@ cudaError_t backward(const float* dy, int rows, int in_dim, int out_dim,
                                          (int)smem);
     if (e != cudaSuccess) return e;
     const int grid = n_tiles < sm_count ? n_tiles : sm_count;
-    mlp_bwd_kernel<<<grid, kThreads, smem, st>>>(dy, rows, out_dim, n_tiles, wt_tiled, zsave,
-                                                 dzsave, tile_base, tile_cap, dx, in_dim, err);
-    return cudaGetLastError();
+    return launch_after(mlp_bwd_kernel, dim3(grid), kThreads, smem, st, dy, rows, out_dim, n_tiles, wt_tiled, zsave,
+                        dzsave, tile_base, tile_cap, dx, in_dim, err);
 }
 
 size_t dw_part_floats() {   // a layer: 256 x NQ and 256 bias sums per split
@@ -693,11 +695,9 @@ cudaError_t weight_grads(const unsigned char* x_tiled, const unsigned char* save
         L.e0 = elem;
         elem += kHidden * L.NQ;
     }
-    mlp_dw_kernel<<<cta, kThreads, smem, st>>>(a);
-    e = cudaGetLastError();
+    e = launch_after(mlp_dw_kernel, dim3(cta), kThreads, smem, st, a);
     if (e != cudaSuccess) return e;
-    mlp_dw_reduce_kernel<<<(elem + 255) / 256, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(mlp_dw_reduce_kernel, dim3((elem + 255) / 256), 256, 0, st, a);
 }
 
 cudaError_t mse(const float* y, const float* t, int n, float* dy, float* loss, cudaStream_t st) {

@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(128)
 cost_kernel(const SimConst sc, int N, const float* __restrict__ src, const float* __restrict__ delta,
             const float* __restrict__ relax, float* __restrict__ cost, float* __restrict__ apose,
             unsigned* __restrict__ stats_min) {
+    after_previous();
     constexpr int M = rollout::Dims<NB>::M, P = M + 2;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -362,8 +363,7 @@ cudaError_t features(const SimConst& sc, const float* theta, int N, int k, uint6
 template <int NB>
 cudaError_t cost(const SimConst& sc, int N, const float* src, const float* delta, const float* relax,
                  float* c, float* apose, unsigned* stats, cudaStream_t st) {
-    cost_kernel<NB><<<(N + 127) / 128, 128, 0, st>>>(sc, N, src, delta, relax, c, apose, stats);
-    return cudaGetLastError();
+    return launch_after(cost_kernel<NB>, dim3((N + 127) / 128), 128, 0, st, sc, N, src, delta, relax, c, apose, stats);
 }
 cudaError_t features_nb(const SimConst& sc, const float* theta, int N, int k, uint64_t seed, int iter,
                         const float* src, const float* delta, float* pose_out, float* x, float* relax,

@@ -572,6 +572,7 @@ __global__ void __launch_bounds__(kThreads, 1) sur_fwd_cluster_kernel(const SimC
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     SurClSmem<TR>& sm = *reinterpret_cast<SurClSmem<TR>*>(smem_raw);
     ClusterSide<TR> s(sm);
+    after_previous();
     const int tile = blockIdx.x / 2;
     // a thread per row: warps 0 .. hold the poses, warps 4 .. fetch the action's features
     const int row = s.tid % 128, i = tile * TR + row;
@@ -664,6 +665,7 @@ __global__ void __launch_bounds__(kThreads, 1) sur_bwd_cluster_kernel(const SimC
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     SurClSmem<TR>& sm = *reinterpret_cast<SurClSmem<TR>*>(smem_raw);
     ClusterSide<TR> s(sm);
+    after_previous();
     const int tile = blockIdx.x / 2, row = s.tid % 128, i = tile * TR + row;
     const bool posed = s.tid < TR, on = posed && i < a.N;   // a thread per row
     if (s.tid == 0) {   // this CTA's rows of the transposed weights, all of W_0^T
@@ -742,12 +744,14 @@ cudaError_t launch_cluster(const SimConst& sc, const SurArgs& a, bool reverse, c
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = sizeof(SurClSmem<TR>);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_after
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)cfg.dynamicSmemBytes);
     if (e != cudaSuccess) return e;

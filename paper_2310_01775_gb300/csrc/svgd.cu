@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(256) pairwise_batch_kernel(const SvgdInst* __r
 
 
 __global__ void __launch_bounds__(256) median_digit_kernel(const __grid_constant__ Matrices ms, int N, int dg) {
+    after_previous();
     const Matrix& m = ms.m[blockIdx.y];
     median_digit_body(N, dg, m.d2, m.hist, m.sel, m.counter + dg, m.h, m.h_out, blockIdx.x, gridDim.x);
 }
@@ -196,6 +197,7 @@ __global__ void adam_kernel(float* __restrict__ theta, const float* __restrict__
                             float* __restrict__ phi_out, float* __restrict__ m,
                             float* __restrict__ v, int n, float lr, float bc1, float bc2,
                             int* flag) {
+    after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     float phi = part[t];
@@ -543,8 +545,7 @@ static cudaError_t median_digit(const Matrices& ms, int n, int N, int digit, cud
     const int cap = (N >= 4096 ? 6 : 2) * sm_count();
     int grid = N - 1 < cap ? N - 1 : cap;
     if (grid < 1) grid = 1;
-    median_digit_kernel<<<dim3(grid, n), 256, 0, st>>>(ms, N, digit);
-    return cudaGetLastError();
+    return launch_after(median_digit_kernel, dim3(grid, n), 256, 0, st, ms, N, digit);
 }
 cudaError_t launch_pairwise(const float* theta, int N, int D, const SvgdScratch& s,
                             cudaStream_t st) {
@@ -597,9 +598,8 @@ cudaError_t launch_adam(float* theta, const float* part, int shares, float* phi_
                         float* v, int n, int step, float lr, int* flag, cudaStream_t st) {
     const float bc1 = 1.f - powf(0.9f, (float)step);
     const float bc2 = 1.f - powf(0.999f, (float)step);
-    adam_kernel<<<(n + 255) / 256, 256, 0, st>>>(theta, part, shares, phi_out, m, v, n, lr, bc1,
-                                                 bc2, flag);
-    return cudaGetLastError();
+    return launch_after(adam_kernel, dim3((n + 255) / 256), 256, 0, st, theta, part, shares, phi_out, m, v,
+                        n, lr, bc1, bc2, flag);
 }
 
 cudaError_t launch_small_step(float* theta, const float* grad, int N, int D, float* m, float* v,

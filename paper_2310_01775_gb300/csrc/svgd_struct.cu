@@ -73,6 +73,7 @@ struct_phi_kernel(const float* __restrict__ theta, const float* __restrict__ gra
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int split = warp % kSplit, k = lane % HP, ks = k < H ? k : 0;
     const int row0 = (warp / kSplit * kGroups + lane / HP) * kRows, i0 = blockIdx.x * kCtaRows<HP>;
+    after_previous();
     const float Hf = (float)H;
     const float inv_hc = Hf / __ldg(hc_dev), inv_hz = Hf / __ldg(hz_dev);   // h = h_plain / H
     const float alpha = 0.5f / Hf, ac = alpha * (2.f * inv_hc), az = alpha * (2.f * inv_hz);
@@ -178,9 +179,8 @@ cudaError_t struct_launch(const float* theta, const float* grad, const float* S,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    struct_phi_kernel<M, HP><<<dim3(rows, *shares), kWarps * 32, smem, st>>>(theta, grad, S, N, H, hc, hz, wn,
-                                                                             phi, j_chunk);
-    return cudaGetLastError();
+    return launch_after(struct_phi_kernel<M, HP>, dim3(rows, *shares), kWarps * 32, smem, st, theta, grad, S, N,
+                        H, hc, hz, wn, phi, j_chunk);
 }
 
 __global__ void scale_scalar_kernel(const float* src, float s, float* dst) { *dst = *src * s; }
