@@ -301,6 +301,7 @@ __device__ __forceinline__ void pair_row(const SimConst& sc, const Blocks<1>& s,
 
 // Relaxed parameters of every (particle, action), as the forward computed them.
 __global__ void relax_kernel(const SimConst sc, const RolloutArgs a, float* __restrict__ rel) {
+    after_previous();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= a.N * sc.H) return;
     const int i = idx % a.N, k = idx / a.N;
@@ -322,6 +323,7 @@ __global__ void relax_kernel(const SimConst sc, const RolloutArgs a, float* __re
 __global__ void __launch_bounds__(128) jac_kernel(const SimConst sc, const RolloutArgs a,
                                                   const float* __restrict__ rel,
                                                   float* __restrict__ coef) {
+    after_previous();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int HT = sc.H * sc.T;
     if (idx >= (long long)a.N * HT) return;
@@ -398,6 +400,7 @@ __global__ void __launch_bounds__(32) scan_kernel(const SimConst sc, const Rollo
                                                   int* __restrict__ flag) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ScanSmem& sm = *reinterpret_cast<ScanSmem*>(smem_raw);
+    after_previous();
     const int tid = threadIdx.x, p = tid >> 2, lane = tid & 3;
     const int grp = blockIdx.x;
     int i = grp * kGroup + p;
@@ -552,10 +555,11 @@ cudaError_t launch_adjoint_time(const SimConst& sc, const RolloutArgs& a, float*
                                                (int)kScanSmem);
     if (e != cudaSuccess) return e;
     const long long pairs = (long long)a.N * sc.H * sc.T;
-    relax_kernel<<<(a.N * sc.H + 127) / 128, 128, 0, st>>>(sc, a, rel);
-    jac_kernel<<<(unsigned)((pairs + 127) / 128), 128, 0, st>>>(sc, a, rel, coef);
-    scan_kernel<<<(a.N + kGroup - 1) / kGroup, 32, kScanSmem, st>>>(sc, a, rel, coef, flag);
-    return cudaGetLastError();
+    cudaError_t l = launch_after(relax_kernel, dim3((a.N * sc.H + 127) / 128), 128, 0, st, sc, a, rel);
+    if (l != cudaSuccess) return l;
+    l = launch_after(jac_kernel, dim3((unsigned)((pairs + 127) / 128)), 128, 0, st, sc, a, rel, coef);
+    if (l != cudaSuccess) return l;
+    return launch_after(scan_kernel, dim3((a.N + kGroup - 1) / kGroup), 32, kScanSmem, st, sc, a, rel, coef, flag);
 }
 
 }  // namespace stamp

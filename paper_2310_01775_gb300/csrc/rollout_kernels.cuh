@@ -19,6 +19,7 @@ __device__ __forceinline__ bool real_team(int gtid, int lanes) {
 
 template <int NB, int QL>
 __global__ void __launch_bounds__(128) rollout_fwd_kernel(const SimConst sc, const RolloutArgs a) {
+    after_previous();
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
     int i = gtid / a.lanes;
     const bool on = i < a.N && real_team<NB, QL>(gtid, a.lanes);
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(128) rollout_fwd_batch_kernel(const SimConst s
 
 template <int NB, int QL>
 __global__ void __launch_bounds__(128) rollout_adj_kernel(const SimConst sc, const RolloutArgs a) {
+    after_previous();
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
     int i = gtid / a.lanes;
     const bool on = i < a.N && real_team<NB, QL>(gtid, a.lanes);
@@ -114,19 +116,14 @@ cudaError_t launch(const SimConst& sc, const RolloutArgs& a, bool adjoint, cudaS
     int cta = 32;
     while (cta < 128 && threads_total / (cta * 2) >= sms) cta *= 2;
     const int grid = (int)((threads_total + cta - 1) / cta);
-    if (!adjoint) {
-        rollout_fwd_kernel<NB, QL><<<grid, cta, 0, st>>>(sc, a);
-    } else {
-        const size_t smem = (size_t)(cta / a.lanes) * seg_stride<NB>(sc.C) * sizeof(float2);
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(rollout_adj_kernel<NB, QL>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        rollout_adj_kernel<NB, QL><<<grid, cta, smem, st>>>(sc, a);
+    if (!adjoint) return launch_after(rollout_fwd_kernel<NB, QL>, dim3(grid), cta, 0, st, sc, a);
+    const size_t smem = (size_t)(cta / a.lanes) * seg_stride<NB>(sc.C) * sizeof(float2);
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(rollout_adj_kernel<NB, QL>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
     }
-    return cudaGetLastError();
+    return launch_after(rollout_adj_kernel<NB, QL>, dim3(grid), cta, smem, st, sc, a);
 }
 
 // Batched launch of one block-count class: b.n_teams teams of L lanes in

@@ -305,6 +305,7 @@ stamp_status svgd(stamp_problem* p, float* theta, const float* grad, int N, floa
             p->inject_wait_timeout = false;
         }
         if (!bw_done) STAMP_TRY(bandwidth(p, theta, N, h_out, p->stream));
+        s.chained = !bw_done;
         STAMP_TRY(timed(p, STAMP_K_PHI, [&] {
             return stamp::launch_phi(theta, grad, N, D, s, p->phi, stamp::kMaxShares, &shares,
                                      p->stream, wn);

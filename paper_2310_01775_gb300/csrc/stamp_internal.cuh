@@ -166,6 +166,7 @@ struct SvgdScratch {
     // shared-memory stage without issuing its copy, so that wait runs out
     unsigned wait_limit = 0;
     int skip_first_copy = 0;
+    bool chained = false;   // the direction follows the median on its stream, no event between
 };
 // A whole RBF Stein step (bandwidth, direction, Adam) of N <= kSmallN particles.
 constexpr int kSmallN = 64;

@@ -194,6 +194,7 @@ __device__ __forceinline__ unsigned cost_key(float cost) {   // a negative or Na
 __global__ void __launch_bounds__(256) select_pass_kernel(const float* __restrict__ cost, int n, int N,
                                                           int p, Select s) {
     __shared__ unsigned h[kSelBins], st[24];
+    after_previous();
     for (int t = threadIdx.x; t < kSelBins; t += 256) h[t] = 0u;
     if (threadIdx.x < 24) st[threadIdx.x] = __ldcg(s.state + threadIdx.x);
     __syncthreads();
@@ -221,6 +222,7 @@ __global__ void __launch_bounds__(256) select_pass_kernel(const float* __restric
 }
 __global__ void __launch_bounds__(256) select_gather_kernel(const float* __restrict__ cost, int n, Select s,
                                                             unsigned long long* __restrict__ out) {
+    after_previous();
     const unsigned* st = s.state;
     const unsigned long long last = (unsigned long long)(st[8] << 21 | st[10] << 10 | st[12]) << 32 |
                                     (st[14] << 10 | st[16]);
@@ -234,6 +236,7 @@ __global__ void __launch_bounds__(256) select_place_kernel(const unsigned long l
                                                            int N, int D, const float* __restrict__ cand,
                                                            float* __restrict__ theta,
                                                            int* __restrict__ index) {
+    after_previous();
     const int lane = threadIdx.x & 31, q = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (q >= N) return;
     const unsigned long long key = keys[q];
@@ -482,11 +485,12 @@ stamp_status surrogate_screen(stamp_surrogate* s, const SimConst& sc, const floa
     // four candidates a thread: enough CTAs to fill the GPU, few flushes of the bins
     const int grid = std::min(2 * net_sms(s), (n_cand + 1023) / 1024);
     for (int p = 0; p < surrogate::kSelPasses; ++p)
-        surrogate::select_pass_kernel<<<grid, 256, 0, s->stream>>>(s->cost, n_cand, N, p, sel);
-    surrogate::select_gather_kernel<<<(n_cand + 255) / 256, 256, 0, s->stream>>>(s->cost, n_cand, sel, s->keys);
-    surrogate::select_place_kernel<<<(N + 7) / 8, 256, 0, s->stream>>>(s->keys, N, sc.D, cand, theta_out,
-                                                                       index_out);
-    SUR_CUDA(cudaGetLastError(), "selection launch failed");
+        SUR_CUDA(launch_after(surrogate::select_pass_kernel, dim3(grid), 256, 0, s->stream, s->cost, n_cand, N, p,
+                              sel), "selection launch failed");
+    SUR_CUDA(launch_after(surrogate::select_gather_kernel, dim3((n_cand + 255) / 256), 256, 0, s->stream, s->cost,
+                          n_cand, sel, s->keys), "selection launch failed");
+    SUR_CUDA(launch_after(surrogate::select_place_kernel, dim3((N + 7) / 8), 256, 0, s->stream, s->keys, N, sc.D,
+                          cand, theta_out, index_out), "selection launch failed");
     return STAMP_OK;
 }
 

@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(kW * 32) phi_kernel(const float* __restrict__ 
                                                       int* err, const float* __restrict__ wn,
                                                       unsigned wait_limit, int skip_first, int row0,
                                                       int rows) {
+    after_previous();
     phi_body<DP, kW, 8, R>(theta, grad, N, D, d2, h_dev, part, j_chunk, err, blockIdx.x, blockIdx.y, wn,
                            wait_limit, skip_first != 0, row0, rows);
 }
@@ -475,7 +476,7 @@ template <int DP, int R>
 cudaError_t phi_launch_rows(const float* theta, const float* grad, int N, int D, const float* d2,
                             const float* h_dev, float* part, int shares, int j_chunk, int* err,
                             const float* wn, unsigned wait_limit, int skip_first, int row0, int rows,
-                            cudaStream_t st) {
+                            bool chained, cudaStream_t st) {
     const size_t smem = phi_smem(D, DP, kW, R);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(phi_kernel<DP, R>,
@@ -483,8 +484,12 @@ cudaError_t phi_launch_rows(const float* theta, const float* grad, int N, int D,
         if (e != cudaSuccess) return e;
     }
     const int per_cta = kW * R;
-    phi_kernel<DP, R><<<dim3((rows + per_cta - 1) / per_cta, shares), kW * 32, smem, st>>>(
-        theta, grad, N, D, d2, h_dev, part, j_chunk, err, wn, wait_limit, skip_first, row0, rows);
+    const dim3 grid((rows + per_cta - 1) / per_cta, shares);
+    if (chained)
+        return launch_after(phi_kernel<DP, R>, grid, kW * 32, smem, st, theta, grad, N, D, d2, h_dev, part, j_chunk,
+                            err, wn, wait_limit, skip_first, row0, rows);
+    phi_kernel<DP, R><<<grid, kW * 32, smem, st>>>(theta, grad, N, D, d2, h_dev, part, j_chunk, err, wn, wait_limit,
+                                                   skip_first, row0, rows);
     return cudaGetLastError();
 }
 // The split of the Stein sum of N particles over j-shares and the rows per
@@ -521,11 +526,11 @@ template <int DP>
 cudaError_t phi_launch(const float* theta, const float* grad, int N, int D, const float* d2,
                        const float* h_dev, float* part, int shares, int j_chunk, int* err,
                        const float* wn, unsigned wait_limit, int skip_first, int row0, int rows,
-                       bool r8, cudaStream_t st) {
+                       bool r8, bool chained, cudaStream_t st) {
     return r8 ? phi_launch_rows<DP, 8>(theta, grad, N, D, d2, h_dev, part, shares, j_chunk, err, wn,
-                                       wait_limit, skip_first, row0, rows, st)
+                                       wait_limit, skip_first, row0, rows, chained, st)
               : phi_launch_rows<DP, 4>(theta, grad, N, D, d2, h_dev, part, shares, j_chunk, err, wn,
-                                       wait_limit, skip_first, row0, rows, st);
+                                       wait_limit, skip_first, row0, rows, chained, st);
 }
 
 }  // namespace
@@ -577,14 +582,14 @@ cudaError_t launch_phi_rows(const float* theta, const float* grad, int N, int D,
     const unsigned limit = s.wait_limit ? s.wait_limit : kWaitLimit;
     const int dp = (D + 31) / 32;
     switch (dp) {
-        case 1: return phi_launch<1>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
-        case 2: return phi_launch<2>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
-        case 3: return phi_launch<3>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
-        case 4: return phi_launch<4>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
+        case 1: return phi_launch<1>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
+        case 2: return phi_launch<2>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
+        case 3: return phi_launch<3>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
+        case 4: return phi_launch<4>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
         case 5: case 6:
-            return phi_launch<6>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
+            return phi_launch<6>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
         case 7: case 8: case 9:
-            return phi_launch<9>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, st);
+            return phi_launch<9>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
     }
     return cudaErrorInvalidValue;
 }
