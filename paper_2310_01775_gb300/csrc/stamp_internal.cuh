@@ -133,8 +133,9 @@ cudaError_t launch_adjoint_time(const SimConst& sc, const RolloutArgs& a, float*
 // SVGD step pieces (svgd.cu).  Scratch buffers are owned by the problem.
 // A launch that may be set up while the kernel before it in the stream ends
 // (programmatic stream serialisation): about 2 us less between two short
-// kernels (GB300: the Stein step of 2048 particles, five kernels, 95 -> 86 us).  The kernel must call after_previous() before it touches global memory;
-// that waits until everything before it is complete and visible.
+// kernels (GB300: the Stein step of 2048 particles, five kernels, 95 -> 86 us).
+// The kernel must call after_previous() before it touches global memory; that
+// waits until everything before it is complete and visible.
 template <class... P, class... A>
 cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                          const A&... args) {

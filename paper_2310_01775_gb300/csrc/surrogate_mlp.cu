@@ -761,8 +761,9 @@ cudaError_t launch_cluster(const SimConst& sc, const SurArgs& a, bool reverse, c
 template <int NB>
 cudaError_t launch(const SimConst& sc, const SurArgs& a, bool reverse, int sms, cudaStream_t st) {
     // The narrowest tile whose clusters all run at once: its time does not depend on
-    // N (GB300, 6 pushes with the gradient, launches one after the other: 78 us on 32 rows, 96 on 64, 181 on
-    // 128-row tiles; a second wave would double it).  The outputs' bits are the same.
+    // N (GB300, 6 pushes with the gradient, launches one after the other: 78 us on 32
+    // rows, 96 on 64, 181 on 128-row tiles; a second wave would double it).  The
+    // outputs' bits are the same.
     if (a.N <= sms / 2 * 32) return launch_cluster<NB, 32>(sc, a, reverse, st);
     if (a.N <= sms / 2 * 64) return launch_cluster<NB, 64>(sc, a, reverse, st);
     const size_t smem = (reverse ? sizeof(FwdSmem) : sizeof(SurSmem)) + 1024;
