@@ -126,11 +126,12 @@ cudaError_t launch(const SimConst& sc, const RolloutArgs& a, bool adjoint, cudaS
     return launch_after(rollout_adj_kernel<NB, QL>, dim3(grid), cta, smem, st, sc, a);
 }
 
-// Batched launch of one block-count class: b.n_teams teams of L lanes in
-// CTAs of `cta` threads (a multiple of 32).
+// Batched launch of one block-count class: b.n_teams teams of b.lanes lanes (as
+// the kernels number them, shadow teams included) in CTAs of `cta` threads (a
+// multiple of 32).
 template <int NB, int QL>
 cudaError_t launch_batch(const SimConst& sc, const BatchArgs& b, int cta, bool adjoint, cudaStream_t st) {
-    const long long threads_total = (long long)b.n_teams * team_lanes(NB, QL);
+    const long long threads_total = (long long)b.n_teams * b.lanes;
     const int grid = (int)((threads_total + cta - 1) / cta);
     if (grid < 1) return cudaSuccess;
     if (!adjoint) {
