@@ -286,8 +286,7 @@ stamp_status stamp_inject_wait_timeout(stamp_problem* prob);
 /* Lanes per particle used by the rollout kernels (one block 1, 2, 4; two
  * blocks 2..16; three and four blocks 8..32; 0 = automatic, by the number of
  * particles).  A particle works on 1, 2 or 4 lanes per block; lanes beyond
- * four per block idle.  The results do not depend on the width, except for the
- * order in which forces between blocks are summed. */
+ * four per block idle.  The width does not change a bit of the results. */
 stamp_status stamp_set_lanes(stamp_problem* prob, int fwd_lanes, int adj_lanes);
 /* Accepted as before (one block 1, 2, 4; two blocks 2..16; three blocks 2..32;
  * four blocks 4..32; 0 = automatic) and without effect: STAMP_ADJ_REPLAY has

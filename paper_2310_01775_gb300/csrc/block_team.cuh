@@ -27,8 +27,11 @@
 // (173 + 306 with QL = 4).  Four blocks, N = 613, H = 5: 539 + 901 against 255 + 355
 // (QL = 4).
 //
-// The arithmetic does not depend on QL: a block's four contact forces are
-// rounded first and added as (f0 + f1) + (f2 + f3) whatever lanes hold them.
+// The results' bits do not depend on QL, nor on the number of particles that a
+// width is picked by: every value that belongs to a side of a block (a contact's
+// force, what it sends to another block, an adjoint) is rounded by itself and a
+// block's four are added as (f0 + f1) + (f2 + f3), whatever lanes hold them; sums
+// of two products say which one is fused (dot2).
 #pragma once
 
 #include "rollout.cuh"
@@ -49,13 +52,6 @@ struct Own {   // this lane's pushers: start centres, displacements per substep,
 };
 
 constexpr unsigned kAll = 0xffffffffu;
-
-// a b + c d with the first product fused.  Where a sum has two products, the
-// compiler may fuse either, and picks by context: written out, every kernel
-// and team width rounds alike (the dynamics amplify a last bit).
-__device__ __forceinline__ float dot2(float a, float b, float c, float d) {
-    return fmaf(a, b, __fmul_rn(c, d));
-}
 
 template <int NB, int QL>
 struct Quad {
@@ -201,11 +197,14 @@ __device__ __forceinline__ void place(const SimConst& sc, const Quad<NB, QL>& q,
     }
 }
 
-// disk_box of rollout.cuh without its early outs: out of contact the results
-// are selected to zero, so the chain has no branch.  (ddx, ddy): the pusher's
-// displacement per substep; the relative velocity takes displacement/dt in one
-// fused multiply-add.
-__device__ __forceinline__ void disk_box_flat(const SimConst& sc, float px, float py, float ddx,
+// Force and torque on a square block (centre b, yaw via cph/sph, velocity v,
+// omega) from a kinematic disk pusher at p (unweighted).  (ddx, ddy): the
+// pusher's displacement per substep; the relative velocity takes displacement/dt
+// in one fused multiply-add.  A pusher's own block: out of contact the results are
+// selected to zero, so the chain has no branch.  kEarly (another block, already
+// behind a branch): return there.
+template <bool kEarly = false>
+__device__ __forceinline__ void disk_box(const SimConst& sc, float px, float py, float ddx,
                                               float ddy, float bx, float by, float cph, float sph,
                                               float vx, float vy, float om, float& fx, float& fy,
                                               float& tq) {
@@ -222,12 +221,17 @@ __device__ __forceinline__ void disk_box_flat(const SimConst& sc, float px, floa
     const float nlx = outside ? sx * mx * il : (xa ? sx : 0.f);
     const float nly = outside ? sy * my * il : (xa ? 0.f : sy);
     const float delta = sc.r - sd;
+    if (kEarly) {
+        fx = fy = tq = 0.f;
+        if (!(delta > 0.f)) return;
+    }
     const float nx = dot2(cph, nlx, -sph, nly), ny = dot2(sph, nlx, cph, nly);
     const float rx = px - sc.r * nx - bx, ry = py - sc.r * ny - by;
     const float wx = fmaf(ddx, sc.inv_dt, -(vx - om * ry)), wy = fmaf(ddy, sc.inv_dt, -(vy + om * rx));
     const float vn = dot2(wx, nx, wy, ny);
     const float fn = dot2(sc.k, delta, -sc.c, vn);
     const bool hit = delta > 0.f && fn > 0.f;
+    if (kEarly && !hit) return;
     const float tx = wx - vn * nx, ty = wy - vn * ny;
     const float gt = sc.mu_c * fn * rsqrtf(dot2(tx, tx, ty, ty) + sc.eps_t2);
     const float gx = dot2(gt, tx, -fn, nx), gy = dot2(gt, ty, -fn, ny);
@@ -304,7 +308,7 @@ __device__ __forceinline__ void block_substep(const SimConst& sc, const Quad<NB,
 #pragma unroll
     for (int j = 0; j < K; ++j) {
         float fx, fy, tq;
-        disk_box_flat(sc, px[j], py[j], o.dx[j], o.dy[j], s.x, s.y, cs, sn, s.vx, s.vy, s.om, fx, fy, tq);
+        disk_box(sc, px[j], py[j], o.dx[j], o.dy[j], s.x, s.y, cs, sn, s.vx, s.vy, s.om, fx, fy, tq);
         Fx[j] = __fmul_rn(o.w[j], fx);
         Fy[j] = __fmul_rn(o.w[j], fy);
         Tq[j] = __fmul_rn(o.w[j], tq);
@@ -322,31 +326,32 @@ __device__ __forceinline__ void block_substep(const SimConst& sc, const Quad<NB,
                 const float bc = from_lane(cs, to), bs = from_lane(sn, to);
                 const float bvx = from_lane(s.vx, to), bvy = from_lane(s.vy, to);
                 const float bom = from_lane(s.om, to);
-                float Rx = 0.f, Ry = 0.f, Rt = 0.f;   // on block b + d
+                float Rx[K], Ry[K], Rt[K];   // each side's, on block b + d
 #pragma unroll
                 for (int j = 0; j < K; ++j) {
                     float fx, fy, tq;
+                    Rx[j] = Ry[j] = Rt[j] = 0.f;
                     if (nd & (1u << (2 * j))) {
-                        disk_box(sc, px[j], py[j], o.dx[j] * sc.inv_dt, o.dy[j] * sc.inv_dt, bx, by, bc,
-                                 bs, bvx, bvy, bom, fx, fy, tq);
-                        Rx += o.w[j] * fx;
-                        Ry += o.w[j] * fy;
-                        Rt += o.w[j] * tq;
+                        disk_box<true>(sc, px[j], py[j], o.dx[j], o.dy[j], bx, by, bc, bs, bvx, bvy, bom, fx,
+                                       fy, tq);
+                        Rx[j] = __fmul_rn(o.w[j], fx);
+                        Ry[j] = __fmul_rn(o.w[j], fy);
+                        Rt[j] = __fmul_rn(o.w[j], tq);
                     }
                     if (nd & (2u << (2 * j))) {
-                        const float kvx = s.vx - s.om * rly[j], kvy = s.vy + s.om * rlx[j];
+                        const float kvx = fmaf(-s.om, rly[j], s.vx), kvy = fmaf(s.om, rlx[j], s.vy);
                         corner_box(sc, kx[j], ky[j], kvx, kvy, bx, by, bc, bs, bvx, bvy, bom, fx, fy);
                         Fx[j] += fx;
                         Fy[j] += fy;
-                        Tq[j] += rlx[j] * fy - rly[j] * fx;
-                        Rx -= fx;
-                        Ry -= fy;
-                        Rt -= (kx[j] - bx) * fy - (ky[j] - by) * fx;
+                        Tq[j] += dot2(rlx[j], fy, -rly[j], fx);
+                        Rx[j] -= fx;
+                        Ry[j] -= fy;
+                        Rt[j] -= dot2(kx[j] - bx, fy, -(ky[j] - by), fx);
                     }
                 }
-                Ix += from_lane(lanes_sum<QL>(Rx), from);
-                Iy += from_lane(lanes_sum<QL>(Ry), from);
-                It += from_lane(lanes_sum<QL>(Rt), from);
+                Ix += from_lane(block_sum<QL>(Rx), from);
+                Iy += from_lane(block_sum<QL>(Ry), from);
+                It += from_lane(block_sum<QL>(Rt), from);
             }
         }
     }
@@ -466,16 +471,18 @@ __device__ __forceinline__ void fwd_block_team(const SimConst& sc, const Rollout
 }
 
 // ------------------------------ reverse sweep --------------------------------
-// disk_box_vjp without its early outs: out of contact the incoming adjoints
-// are selected to zero.  The block's position and velocity adjoints are the
-// negatives of the pusher's.
+// VJP of disk_box for the weighted force (w f, w torque).  gFx, gFy, gT: adjoints
+// of the block's force and torque.  The block's position and velocity adjoints
+// are the negatives of the pusher's.  Out of contact: the incoming adjoints are
+// selected to zero, or (kEarly) all zero at once.
 struct DiskAdj {
     float px, py, vpx, vpy, ph, om, w;
 };
-__device__ __forceinline__ DiskAdj disk_box_vjp_flat(const SimConst& sc, float px, float py, float ddx,
-                                                     float ddy, float bx, float by, float cph, float sph,
-                                                     float vx, float vy, float om, float w, float gFx,
-                                                     float gFy, float gT) {
+template <bool kEarly = false>
+__device__ __forceinline__ DiskAdj disk_box_vjp(const SimConst& sc, float px, float py, float ddx,
+                                                float ddy, float bx, float by, float cph, float sph,
+                                                float vx, float vy, float om, float w, float gFx,
+                                                float gFy, float gT) {
     const float dx = px - bx, dy = py - by;
     const float lx = dot2(cph, dx, sph, dy), ly = dot2(cph, dy, -sph, dx);
     const float qx = fabsf(lx) - sc.hs, qy = fabsf(ly) - sc.hs;
@@ -490,12 +497,14 @@ __device__ __forceinline__ DiskAdj disk_box_vjp_flat(const SimConst& sc, float p
     const float nlx = outside ? sx * mx * il : (xa ? sx : 0.f);
     const float nly = outside ? sy * my * il : (xa ? 0.f : sy);
     const float delta = sc.r - sd;
+    if (kEarly && !(delta > 0.f)) return DiskAdj{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     const float nx = dot2(cph, nlx, -sph, nly), ny = dot2(sph, nlx, cph, nly);
     const float rx = px - sc.r * nx - bx, ry = py - sc.r * ny - by;
     const float wx = fmaf(ddx, sc.inv_dt, -(vx - om * ry)), wy = fmaf(ddy, sc.inv_dt, -(vy + om * rx));
     const float vn = dot2(wx, nx, wy, ny);
     const float fn = dot2(sc.k, delta, -sc.c, vn);
     const bool hit = delta > 0.f && fn > 0.f;
+    if (kEarly && !hit) return DiskAdj{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     gFx = hit ? gFx : 0.f;
     gFy = hit ? gFy : 0.f;
     gT = hit ? gT : 0.f;
@@ -560,6 +569,15 @@ struct OwnAcc {   // adjoints of the lane's pushers
     float p0x[K], p0y[K], dx[K], dy[K], w[K];
 };
 
+template <int K>
+struct Sides {   // adjoints of a block's state, by the side they come through
+    float x[K], y[K], ph[K], vx[K], vy[K], om[K];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int j = 0; j < K; ++j) x[j] = y[j] = ph[j] = vx[j] = vy[j] = om[j] = 0.f;
+    }
+};
+
 // Reverse of block_substep: `a` is the adjoint of the block's state after
 // the substep on entry, before it on exit.
 template <int NB, int QL>
@@ -589,7 +607,7 @@ __device__ __forceinline__ void block_substep_vjp(const SimConst& sc, const Quad
     float dpx[K], dpy[K], dph[K], dvx[K], dvy[K], dom[K];   // own contacts (position, velocity negated)
 #pragma unroll
     for (int j = 0; j < K; ++j) {
-        const DiskAdj g = disk_box_vjp_flat(sc, px[j], py[j], o.dx[j], o.dy[j], s.x, s.y, cs, sn, s.vx,
+        const DiskAdj g = disk_box_vjp(sc, px[j], py[j], o.dx[j], o.dy[j], s.x, s.y, cs, sn, s.vx,
                                             s.vy, s.om, o.w[j], aFx, aFy, aT);
         acc.p0x[j] += g.px;
         acc.p0y[j] += g.py;
@@ -602,7 +620,8 @@ __device__ __forceinline__ void block_substep_vjp(const SimConst& sc, const Quad
     One in{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // from the pairs with other blocks
     if constexpr (NB > 1) {
         if (__any_sync(kAll, near)) {
-            One c{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // from this lane's corners
+            Sides<K> c;   // to this block, from its corners
+            c.clear();
 #pragma unroll 1
             for (int d = 1; d < NB; ++d) {
                 const unsigned nd = (near >> (2 * K * (d - 1))) & ((1u << (2 * K)) - 1u);
@@ -614,20 +633,20 @@ __device__ __forceinline__ void block_substep_vjp(const SimConst& sc, const Quad
                 const float bvx = from_lane(s.vx, to), bvy = from_lane(s.vy, to);
                 const float bom = from_lane(s.om, to);
                 const float bFx = from_lane(aFx, to), bFy = from_lane(aFy, to), bT = from_lane(aT, to);
-                One r{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // to block b + d
+                Sides<K> r;   // to block b + d
+                r.clear();
 #pragma unroll
                 for (int j = 0; j < K; ++j) {
                     if (nd & (1u << (2 * j))) {
-                        const DiskGrad h = disk_box_vjp(
-                            sc, px[j], py[j], o.dx[j] * sc.inv_dt, o.dy[j] * sc.inv_dt, bx, by, bc, bs,
-                            bvx, bvy, bom, o.w[j], bFx, bFy, bT);
+                        const DiskAdj h = disk_box_vjp<true>(sc, px[j], py[j], o.dx[j], o.dy[j], bx, by, bc, bs,
+                                                             bvx, bvy, bom, o.w[j], bFx, bFy, bT);
                         acc.p0x[j] += h.px;
                         acc.p0y[j] += h.py;
-                        acc.dx[j] += j1 * h.px + h.vpx * sc.inv_dt;
-                        acc.dy[j] += j1 * h.py + h.vpy * sc.inv_dt;
+                        acc.dx[j] += dot2(j1, h.px, h.vpx, sc.inv_dt);
+                        acc.dy[j] += dot2(j1, h.py, h.vpy, sc.inv_dt);
                         acc.w[j] += h.w;
-                        r.x += h.bx; r.y += h.by; r.ph += h.ph;
-                        r.vx += h.vx; r.vy += h.vy; r.om += h.om;
+                        r.x[j] = -h.px; r.y[j] = -h.py; r.ph[j] = h.ph;
+                        r.vx[j] = -h.vpx; r.vy[j] = -h.vpy; r.om[j] = h.om;
                     }
                     if (nd & (2u << (2 * j))) {
                         float ex, ey;
@@ -635,25 +654,25 @@ __device__ __forceinline__ void block_substep_vjp(const SimConst& sc, const Quad
                         const CornerGrad h = corner_vjp(sc, s.x, s.y, cs, sn, s.vx, s.vy, s.om, bx, by, bc,
                                                         bs, bvx, bvy, bom, ex * sc.hs, ey * sc.hs, aFx,
                                                         aFy, aT, bFx, bFy, bT);
-                        c.x += h.ox; c.y += h.oy; c.ph += h.oph;
-                        c.vx += h.ovx; c.vy += h.ovy; c.om += h.oom;
-                        r.x += h.bx; r.y += h.by; r.ph += h.bph;
-                        r.vx += h.bvx; r.vy += h.bvy; r.om += h.bom;
+                        c.x[j] += h.ox; c.y[j] += h.oy; c.ph[j] += h.oph;
+                        c.vx[j] += h.ovx; c.vy[j] += h.ovy; c.om[j] += h.oom;
+                        r.x[j] += h.bx; r.y[j] += h.by; r.ph[j] += h.bph;
+                        r.vx[j] += h.bvx; r.vy[j] += h.bvy; r.om[j] += h.bom;
                     }
                 }
-                in.x += from_lane(lanes_sum<QL>(r.x), from);
-                in.y += from_lane(lanes_sum<QL>(r.y), from);
-                in.ph += from_lane(lanes_sum<QL>(r.ph), from);
-                in.vx += from_lane(lanes_sum<QL>(r.vx), from);
-                in.vy += from_lane(lanes_sum<QL>(r.vy), from);
-                in.om += from_lane(lanes_sum<QL>(r.om), from);
+                in.x += from_lane(block_sum<QL>(r.x), from);
+                in.y += from_lane(block_sum<QL>(r.y), from);
+                in.ph += from_lane(block_sum<QL>(r.ph), from);
+                in.vx += from_lane(block_sum<QL>(r.vx), from);
+                in.vy += from_lane(block_sum<QL>(r.vy), from);
+                in.om += from_lane(block_sum<QL>(r.om), from);
             }
-            in.x += lanes_sum<QL>(c.x);
-            in.y += lanes_sum<QL>(c.y);
-            in.ph += lanes_sum<QL>(c.ph);
-            in.vx += lanes_sum<QL>(c.vx);
-            in.vy += lanes_sum<QL>(c.vy);
-            in.om += lanes_sum<QL>(c.om);
+            in.x += block_sum<QL>(c.x);
+            in.y += block_sum<QL>(c.y);
+            in.ph += block_sum<QL>(c.ph);
+            in.vx += block_sum<QL>(c.vx);
+            in.vy += block_sum<QL>(c.vy);
+            in.om += block_sum<QL>(c.om);
         }
     }
     a.x += in.x - block_sum<QL>(dpx);

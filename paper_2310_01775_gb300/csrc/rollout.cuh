@@ -88,6 +88,13 @@ __device__ __forceinline__ void relax_action(const SimConst& sc, const float* th
     vv = a[M + 1];
 }
 
+// a b + c d with the first product fused.  Where a sum has two products, the
+// compiler may fuse either, and picks by context: written out, every kernel
+// and team width rounds alike (the dynamics amplify a last bit).
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) {
+    return fmaf(a, b, __fmul_rn(c, d));
+}
+
 __device__ __forceinline__ float sigmoidf_(float v) { return 1.f / (1.f + expf(-v)); }
 
 // ------------------------------- forces -------------------------------------
@@ -95,42 +102,7 @@ __device__ __forceinline__ float sigmoidf_(float v) { return 1.f / (1.f + expf(-
 // than the block's reach cannot touch it: the contact tests below return no
 // contact there, so callers may skip them.
 __device__ __forceinline__ bool out_of_reach(float dx, float dy, float reach2) {
-    return dx * dx + dy * dy > reach2;
-}
-
-// Force and torque on a square block (centre b, yaw via cph/sph, velocity v,
-// omega) from a kinematic disk pusher at p moving with vp (unweighted).
-__device__ __forceinline__ void disk_box(const SimConst& sc, float px, float py, float vpx,
-                                         float vpy, float bx, float by, float cph, float sph,
-                                         float vx, float vy, float om, float& fx, float& fy,
-                                         float& tq) {
-    fx = fy = tq = 0.f;
-    const float dx = px - bx, dy = py - by;
-    const float lx = cph * dx + sph * dy, ly = -sph * dx + cph * dy;
-    const float qx = fabsf(lx) - sc.hs, qy = fabsf(ly) - sc.hs;
-    const float sx = lx >= 0.f ? 1.f : -1.f, sy = ly >= 0.f ? 1.f : -1.f;
-    // outside: normalised clamped offset; inside: the axis of the larger q
-    // (selects, not branches: both are cheap and the chain stays straight)
-    const bool outside = qx > 0.f || qy > 0.f;
-    const float mx = fmaxf(qx, 0.f), my = fmaxf(qy, 0.f);
-    const float il = rsqrtf(fmaxf(mx * mx + my * my, 1e-30f));
-    const bool xa = qx >= qy;
-    const float sd = outside ? (mx * mx + my * my) * il : fmaxf(qx, qy);
-    const float nlx = outside ? sx * mx * il : (xa ? sx : 0.f);
-    const float nly = outside ? sy * my * il : (xa ? 0.f : sy);
-    const float delta = sc.r - sd;
-    if (!(delta > 0.f)) return;
-    const float nx = cph * nlx - sph * nly, ny = sph * nlx + cph * nly;
-    const float rx = px - sc.r * nx - bx, ry = py - sc.r * ny - by;
-    const float wx = vpx - (vx - om * ry), wy = vpy - (vy + om * rx);
-    const float vn = wx * nx + wy * ny;
-    const float fn = sc.k * delta - sc.c * vn;
-    if (!(fn > 0.f)) return;
-    const float tx = wx - vn * nx, ty = wy - vn * ny;
-    const float gt = sc.mu_c * fn * rsqrtf(tx * tx + ty * ty + sc.eps_t2);
-    fx = -fn * nx + gt * tx;
-    fy = -fn * ny + gt * ty;
-    tq = rx * fy - ry * fx;
+    return dot2(dx, dx, dy, dy) > reach2;
 }
 
 // Corner k (position, velocity) of one box against square B: force on the
@@ -140,23 +112,23 @@ __device__ __forceinline__ void corner_box(const SimConst& sc, float kx, float k
                                            float vx, float vy, float om, float& fx, float& fy) {
     fx = fy = 0.f;
     const float dx = kx - bx, dy = ky - by;
-    if (dx * dx + dy * dy > sc.corner_reach2) return;   // out of reach: no contact
-    const float lx = cph * dx + sph * dy, ly = -sph * dx + cph * dy;
+    if (out_of_reach(dx, dy, sc.corner_reach2)) return;   // no contact
+    const float lx = dot2(cph, dx, sph, dy), ly = dot2(cph, dy, -sph, dx);
     const float qx = fabsf(lx) - sc.hs, qy = fabsf(ly) - sc.hs;
     if (!(qx < 0.f && qy < 0.f)) return;
     const float sx = lx >= 0.f ? 1.f : -1.f, sy = ly >= 0.f ? 1.f : -1.f;
     const bool xa = qx >= qy;
     const float nlx = xa ? sx : 0.f, nly = xa ? 0.f : sy;
     const float delta = -(xa ? qx : qy);
-    const float nx = cph * nlx - sph * nly, ny = sph * nlx + cph * nly;
-    const float wx = kvx - (vx - om * dy), wy = kvy - (vy + om * dx);
-    const float vn = wx * nx + wy * ny;
-    const float fn = sc.k * delta - sc.c * vn;
+    const float nx = dot2(cph, nlx, -sph, nly), ny = dot2(sph, nlx, cph, nly);
+    const float wx = kvx - fmaf(-om, dy, vx), wy = kvy - fmaf(om, dx, vy);
+    const float vn = dot2(wx, nx, wy, ny);
+    const float fn = dot2(sc.k, delta, -sc.c, vn);
     if (!(fn > 0.f)) return;
-    const float tx = wx - vn * nx, ty = wy - vn * ny;
-    const float gt = sc.mu_c * fn * rsqrtf(tx * tx + ty * ty + sc.eps_t2);
-    fx = fn * nx - gt * tx;
-    fy = fn * ny - gt * ty;
+    const float tx = fmaf(-vn, nx, wx), ty = fmaf(-vn, ny, wy);
+    const float gt = sc.mu_c * fn * rsqrtf(dot2(tx, tx, ty, ty) + sc.eps_t2);
+    fx = dot2(fn, nx, -gt, tx);
+    fy = dot2(fn, ny, -gt, ty);
 }
 
 // State row of one particle: per block (x, y), (ph, vx), (vy, om).
@@ -174,102 +146,6 @@ __device__ __forceinline__ void load_state(const float2* src, Blocks<NB>& s) {
 __device__ __forceinline__ float wrapf(float e) { return atan2f(sinf(e), cosf(e)); }
 
 // ------------------------------ adjoint pieces -------------------------------
-// VJP of disk_box for the weighted force (w*f, w*torque).  Inputs gFx, gFy,
-// gT: adjoints of the block's force and torque.  Outputs are overwritten.
-struct DiskGrad {
-    float px, py, vpx, vpy, bx, by, ph, vx, vy, om, w;
-};
-__device__ __forceinline__ DiskGrad disk_box_vjp(const SimConst& sc, float px, float py,
-                                                 float vpx, float vpy, float bx, float by,
-                                                 float cph, float sph, float vx, float vy,
-                                                 float om, float w, float gFx, float gFy,
-                                                 float gT) {
-    DiskGrad g = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const float dx = px - bx, dy = py - by;
-    const float lx = cph * dx + sph * dy, ly = -sph * dx + cph * dy;
-    const float qx = fabsf(lx) - sc.hs, qy = fabsf(ly) - sc.hs;
-    const float sx = lx >= 0.f ? 1.f : -1.f, sy = ly >= 0.f ? 1.f : -1.f;
-    const bool outside = qx > 0.f || qy > 0.f;
-    const bool xa = qx >= qy;
-    const float mx = fmaxf(qx, 0.f), my = fmaxf(qy, 0.f);
-    const float il = rsqrtf(fmaxf(mx * mx + my * my, 1e-30f));
-    const float ln = (mx * mx + my * my) * il;
-    const float sd = outside ? ln : fmaxf(qx, qy);
-    const float nlx = outside ? sx * mx * il : (xa ? sx : 0.f);
-    const float nly = outside ? sy * my * il : (xa ? 0.f : sy);
-    const float delta = sc.r - sd;
-    if (!(delta > 0.f)) return g;
-    const float nx = cph * nlx - sph * nly, ny = sph * nlx + cph * nly;
-    const float rx = px - sc.r * nx - bx, ry = py - sc.r * ny - by;
-    const float wx = vpx - (vx - om * ry), wy = vpy - (vy + om * rx);
-    const float vn = wx * nx + wy * ny;
-    const float fn = sc.k * delta - sc.c * vn;
-    if (!(fn > 0.f)) return g;
-    const float tx = wx - vn * nx, ty = wy - vn * ny;
-    const float iden = rsqrtf(tx * tx + ty * ty + sc.eps_t2);
-    const float gt = sc.mu_c * fn * iden;
-    const float fx = -fn * nx + gt * tx, fy = -fn * ny + gt * ty;
-    // torque T = rx*(w fy) - ry*(w fx)
-    const float aFx = gFx - gT * ry, aFy = gFy + gT * rx;
-    float arx = gT * (w * fy), ary = -gT * (w * fx);
-    g.w = aFx * fx + aFy * fy;
-    const float afx = w * aFx, afy = w * aFy;
-    // f = -fn n + gt t
-    float afn = -(afx * nx + afy * ny);
-    float anx = -afx * fn, any = -afy * fn;
-    const float agt = afx * tx + afy * ty;
-    float atx = afx * gt, aty = afy * gt;
-    // gt = mu_c fn / den, den = sqrt(|t|^2 + eps^2)
-    afn += agt * sc.mu_c * iden;
-    const float aden = -agt * gt * iden;
-    atx += aden * tx * iden;
-    aty += aden * ty * iden;
-    // t = w - vn n
-    float awx = atx, awy = aty;
-    float avn = -(atx * nx + aty * ny);
-    anx -= atx * vn;
-    any -= aty * vn;
-    // fn = k delta - c vn
-    const float adelta = sc.k * afn;
-    avn -= sc.c * afn;
-    // vn = w . n
-    awx += avn * nx;
-    awy += avn * ny;
-    anx += avn * wx;
-    any += avn * wy;
-    // w = vp - v - om x r:  wx = vpx - vx + om ry, wy = vpy - vy - om rx
-    g.vpx = awx; g.vpy = awy;
-    g.vx = -awx; g.vy = -awy;
-    g.om = awx * ry - awy * rx;
-    ary += awx * om;
-    arx -= awy * om;
-    // r = p - r_p n - b
-    g.px = arx; g.py = ary;
-    anx -= sc.r * arx;
-    any -= sc.r * ary;
-    g.bx = -arx; g.by = -ary;
-    // n = R nl
-    const float anlx = cph * anx + sph * any;
-    const float anly = -sph * anx + cph * any;
-    float acph = anx * nlx + any * nly;
-    float asph = -anx * nly + any * nlx;
-    // delta = r - sd
-    const float asd = -adelta;
-    // outside: through the normalised clamped offset; inside: the chosen axis
-    const float aln = asd - (anlx * nlx + anly * nly) * il;
-    const float amx = (sx * anlx + aln * mx) * il, amy = (sy * anly + aln * my) * il;
-    const float aqx = outside ? (qx > 0.f ? amx : 0.f) : (xa ? asd : 0.f);
-    const float aqy = outside ? (qy > 0.f ? amy : 0.f) : (xa ? 0.f : asd);
-    const float alx = aqx * sx, aly = aqy * sy;
-    const float adx = cph * alx - sph * aly, ady = sph * alx + cph * aly;
-    acph += alx * dx + aly * dy;
-    asph += alx * dy - aly * dx;
-    g.px += adx; g.py += ady;
-    g.bx -= adx; g.by -= ady;
-    g.ph = -sph * acph + cph * asph;
-    return g;
-}
-
 // VJP of one corner test.  gO*/gB*: adjoints of the owner's / other box's
 // force and torque.  Returns the adjoints of both boxes' states.
 struct CornerGrad {
@@ -282,82 +158,69 @@ __device__ __forceinline__ CornerGrad corner_vjp(const SimConst& sc, float xo, f
                                                  float clx, float cly, float gOx, float gOy,
                                                  float gOT, float gBx, float gBy, float gBT) {
     CornerGrad g = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const float rlx = co * clx - so * cly, rly = so * clx + co * cly;
+    const float rlx = dot2(co, clx, -so, cly), rly = dot2(so, clx, co, cly);
     const float kx = xo + rlx, ky = yo + rly;
-    const float kvx = vxo - omo * rly, kvy = vyo + omo * rlx;
+    const float kvx = fmaf(-omo, rly, vxo), kvy = fmaf(omo, rlx, vyo);
     const float dx = kx - xb, dy = ky - yb;
-    if (dx * dx + dy * dy > sc.corner_reach2) return g;   // out of reach: no contact
-    const float lx = cb * dx + sb * dy, ly = -sb * dx + cb * dy;
+    if (out_of_reach(dx, dy, sc.corner_reach2)) return g;   // no contact
+    const float lx = dot2(cb, dx, sb, dy), ly = dot2(cb, dy, -sb, dx);
     const float qx = fabsf(lx) - sc.hs, qy = fabsf(ly) - sc.hs;
     if (!(qx < 0.f && qy < 0.f)) return g;
     const float sx = lx >= 0.f ? 1.f : -1.f, sy = ly >= 0.f ? 1.f : -1.f;
     const bool xa = qx >= qy;
     const float nlx = xa ? sx : 0.f, nly = xa ? 0.f : sy;
     const float delta = -(xa ? qx : qy);
-    const float nx = cb * nlx - sb * nly, ny = sb * nlx + cb * nly;
-    const float wx = kvx - (vxb - omb * dy), wy = kvy - (vyb + omb * dx);
-    const float vn = wx * nx + wy * ny;
-    const float fn = sc.k * delta - sc.c * vn;
+    const float nx = dot2(cb, nlx, -sb, nly), ny = dot2(sb, nlx, cb, nly);
+    const float wx = kvx - fmaf(-omb, dy, vxb), wy = kvy - fmaf(omb, dx, vyb);
+    const float vn = dot2(wx, nx, wy, ny);
+    const float fn = dot2(sc.k, delta, -sc.c, vn);
     if (!(fn > 0.f)) return g;
-    const float tx = wx - vn * nx, ty = wy - vn * ny;
-    const float iden = rsqrtf(tx * tx + ty * ty + sc.eps_t2);
+    const float tx = fmaf(-vn, nx, wx), ty = fmaf(-vn, ny, wy);
+    const float iden = rsqrtf(dot2(tx, tx, ty, ty) + sc.eps_t2);
     const float gt = sc.mu_c * fn * iden;
-    const float fx = fn * nx - gt * tx, fy = fn * ny - gt * ty;
+    const float fx = dot2(fn, nx, -gt, tx), fy = dot2(fn, ny, -gt, ty);
     // owner: +f, torque rl x f; other: -f, torque -(d x f)
-    const float afx = gOx - gBx - gOT * rly + gBT * dy;
-    const float afy = gOy - gBy + gOT * rlx - gBT * dx;
-    float arlx = gOT * fy, arly = -gOT * fx;
-    float adx = -gBT * fy, ady = gBT * fx;
+    const float afx = fmaf(gBT, dy, fmaf(-gOT, rly, gOx - gBx));
+    const float afy = fmaf(-gBT, dx, fmaf(gOT, rlx, gOy - gBy));
     // f = fn n - gt t
-    float afn = afx * nx + afy * ny;
-    float anx = afx * fn, any = afy * fn;
-    const float agt = -(afx * tx + afy * ty);
-    float atx = -afx * gt, aty = -afy * gt;
-    afn += agt * sc.mu_c * iden;
+    float afn = dot2(afx, nx, afy, ny);
+    const float agt = -dot2(afx, tx, afy, ty);
+    afn = fmaf(agt * sc.mu_c, iden, afn);
     const float aden = -agt * gt * iden;
-    atx += aden * tx * iden;
-    aty += aden * ty * iden;
-    float awx = atx, awy = aty;
-    float avn = -(atx * nx + aty * ny);
-    anx -= atx * vn;
-    any -= aty * vn;
+    const float atx = dot2(aden * tx, iden, -afx, gt), aty = dot2(aden * ty, iden, -afy, gt);
+    float avn = -dot2(atx, nx, aty, ny);
+    float anx = dot2(afx, fn, -atx, vn), any = dot2(afy, fn, -aty, vn);
     const float adelta = sc.k * afn;
-    avn -= sc.c * afn;
-    awx += avn * nx;
-    awy += avn * ny;
-    anx += avn * wx;
-    any += avn * wy;
+    avn = fmaf(-sc.c, afn, avn);
+    const float awx = fmaf(avn, nx, atx), awy = fmaf(avn, ny, aty);
+    anx = fmaf(avn, wx, anx);
+    any = fmaf(avn, wy, any);
     // w = kv - vb - omb x d:  wx = kvx - vxb + omb dy, wy = kvy - vyb - omb dx
     const float akvx = awx, akvy = awy;
     g.bvx = -awx; g.bvy = -awy;
-    g.bom = awx * dy - awy * dx;
-    ady += awx * omb;
-    adx -= awy * omb;
+    g.bom = dot2(awx, dy, -awy, dx);
     // n = R_b nl (nl constant)
-    float acb = anx * nlx + any * nly;
-    float asb = -anx * nly + any * nlx;
+    float acb = dot2(anx, nlx, any, nly);
+    float asb = dot2(any, nlx, -anx, nly);
     // delta = -(q on the axis), q = |l| - hs
     const float aqx = xa ? -adelta : 0.f, aqy = xa ? 0.f : -adelta;
     const float alx = aqx * sx, aly = aqy * sy;
-    adx += cb * alx - sb * aly;
-    ady += sb * alx + cb * aly;
-    acb += alx * dx + aly * dy;
-    asb += alx * dy - aly * dx;
+    const float adx = dot2(-awy, omb, -gBT, fy) + dot2(cb, alx, -sb, aly);
+    const float ady = dot2(awx, omb, gBT, fx) + dot2(sb, alx, cb, aly);
+    acb += dot2(alx, dx, aly, dy);
+    asb += dot2(alx, dy, -aly, dx);
     // d = k - b
-    float akx = adx, aky = ady;
     g.bx = -adx; g.by = -ady;
     // kv = vo + omo x rl
     g.ovx = akvx; g.ovy = akvy;
-    g.oom = -akvx * rly + akvy * rlx;
-    arly -= akvx * omo;
-    arlx += akvy * omo;
+    g.oom = dot2(akvy, rlx, -akvx, rly);
     // k = o + rl
-    g.ox = akx; g.oy = aky;
-    arlx += akx;
-    arly += aky;
-    const float aco = arlx * clx + arly * cly, aso = -arlx * cly + arly * clx;
-    g.oph = -so * aco + co * aso;
-    g.bph = -sb * acb + cb * asb;
+    g.ox = adx; g.oy = ady;
+    const float arlx = dot2(akvy, omo, gOT, fy) + adx;
+    const float arly = dot2(-akvx, omo, -gOT, fx) + ady;
+    const float aco = dot2(arlx, clx, arly, cly), aso = dot2(arly, clx, -arlx, cly);
+    g.oph = dot2(co, aso, -so, aco);
+    g.bph = dot2(cb, asb, -sb, acb);
     return g;
 }
 
