@@ -162,7 +162,9 @@ stamp_status stamp_svgd_step(stamp_problem* prob, float* theta, const float* gra
  *
  * stamp_set_particle_offset: later rollouts of this problem treat their row
  * r as particle particle0 + r of the full set (its Gumbel draws, Eq.
- * gamma_map); 0 (the default) for an unsharded problem. */
+ * gamma_map); 0 is the default.  A problem that was given an offset (0 too: call
+ * it on the first shard as well) is one of a set of max_particles particles: the
+ * automatic reverse sweep is picked by that size, as for the whole set. */
 stamp_status stamp_set_particle_offset(stamp_problem* prob, int particle0);
 /* The update of rows [row0, row0 + rows) of an N-particle set:
  *   theta_all, grad_all: device N x D, the gathered particles and

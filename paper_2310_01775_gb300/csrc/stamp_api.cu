@@ -65,6 +65,7 @@ struct stamp_problem {
     unsigned long long* dropped = nullptr;
     // global index of the first particle of later calls (a shard of a larger set)
     int particle0 = 0;
+    bool shard = false;   // an offset was set: calls hold a part of a set of max_n particles
     // last forward
     bool have_tape = false;
     int last_n = 0, last_iter = 0, last_hard = 0, last_particle0 = 0;
@@ -181,10 +182,11 @@ stamp_status check_dev(const void* ptr, const char* name, bool allow_null = fals
 // the serial chain), the time-parallel sweep 39 at 128 particles, 67 at 1024,
 // 105 at 2048 and 163 at 3072, where the Jacobians' extra arithmetic no longer
 // comes for free (H = 1 or 2: 33 to 35 us against 34 at 1600, 37 at 2048, 52 at 3072).
+// A shard goes by the size of its whole set: the two sweeps round differently.
 bool time_parallel(const stamp_problem* p, int N) {
     if (!p->pit_ok || p->adj_mode == STAMP_ADJ_SEQUENTIAL || p->adj_mode == STAMP_ADJ_REPLAY)
         return false;
-    return p->adj_mode == STAMP_ADJ_TIME_PARALLEL || N <= kTimeParallelMaxN;
+    return p->adj_mode == STAMP_ADJ_TIME_PARALLEL || (p->shard ? p->max_n : N) <= kTimeParallelMaxN;
 }
 
 // The sweep a call with N particles runs: time-parallel (above), else on the
@@ -778,6 +780,7 @@ stamp_status stamp_set_particle_offset(stamp_problem* p, int particle0) {
     if (!p) return fail(STAMP_EINVAL, "NULL problem");
     if (particle0 < 0) return fail(STAMP_EINVAL, "particle0 must be >= 0");
     p->particle0 = particle0;
+    p->shard = true;
     return STAMP_OK;
 }
 
