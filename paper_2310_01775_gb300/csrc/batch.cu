@@ -564,8 +564,7 @@ stamp_status stamp_batch_create(const stamp_problem_desc* physics, const stamp_i
         const int D = d.H * (4 * d.n_blocks + 2);
         b->D[g] = D;
         b->max_D = std::max(b->max_D, D);
-        int shares, jc;
-        stamp::phi_batch_plan(d.N, &shares, &jc);
+        const int shares = stamp::phi_batch_shares(d.N);
         b->elem0.push_back(e);
         e += al32((long long)d.N * D);
         b->part0.push_back(p);
@@ -641,7 +640,7 @@ stamp_status stamp_batch_create(const stamp_problem_desc* physics, const stamp_i
             const long long pairs = (long long)d.N * (d.N - 1) / 2;
             s.med_ctas = (int)std::max(1LL, std::min<long long>(kMedCtasMax, pairs / 8192));
             s.med_ctas = std::min(s.med_ctas, std::max(d.N - 1, 1));
-            stamp::phi_batch_plan(d.N, &s.shares, &s.j_chunk);
+            s.shares = stamp::phi_batch_shares(d.N);
             s.gid = g;
             s.elem0 = b->elem0[g];
             nv[g] = d.N;

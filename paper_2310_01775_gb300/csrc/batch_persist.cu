@@ -165,14 +165,10 @@ __device__ __forceinline__ void adam_chunk(const PersistArgs& p, const SvgdInst&
         for (int u = 0; u < U; ++u) {
             const long long loc = l0 + u * kPersistThreads, t = s.elem0 + loc;
             if (loc >= e0) continue;
-            const float gr = -phi[u];
-            const float mt = 0.9f * m0[u] + 0.1f * gr;
-            const float vt = 0.999f * v0[u] + 0.001f * gr * gr;
-            const float th = t0[u] - p.lr * (mt / bc1) / (sqrtf(vt / bc2) + 1e-8f);
-            p.m[t] = mt;
-            p.v[t] = vt;
-            p.theta[t] = th;
-            if (!isfinite(th) || !isfinite(gr)) atomicOr(p.flag, 1);
+            if (!adam_update(-phi[u], p.lr, bc1, bc2, m0[u], v0[u], t0[u])) atomicOr(p.flag, 1);
+            p.m[t] = m0[u];
+            p.v[t] = v0[u];
+            p.theta[t] = t0[u];
         }
     }
 }
@@ -182,15 +178,15 @@ __device__ __forceinline__ bool run_phi(const PersistArgs& p, const SvgdInst& s,
     switch (p.dp) {
         case 3:
             return phi_body<3, kPersistWarps, 1>(s.theta, s.grad, s.N, s.D, s.d2, s.h, s.part,
-                                              s.j_chunk, p.flag, rblock, share, nullptr,
+                                              s.shares, p.flag, rblock, share, nullptr,
                                               kWaitLimit, false, 0, s.N);
         case 6:
             return phi_body<6, kPersistWarps, 1>(s.theta, s.grad, s.N, s.D, s.d2, s.h, s.part,
-                                              s.j_chunk, p.flag, rblock, share, nullptr,
+                                              s.shares, p.flag, rblock, share, nullptr,
                                               kWaitLimit, false, 0, s.N);
         default:
             return phi_body<9, kPersistWarps, 1>(s.theta, s.grad, s.N, s.D, s.d2, s.h, s.part,
-                                              s.j_chunk, p.flag, rblock, share, nullptr,
+                                              s.shares, p.flag, rblock, share, nullptr,
                                               kWaitLimit, false, 0, s.N);
     }
 }
@@ -324,7 +320,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
 
 size_t persist_smem(int max_D, int seg_warp) {
     const int dp = persist_dp(max_D);
-    const size_t phi = phi_smem(max_D, dp, kPersistWarps, kR);
+    const size_t phi = phi_smem(max_D, dp, kPersistWarps);
     const size_t pw = 2 * kTile * (size_t)(max_D + 1) * sizeof(float);
     const size_t seg = (size_t)kPersistWarps * seg_warp * sizeof(float2);
     size_t m = phi > pw ? phi : pw;

@@ -228,7 +228,7 @@ struct SvgdInst {
     int N, D;
     int nt;                 // pairwise tiles per side
     int med_ctas;           // CTAs of each median-digit pass
-    int shares, j_chunk;    // Stein-sum split (as for one problem of N particles)
+    int shares;             // Stein-sum split (as for one problem of N particles)
     int gid;                // index in the batch (active flags)
     long long elem0;        // first element of the instance in the concatenated particles
 };
@@ -255,7 +255,7 @@ struct InstItem {
 cudaError_t launch_init_theta_batch(const InstItem* items, int n, long long n_elem, cudaStream_t st);
 cudaError_t launch_topk_batch(const InstItem* items, int n, int max_n, cudaStream_t st);
 // The single-problem Stein-sum split for N particles, and rows per phi CTA.
-void phi_batch_plan(int N, int* shares, int* j_chunk);
+int phi_batch_shares(int N);
 int phi_rows_per_block();
 cudaError_t launch_topk(const float* theta, const float* cost, int N, const SimConst& sc, int k,
                         int* topk_out, cudaStream_t st);

@@ -1,3 +1,4 @@
+#include <climits>
 // Stein update of Algorithm 1 (Eq. svgd with unit weights), its median
 // bandwidth, Adam, the initial particles and the final distinct-plan top-k.
 //
@@ -164,17 +165,20 @@ __global__ void __launch_bounds__(256) median_digit_batch_kernel(const SvgdInst*
 }
 
 
-template <int DP, int R>
-__global__ void __launch_bounds__(kW * 32) phi_kernel(const float* __restrict__ theta,
+// CTAs per SM that the registers are kept to (GB300, N = 3000, D = 60: 92 -> 87 us with
+// the bound, N = 4096, D = 144: 392 -> 383).
+constexpr int phi_resident(int DP) { return DP <= 3 ? 4 : DP <= 4 ? 3 : 2; }
+template <int DP>
+__global__ void __launch_bounds__(kW * 32, phi_resident(DP)) phi_kernel(const float* __restrict__ theta,
                                                       const float* __restrict__ grad, int N, int D,
                                                       const float* __restrict__ d2,
                                                       const float* __restrict__ h_dev,
-                                                      float* __restrict__ part, int j_chunk,
+                                                      float* __restrict__ part, int shares,
                                                       int* err, const float* __restrict__ wn,
                                                       unsigned wait_limit, int skip_first, int row0,
                                                       int rows) {
     after_previous();
-    phi_body<DP, kW, 8, R>(theta, grad, N, D, d2, h_dev, part, j_chunk, err, blockIdx.x, blockIdx.y, wn,
+    phi_body<DP, kW, 8>(theta, grad, N, D, d2, h_dev, part, shares, err, blockIdx.x, blockIdx.y, wn,
                            wait_limit, skip_first != 0, row0, rows);
 }
 
@@ -187,7 +191,7 @@ __global__ void __launch_bounds__(kW * 32) phi_batch_kernel(const SvgdInst* __re
     const int4 it = items[blockIdx.x];
     const SvgdInst& g = inst[it.x];
     if (!active[g.gid]) return;
-    phi_body<DP>(g.theta, g.grad, g.N, g.D, g.d2, g.h, g.part, g.j_chunk, err, it.y, it.z, nullptr,
+    phi_body<DP>(g.theta, g.grad, g.N, g.D, g.d2, g.h, g.part, g.shares, err, it.y, it.z, nullptr,
                  kWaitLimit, false, 0, g.N);
 }
 
@@ -204,14 +208,11 @@ __global__ void adam_kernel(float* __restrict__ theta, const float* __restrict__
     float phi = part[t];
     for (int q = 1; q < shares; ++q) phi += part[(size_t)q * n + t];
     if (phi_out) phi_out[t] = phi;
-    const float g = -phi;
-    const float mt = 0.9f * m[t] + 0.1f * g;
-    const float vt = 0.999f * v[t] + 0.001f * g * g;
-    const float th = theta[t] - lr * (mt / bc1) / (sqrtf(vt / bc2) + 1e-8f);
+    float mt = m[t], vt = v[t], th = theta[t];
+    if (!adam_update(-phi, lr, bc1, bc2, mt, vt, th)) atomicOr(flag, 1);
     m[t] = mt;
     v[t] = vt;
     theta[t] = th;
-    if (!isfinite(th) || !isfinite(g)) atomicOr(flag, 1);
 }
 
 // Batched Adam over the concatenated particles of all instances: element t
@@ -236,15 +237,11 @@ __global__ void adam_batch_kernel(float* __restrict__ theta, float* __restrict__
     float phi = part[loc];
     for (int q = 1; q < g.shares; ++q) phi += part[(size_t)q * ne + loc];
     const float2 b12 = bc[*step_dev + 1];
-    const float bc1 = b12.x, bc2 = b12.y;
-    const float gr = -phi;
-    const float mt = 0.9f * m[t] + 0.1f * gr;
-    const float vt = 0.999f * v[t] + 0.001f * gr * gr;
-    const float th = theta[t] - lr * (mt / bc1) / (sqrtf(vt / bc2) + 1e-8f);
+    float mt = m[t], vt = v[t], th = theta[t];
+    if (!adam_update(-phi, lr, b12.x, b12.y, mt, vt, th)) atomicOr(flag, 1);
     m[t] = mt;
     v[t] = vt;
     theta[t] = th;
-    if (!isfinite(th) || !isfinite(gr)) atomicOr(flag, 1);
 }
 
 // A whole Stein step of at most kSmallN particles in one CTA: distances, their
@@ -263,7 +260,6 @@ __global__ void __launch_bounds__(1024) small_step_kernel(
     float* T = ssm;
     float* G = T + E * ld;
     __shared__ float K[E][E + 1];   // d2, then the kernel values
-    __shared__ float S[E][E / 32];  // a share's kernel values summed
     const int tid = threadIdx.x;
     for (int t = tid; t < N * D; t += 1024) {
         T[(t / D) * ld + t % D] = theta[t];
@@ -309,22 +305,15 @@ __global__ void __launch_bounds__(1024) small_step_kernel(
         *h_dev = h;
         if (h_out) *h_out = h;
     }
-    const float inv_h = 1.f / h, two_h = 2.f * inv_h;
-    for (int t = tid; t < E * E; t += 1024) {   // a warp: a row and share
-        const int i = t / E, j = t % E;
+    const float inv_h = 1.f / h, m2h = -2.f * inv_h;
+    for (int t = tid; t < N * N; t += 1024) {
+        const int i = t / N, j = t % N;
         float k = 0.f;
-        if (i < N && j < N && i != j) {
+        if (i != j) {
             k = expf(-K[i][j] * inv_h);
             if (wn) k *= wn[j];
         }
         K[i][j] = k;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(~0u, k, o);
-        if (tid % 32 == 0) S[i][j / 32] = k;
-    }
-    for (int t = tid; t < N * D; t += 1024) {   // u in place of g
-        const int j = t / D, d = t % D;
-        G[j * ld + d] = fmaf(-two_h, T[j * ld + d] - T[d], G[j * ld + d]);
     }
     __syncthreads();
     const float inv_n = wn ? 1.f : 1.f / (float)N;
@@ -334,20 +323,18 @@ __global__ void __launch_bounds__(1024) small_step_kernel(
         float phi = 0.f;
         for (int j0 = 0; j0 < N; j0 += kTJ) {
             float a = 0.f;
-            for (int j = j0; j < min(N, j0 + kTJ); ++j) a = fmaf(K[i][j], G[j * ld + d], a);
-            a = fmaf(two_h * (ti - T[d]), S[i][j0 / kTJ], a);
-            if (self != 0.f && i / kTJ == j0 / kTJ) a = fmaf(self, grad[t], a);
-            phi = j0 ? phi + a * inv_n : a * inv_n;
+            for (int j = j0; j < min(N, j0 + kTJ); ++j)
+                a = fmaf(K[i][j], fmaf(m2h, T[j * ld + d] - ti, G[j * ld + d]), a);
+            if (self != 0.f && i / kTJ == j0 / kTJ) a = fmaf(self, G[i * ld + d], a);
+            const float share = __fmul_rn(a, inv_n);
+            phi = j0 ? __fadd_rn(phi, share) : share;
         }
         if (phi_out) phi_out[t] = phi;
-        const float g = -phi;
-        const float mt = 0.9f * m[t] + 0.1f * g;
-        const float vt = 0.999f * v[t] + 0.001f * g * g;
-        const float th = ti - lr * (mt / bc1) / (sqrtf(vt / bc2) + 1e-8f);
+        float mt = m[t], vt = v[t], th = ti;
+        if (!adam_update(-phi, lr, bc1, bc2, mt, vt, th)) atomicOr(flag, 1);
         m[t] = mt;
         v[t] = vt;
         theta[t] = th;
-        if (!isfinite(th) || !isfinite(g)) atomicOr(flag, 1);
     }
 }
 
@@ -472,65 +459,43 @@ __global__ void init_theta_batch_kernel(const InstItem* __restrict__ items, int 
     if (loc < (long long)it.N * it.H * (it.M + 2)) it.theta[loc] = 2.f * u23(sm64(it.key, (uint64_t)loc)) - 1.f;
 }
 
-template <int DP, int R>
-cudaError_t phi_launch_rows(const float* theta, const float* grad, int N, int D, const float* d2,
-                            const float* h_dev, float* part, int shares, int j_chunk, int* err,
-                            const float* wn, unsigned wait_limit, int skip_first, int row0, int rows,
-                            bool chained, cudaStream_t st) {
-    const size_t smem = phi_smem(D, DP, kW, R);
+template <int DP>
+cudaError_t phi_launch(const float* theta, const float* grad, int N, int D, const float* d2,
+                       const float* h_dev, float* part, int shares, int* err, const float* wn,
+                       unsigned wait_limit, int skip_first, int row0, int rows, bool chained,
+                       cudaStream_t st) {
+    const size_t smem = phi_smem(D, DP, kW);
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(phi_kernel<DP, R>,
+        cudaError_t e = cudaFuncSetAttribute(phi_kernel<DP>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    const int per_cta = kW * R;
+    const int per_cta = kW * kR;
     const dim3 grid((rows + per_cta - 1) / per_cta, shares);
     if (chained)
-        return launch_after(phi_kernel<DP, R>, grid, kW * 32, smem, st, theta, grad, N, D, d2, h_dev, part, j_chunk,
+        return launch_after(phi_kernel<DP>, grid, kW * 32, smem, st, theta, grad, N, D, d2, h_dev, part, shares,
                             err, wn, wait_limit, skip_first, row0, rows);
-    phi_kernel<DP, R><<<grid, kW * 32, smem, st>>>(theta, grad, N, D, d2, h_dev, part, j_chunk, err, wn, wait_limit,
+    phi_kernel<DP><<<grid, kW * 32, smem, st>>>(theta, grad, N, D, d2, h_dev, part, shares, err, wn, wait_limit,
                                                    skip_first, row0, rows);
     return cudaGetLastError();
 }
-// The split of the Stein sum of N particles over j-shares and the rows per
-// warp; a function of N alone, so that a shard of the rows sums as all do (a
-// row's sum depends on the shares, not on the rows per warp).  Eight rows per
-// warp (two resident CTAs of 64 rows per SM) once eight shares of them give 1.6
-// CTAs per SM; there the shares are the count, at most max_shares, that fills
-// whole waves best.  Below that four rows per warp and about four CTAs per SM.
-void phi_plan(int N, int max_shares, int* rows_per_warp, int* shares, int* j_chunk) {
-    const int sms = sm_count(), b8 = (N + 8 * kW - 1) / (8 * kW), b4 = (N + 4 * kW - 1) / (4 * kW);
-    int want;
-    if (10 * b8 * kMaxShares >= 16 * sms) {
-        *rows_per_warp = 8;
-        want = 1;
-        double best = 0.0;
-        for (int s = 1; s <= max_shares; ++s) {
-            const int ctas = b8 * s, waves = (ctas + 2 * sms - 1) / (2 * sms);
-            const double fill = (double)ctas / ((double)waves * 2 * sms);
-            if (fill > best + 0.01) {
-                best = fill;
-                want = s;
-            }
+// Shares of the Stein sum of N particles: the tiles of the busiest SM, CTAs times
+// tiles of the longest share, are the time (GB300, D = 108, N = 6001: 2.3 to 2.5 us a tile
+// at any split, 561 us at 4 shares, 618 at 5); among equal ones the more CTAs, which
+// hide more latency.  A function of N alone, so that a shard of the rows sums as
+// all do; at most max_shares.
+int phi_plan(int N, int max_shares) {
+    const int sms = sm_count(), rows = (N + kR * kW - 1) / (kR * kW), tiles = (N + kTJ - 1) / kTJ;
+    int best = 1;
+    long long least = LLONG_MAX;
+    for (int s = 1; s <= max_shares && s <= tiles; ++s) {
+        const long long t = (long long)((rows * s + sms - 1) / sms) * ((tiles + s - 1) / s);
+        if (t <= least) {
+            least = t;
+            best = s;
         }
-    } else {
-        *rows_per_warp = 4;
-        want = (4 * sms + b4 - 1) / b4;
-        want = want < 1 ? 1 : (want > max_shares ? max_shares : want);
     }
-    // the shares start on kTJ-row boundaries (16-byte aligned TMA sources)
-    *j_chunk = ((N + want - 1) / want + kTJ - 1) / kTJ * kTJ;
-    *shares = (N + *j_chunk - 1) / *j_chunk;
-}
-template <int DP>
-cudaError_t phi_launch(const float* theta, const float* grad, int N, int D, const float* d2,
-                       const float* h_dev, float* part, int shares, int j_chunk, int* err,
-                       const float* wn, unsigned wait_limit, int skip_first, int row0, int rows,
-                       bool r8, bool chained, cudaStream_t st) {
-    return r8 ? phi_launch_rows<DP, 8>(theta, grad, N, D, d2, h_dev, part, shares, j_chunk, err, wn,
-                                       wait_limit, skip_first, row0, rows, chained, st)
-              : phi_launch_rows<DP, 4>(theta, grad, N, D, d2, h_dev, part, shares, j_chunk, err, wn,
-                                       wait_limit, skip_first, row0, rows, chained, st);
+    return best;
 }
 
 }  // namespace
@@ -576,20 +541,18 @@ cudaError_t launch_phi_rows(const float* theta, const float* grad, int N, int D,
     // TMA bulk copies need 16-byte aligned sources
     if ((reinterpret_cast<uintptr_t>(theta) | reinterpret_cast<uintptr_t>(grad)) & 15u)
         return cudaErrorMisalignedAddress;
-    int j_chunk, rpw;
-    phi_plan(N, max_shares, &rpw, shares, &j_chunk);
-    const bool r8 = rpw == 8;
+    *shares = phi_plan(N, max_shares);
     const unsigned limit = s.wait_limit ? s.wait_limit : kWaitLimit;
     const int dp = (D + 31) / 32;
     switch (dp) {
-        case 1: return phi_launch<1>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
-        case 2: return phi_launch<2>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
-        case 3: return phi_launch<3>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
-        case 4: return phi_launch<4>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
+        case 1: return phi_launch<1>(theta, grad, N, D, s.d2, s.h, part, *shares, s.err, wn, limit, s.skip_first_copy, row0, rows, s.chained, st);
+        case 2: return phi_launch<2>(theta, grad, N, D, s.d2, s.h, part, *shares, s.err, wn, limit, s.skip_first_copy, row0, rows, s.chained, st);
+        case 3: return phi_launch<3>(theta, grad, N, D, s.d2, s.h, part, *shares, s.err, wn, limit, s.skip_first_copy, row0, rows, s.chained, st);
+        case 4: return phi_launch<4>(theta, grad, N, D, s.d2, s.h, part, *shares, s.err, wn, limit, s.skip_first_copy, row0, rows, s.chained, st);
         case 5: case 6:
-            return phi_launch<6>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
+            return phi_launch<6>(theta, grad, N, D, s.d2, s.h, part, *shares, s.err, wn, limit, s.skip_first_copy, row0, rows, s.chained, st);
         case 7: case 8: case 9:
-            return phi_launch<9>(theta, grad, N, D, s.d2, s.h, part, *shares, j_chunk, s.err, wn, limit, s.skip_first_copy, row0, rows, r8, s.chained, st);
+            return phi_launch<9>(theta, grad, N, D, s.d2, s.h, part, *shares, s.err, wn, limit, s.skip_first_copy, row0, rows, s.chained, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -639,16 +602,13 @@ cudaError_t launch_median_digit_batch(const SvgdInst* inst, const int2* items, i
     return cudaGetLastError();
 }
 
-void phi_batch_plan(int N, int* shares, int* j_chunk) {
-    int rpw;
-    phi_plan(N, kMaxShares, &rpw, shares, j_chunk);
-}
+int phi_batch_shares(int N) { return phi_plan(N, kMaxShares); }
 int phi_rows_per_block() { return kW * kR; }
 
 template <int DP>
 cudaError_t phi_batch_launch(const SvgdInst* inst, const int4* items, int n_items, int max_D,
                              const int* active, int* err, cudaStream_t st) {
-    const size_t smem = phi_smem(max_D, DP, kW, kR);
+    const size_t smem = phi_smem(max_D, DP, kW);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(phi_batch_kernel<DP>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -260,6 +260,17 @@ __device__ __forceinline__ void median_digit_body(int N, int dg, const float* __
     }
 }
 
+// One Adam update (Kingma & Ba 2015) with gradient g of an element; false if it
+// is not finite.  Which product of a sum is fused is written out: the kernels that
+// move particles agree to the bit.
+__device__ __forceinline__ bool adam_update(float g, float lr, float bc1, float bc2, float& m, float& v,
+                                            float& th) {
+    m = fmaf(0.9f, m, __fmul_rn(0.1f, g));
+    v = fmaf(0.999f, v, __fmul_rn(__fmul_rn(0.001f, g), g));
+    th = __fsub_rn(th, lr * (m / bc1) / (sqrtf(v / bc2) + 1e-8f));
+    return isfinite(th) && isfinite(g);
+}
+
 // TMA bulk copies and mbarriers: the shared helpers of async_copy.cuh, whose
 // kWaitLimit bounds every wait (then the error flag).
 using async::fence_async_shared;
@@ -271,58 +282,63 @@ using async::mbar_try_wait;
 using async::tma_load_1d;
 
 // phi_i = (1/N) sum_j [k_ij g_j + (2/h) k_ij (theta_i - theta_j)], k_ij = exp(-d2_ij/h).
-// With u_j = g_j - (2/h) (theta_j - c), c = theta_0, and S_i = sum_{j != i} k_ij,
-//   N phi_i = g_i + sum_{j != i} k_ij u_j + (2/h) (theta_i - c) S_i:
-// one multiply-add per (i, j, column) instead of a subtraction and two.  c is
-// one of the particles, so theta - c is of the size of their distances (no
-// offset common to all particles is multiplied by the kernel), and the term
-// j = i, whose parts would only cancel, is left out of the sums.
+// The term j = i, whose difference is 0, is added last: it is often the largest,
+// and the other N - 1 are then rounded at their own size.  theta_i - theta_j is
+// formed pair by pair: (theta_i - c) sum k - sum k (theta_j - c) takes one multiply-add
+// instead of three operations, but cancels wherever theta_i - c is large beside
+// sqrt(h) -- a particle far from c, a second mode -- for any c common to the rows
+// of a CTA.  Error of phi against 64 bits, of its norm (512 particles, D = 84; in
+// brackets that form with c = theta_0): uniform 1.6e-7 (1.6e-7), a cloud of sigma 0.01
+// with particle 0 three away in every column 3.2e-7 (2.0e-5), two clouds of sigma
+// 0.01 8.7e-8 (1.0e-5).
 //
-// A warp owns R rows; lane l owns columns l, l+32, ...  (DP slots).  The j
+// A warp owns kR rows; lane l owns columns l, l+32, ...  (DP slots).  The j
 // range is walked in tiles of kTJ rows of theta and grad, which are
 // contiguous in HBM: one thread streams each tile into one of two shared
 // memory stages with 1-D TMA bulk copies (mbarrier completion), one tile
-// ahead of the compute; the CTA turns the grad tile into u in place.  The d2
-// values of the next tile are prefetched into registers; k_ij for the warp's
-// rows is R/4 float4 per j (broadcast loads).  The shared-memory loads per j
-// (DP + R/4) against R DP multiply-adds, and the instructions around them,
-// bound it: two rows' multiply-adds per instruction (f32x2), R = 8 where that
-// still leaves enough CTAs.  GB300: 72 -> 38 us at N = 2048, D = 84, 672 -> 302 us
-// at N = 6001, D = 108 (FP32 pipe 33% busy).  Error of phi against 64 bits, theta
-// uniform in (-1, 1): 3.0e-7 (direct form 3.2e-7) and 7.0e-7 (7.8e-7).
+// ahead of the compute.  The d2 values of the next tile are prefetched into
+// registers; k_ij for the warp's rows is one float4 per j (a broadcast load).
+// What bounds it is the FP32 pipe: a fused multiply-add of three different
+// registers issues every 1.63 cycles, an addition every 1.05 (measured alone), and
+// rows are taken in pairs (f32x2) to leave issue slots for the rest.  GB300: 63 us
+// at N = 2048, D = 84 and 563 us at N = 6001, D = 108 (one row per instruction, two sums per
+// row and column: 73 and 674; the form with a common centre, whose error is above: 40 and
+// 305).
 constexpr int kR = 4, kW = 8, kTJ = 32;   // rows per warp, warps per CTA, j rows per tile
 __host__ __device__ constexpr int phi_stage_floats(int D, int DP) {
     return ((kTJ * D + 32 * DP) + 3) / 4 * 4;   // per array, 16-byte multiple
 }
-// Dynamic shared memory of a CTA of KW warps with R rows each.
-__host__ __device__ constexpr size_t phi_smem(int D, int DP, int KW, int R) {
+// Dynamic shared memory of a CTA of KW warps.
+__host__ __device__ constexpr size_t phi_smem(int D, int DP, int KW) {
     return (size_t)4 * phi_stage_floats(D, DP) * sizeof(float) +
-           (size_t)KW * kTJ * R * sizeof(float) + 2 * sizeof(uint64_t);
+           (size_t)KW * kTJ * kR * sizeof(float) + 2 * sizeof(uint64_t);
 }
 // KW warps per CTA (kW in the per-piece kernels), the j loop unrolled
 // UNROLL times; false if a copy never
 // landed (error bit 2 set).  A CTA that goes on to other work may reuse the
 // shared memory: the mbarriers are invalidated on the way out.
-template <int DP, int KW = kW, int UNROLL = 8, int R = kR>
+template <int DP, int KW = kW, int UNROLL = 8>
 __device__ __forceinline__ bool phi_body(const float* __restrict__ theta,
                                          const float* __restrict__ grad, int N, int D,
                                          const float* __restrict__ d2,
                                          const float* __restrict__ h_dev, float* __restrict__ part,
-                                         int j_chunk, int* err, int rblock, int share,
+                                         int shares, int* err, int rblock, int share,
                                          const float* __restrict__ wn, unsigned wait_limit,
                                          bool skip_first, int row0, int rows) {
     extern __shared__ __align__(128) float sm[];
-    constexpr int R4 = R / 4;
+    constexpr int R = kR;
     const int sf = phi_stage_floats(D, DP);
     // stage s: theta tile at sm + 2*s*sf, grad tile right after it
-    float4* Ks = reinterpret_cast<float4*>(sm + 4 * sf);              // KW x kTJ x R4
-    uint64_t* bar = reinterpret_cast<uint64_t*>(Ks + KW * kTJ * R4);   // 2 stages
+    float4* Ks = reinterpret_cast<float4*>(sm + 4 * sf);              // KW x kTJ
+    uint64_t* bar = reinterpret_cast<uint64_t*>(Ks + KW * kTJ);       // 2 stages
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // rows [row0, row0 + rows) of phi (all N: row0 = 0, rows = N)
     const int ib = row0 + (rblock * KW + warp) * R, re = row0 + rows;
-    // this CTA's share of the sum over j: rows [jb, je) of theta and grad
-    const int jb = share * j_chunk, je = min(N, jb + j_chunk);
-    const int ntiles = (je - jb + kTJ - 1) / kTJ;
+    // this CTA's share of the sum over j: rows [jb, je) of theta and grad, whole
+    // tiles (16-byte aligned TMA sources), as many as any other share or one more
+    const int nt = (N + kTJ - 1) / kTJ;
+    const int t0 = nt * share / shares, ntiles = nt * (share + 1) / shares - t0;
+    const int jb = t0 * kTJ, je = min(N, jb + ntiles * kTJ);
     const float inv_h = 1.f / __ldcg(h_dev);
 
     if (tid == 0) {
@@ -352,20 +368,21 @@ __device__ __forceinline__ bool phi_body(const float* __restrict__ theta,
         issue(0);
         if (ntiles > 1) issue(1);
     }
-    const float two_h = 2.f * inv_h;
-    float c[DP], dv[R], ksum[R];
-    f32x2 acc[R / 2][DP];   // rows 2 p and 2 p + 1
+    const f32x2 m2h = pack2(-2.f * inv_h, -2.f * inv_h);
+    float dv[R];
+    f32x2 acc[R / 2][DP], mti[R / 2][DP];   // rows 2 p and 2 p + 1: the sum, -theta_i
 #pragma unroll
-    for (int q = 0; q < DP; ++q) {
-        const int d = lane + 32 * q;
-        c[q] = d < D ? theta[d] : 0.f;
-    }
+    for (int p = 0; p < R / 2; ++p)
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        for (int q = 0; q < DP; ++q) acc[r / 2][q] = 0ull;
-        ksum[r] = 0.f;
+        for (int q = 0; q < DP; ++q) {
+            const int i = ib + 2 * p, d = lane + 32 * q;
+            acc[p][q] = 0ull;
+            mti[p][q] = pack2(i < re && d < D ? -theta[(size_t)i * D + d] : 0.f,
+                             i + 1 < re && d < D ? -theta[(size_t)(i + 1) * D + d] : 0.f);
+        }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
         dv[r] = (ib + r < re && jb + lane < je) ? d2[(size_t)(ib + r) * N + jb + lane] : 0.f;
-    }
     unsigned phases = 0u;                       // bit s: parity of stage s
     for (int t = 0; t < ntiles; ++t) {
         const int s = t & 1, j0 = jb + t * kTJ, nj = min(kTJ, je - j0);
@@ -377,11 +394,8 @@ __device__ __forceinline__ bool phi_body(const float* __restrict__ theta,
             for (int r = 0; r < R; ++r) {
                 const bool in = ib + r < re && lane < nj && j0 + lane != ib + r;
                 kv[r] = in ? expf(-dv[r] * inv_h) * wj : 0.f;
-                ksum[r] += kv[r];
             }
-#pragma unroll
-            for (int v = 0; v < R4; ++v)
-                Ks[(warp * kTJ + lane) * R4 + v] = make_float4(kv[4 * v], kv[4 * v + 1], kv[4 * v + 2], kv[4 * v + 3]);
+            Ks[warp * kTJ + lane] = make_float4(kv[0], kv[1], kv[2], kv[3]);
         }
         if (t + 1 < ntiles) {   // next tile's distances, consumed one iteration later
             const int jn = j0 + kTJ + lane;
@@ -407,34 +421,26 @@ __device__ __forceinline__ bool phi_body(const float* __restrict__ theta,
             return false;
         }
         phases ^= 1u << s;
-        const float* Tj = sm + 2 * s * sf;
-        float* Uj = sm + (2 * s + 1) * sf;
-        for (int jj = warp; jj < nj; jj += KW)   // u in place of g
-#pragma unroll
-            for (int q = 0; q < DP; ++q) {
-                const int d = lane + 32 * q;
-                if (d < D) Uj[jj * D + d] = fmaf(-two_h, Tj[jj * D + d] - c[q], Uj[jj * D + d]);
-            }
-        __syncthreads();
-        const float* up = Uj + lane;
-        const ulonglong2* kp = reinterpret_cast<const ulonglong2*>(Ks + warp * kTJ * R4);
+        const float* tp = sm + 2 * s * sf + lane;
+        const float* gp = tp + sf;
+        const ulonglong2* kp = reinterpret_cast<const ulonglong2*>(Ks + warp * kTJ);
         auto one_j = [&]() {
-            f32x2 kk[R / 2];
-#pragma unroll
-            for (int v = 0; v < R4; ++v) {
-                const ulonglong2 k4 = kp[v];
-                kk[2 * v] = k4.x;
-                kk[2 * v + 1] = k4.y;
-            }
+            const ulonglong2 k4 = *kp;
+            const f32x2 kk[2] = {k4.x, k4.y};
+            f32x2 tj[DP], gj[DP];
 #pragma unroll
             for (int q = 0; q < DP; ++q) {
-                const float u = up[32 * q];
-                const f32x2 uu = pack2(u, u);
-#pragma unroll
-                for (int p = 0; p < R / 2; ++p) acc[p][q] = fma2(kk[p], uu, acc[p][q]);
+                tj[q] = pack2(tp[32 * q], tp[32 * q]);
+                gj[q] = pack2(gp[32 * q], gp[32 * q]);
             }
-            up += D;
-            kp += R4;
+#pragma unroll
+            for (int p = 0; p < R / 2; ++p)
+#pragma unroll
+                for (int q = 0; q < DP; ++q)   // k (g_j - (2/h) (theta_j - theta_i))
+                    acc[p][q] = fma2(kk[p], fma2(m2h, add2(tj[q], mti[p][q]), gj[q]), acc[p][q]);
+            tp += D;
+            gp += D;
+            ++kp;
         };
         int jj = 0;
         if constexpr (UNROLL > 1)   // several j's shared-memory loads in flight
@@ -456,8 +462,6 @@ __device__ __forceinline__ bool phi_body(const float* __restrict__ theta,
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int i = ib + r;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ksum[r] += __shfl_xor_sync(0xffffffffu, ksum[r], o);
         const float self = i >= jb && i < je && i < re ? (wn ? wn[i] : 1.f) : 0.f;
 #pragma unroll
         for (int q = 0; q < DP; ++q) {
@@ -465,9 +469,9 @@ __device__ __forceinline__ bool phi_body(const float* __restrict__ theta,
             if (i < re && d < D) {
                 float a0, a1;
                 unpack2(acc[r / 2][q], a0, a1);
-                float v = fmaf(two_h * (theta[(size_t)i * D + d] - c[q]), ksum[r], r % 2 ? a1 : a0);
+                float v = r % 2 ? a1 : a0;
                 if (self != 0.f) v = fmaf(self, grad[(size_t)i * D + d], v);
-                out[(size_t)(i - row0) * D + d] = v * inv_n;
+                out[(size_t)(i - row0) * D + d] = __fmul_rn(v, inv_n);
             }
         }
     }
