@@ -108,6 +108,8 @@ __global__ void __launch_bounds__(128) rollout_adj_batch_kernel(const SimConst s
 }
 
 // ------------------------------ launch --------------------------------------
+constexpr size_t kMaxSmem = 227 * 1024;   // of a CTA
+
 template <int NB, int QL>
 cudaError_t launch(const SimConst& sc, const RolloutArgs& a, bool adjoint, cudaStream_t st) {
     const long long threads_total = (long long)a.N * a.lanes;
@@ -115,9 +117,14 @@ cudaError_t launch(const SimConst& sc, const RolloutArgs& a, bool adjoint, cudaS
     const int sms = sm_count();
     int cta = 32;
     while (cta < 128 && threads_total / (cta * 2) >= sms) cta *= 2;
+    if (!adjoint)
+        return launch_after(rollout_fwd_kernel<NB, QL>, dim3((unsigned)((threads_total + cta - 1) / cta)), cta, 0,
+                            st, sc, a);
+    // narrow teams with long segments: fewer of them per CTA, so that theirs fit
+    const size_t seg = seg_stride<NB>(sc.C) * sizeof(float2);
+    while (cta > 32 && cta / a.lanes * seg > kMaxSmem) cta /= 2;
     const int grid = (int)((threads_total + cta - 1) / cta);
-    if (!adjoint) return launch_after(rollout_fwd_kernel<NB, QL>, dim3(grid), cta, 0, st, sc, a);
-    const size_t smem = (size_t)(cta / a.lanes) * seg_stride<NB>(sc.C) * sizeof(float2);
+    const size_t smem = cta / a.lanes * seg;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(rollout_adj_kernel<NB, QL>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
