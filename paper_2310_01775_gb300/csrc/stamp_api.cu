@@ -258,16 +258,29 @@ stamp_status bandwidth(stamp_problem* p, const float* theta, int N, float* h_out
 }
 
 // Few particles: the whole step is one CTA's work (timed as STAMP_K_PHI).  A
-// wait made to run out (test hook) needs the Stein-direction kernel.
-bool small_step(const stamp_problem* p, int N) {
-    return N <= stamp::kSmallN && p->kernel_kind == 0 && !p->inject_wait_timeout;
+// wait made to run out (test hook) needs the Stein-direction kernel.  The bits do
+// not depend on the choice.  One CTA's time grows by 8 us per 100000 differences (N
+// N D) above some 17 us + D / 40 (9 us for up to 32 particles), the other kernels take
+// 24 us + 0.09 D at any N <= 64.  GB300, one CTA / kernels, us:
+//   N = 32   D = 12   9.1/24.2   D = 84  18.0/32.1   D = 288  37.3/49.7
+//   N = 40   D = 24  19.0/25.6   D = 84  31.2/32.3   D = 160  41.6/38.8   D = 288  60.6/50.2
+//   N = 48   D = 24  23.0/25.4   D = 56  29.3/28.7   D = 84   35.5/32.5   D = 288  76.4/50.8
+//   N = 64   D = 24  25.2/26.0   D = 36  33.3/28.1   D = 84   49.6/32.5   D = 288 111.3/51.7
+// beside: a solve can run the bandwidth beside its rollouts, which leaves the direction
+// and Adam on its path.  An iteration of such a solve, one CTA / kernels, us:
+//   N = 32   D = 12  72.0/73.6   D = 36  185/185   D = 84  206/202   D = 288  503/490
+//   N = 16   D = 84   198/200    D = 288  482/484;  N = 33   D = 12  83/77   D = 84  214/201
+bool small_step(const stamp_problem* p, int N, bool beside) {
+    if (N > stamp::kSmallN || p->kernel_kind != 0 || p->inject_wait_timeout) return false;
+    const int D = p->sc.D, differences = N * N * D;
+    return beside ? N <= 32 && differences <= 50000 : differences <= 80000 + 800 * D;
 }
 
 // bw_done: the RBF bandwidth of theta is already in p->h (launched beside the
-// rollouts and waited for).
+// rollouts and waited for).  Else beside: it could have been.
 stamp_status svgd(stamp_problem* p, float* theta, const float* grad, int N, float* m, float* v,
                   int step, float lr, int sgd_phase, float* h_out, float* phi_out,
-                  const float* wn = nullptr, bool bw_done = false) {
+                  const float* wn = nullptr, bool bw_done = false, bool beside = false) {
     const int D = p->sc.D;
     const float* part = grad;   // SGD phase: phi = grad log rho, one share
     int shares = 1;
@@ -293,7 +306,7 @@ stamp_status svgd(stamp_problem* p, float* theta, const float* grad, int N, floa
                                             p->phi, stamp::kMaxShares, &shares, p->stream);
         }));
         part = p->phi;
-    } else if (!sgd_phase && small_step(p, N)) {
+    } else if (!sgd_phase && !bw_done && small_step(p, N, beside)) {
         stamp::SvgdScratch s{p->d2, p->hist, p->sel, p->counter, p->h, p->flag};
         return timed(p, STAMP_K_PHI, [&] {
             return stamp::launch_small_step(theta, grad, N, D, m, v, wn, step, lr, s, h_out, phi_out,
@@ -393,7 +406,8 @@ stamp_status run_solve(stamp_problem* p, const Phases& ph, int N, unsigned long 
         unsigned* sw = stats_out ? p->stats + it : nullptr;
         const bool sgd = it >= (long long)ph.sur + ph.svgd;
         // the bandwidth needs theta only: start it beside this iteration's rollouts
-        const bool side_bw = p->overlap && !sgd && p->kernel_kind == 0 && N >= 2 && !small_step(p, N);
+        const bool beside = p->overlap && N >= 2;
+        const bool side_bw = beside && !sgd && p->kernel_kind == 0 && !small_step(p, N, true);
         if (side_bw) {
             STAMP_CUDA(cudaEventRecord(p->ev_theta, p->stream));
             STAMP_CUDA(cudaStreamWaitEvent(p->side, p->ev_theta, 0));
@@ -417,7 +431,7 @@ stamp_status run_solve(stamp_problem* p, const Phases& ph, int N, unsigned long 
         }
         if (side_bw) STAMP_CUDA(cudaStreamWaitEvent(p->stream, p->ev_h, 0));
         STAMP_TRY(svgd(p, th, p->grad, N, p->m, p->v, (int)it + 1, lr, sgd ? 1 : 0, nullptr,
-                       nullptr, wn, side_bw));
+                       nullptr, wn, side_bw, beside));
         if (p->check_every > 0 && (it + 1) % p->check_every == 0) {
             STAMP_TRY(hard_min(p, th, N, seed, p->cost, &p->best_hard));
             if (p->best_hard < p->target) {
