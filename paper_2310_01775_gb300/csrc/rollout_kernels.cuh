@@ -17,14 +17,14 @@ __device__ __forceinline__ bool real_team(int gtid, int lanes) {
     return (gtid & (lanes - 1)) < team_lanes(NB, QL);
 }
 
-template <int NB, int QL>
+template <int NB, int QL, bool kRows>
 __global__ void __launch_bounds__(128) rollout_fwd_kernel(const SimConst sc, const RolloutArgs a) {
     after_previous();
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
     int i = gtid / a.lanes;
     const bool on = i < a.N && real_team<NB, QL>(gtid, a.lanes);
     if (i >= a.N) i = a.N - 1;   // surplus teams shadow the last particle, store nothing
-    fwd_block_team<NB, QL>(sc, a, i, on);
+    fwd_block_team<NB, QL, kRows>(sc, a, i, on);
 }
 
 // Batched launch: team t -> (instance, particle) through the instances' first
@@ -117,9 +117,14 @@ cudaError_t launch(const SimConst& sc, const RolloutArgs& a, bool adjoint, cudaS
     const int sms = sm_count();
     int cta = 32;
     while (cta < 128 && threads_total / (cta * 2) >= sms) cta *= 2;
-    if (!adjoint)
-        return launch_after(rollout_fwd_kernel<NB, QL>, dim3((unsigned)((threads_total + cta - 1) / cta)), cta, 0,
-                            st, sc, a);
+    if (!adjoint) {
+        const dim3 grid((unsigned)((threads_total + cta - 1) / cta));
+        // one block on two lanes (N = 16384) is the other way round: 123 us, 128 without stores
+        if constexpr (NB > 1 || QL == 4)
+            if (sc.C > 1 && !a.full)
+                return launch_after(rollout_fwd_kernel<NB, QL, false>, grid, cta, 0, st, sc, a);
+        return launch_after(rollout_fwd_kernel<NB, QL, true>, grid, cta, 0, st, sc, a);
+    }
     // narrow teams with long segments: fewer of them per CTA, so that theirs fit
     const size_t seg = seg_stride<NB>(sc.C) * sizeof(float2);
     while (cta > 32 && cta / a.lanes * seg > kMaxSmem) cta /= 2;
