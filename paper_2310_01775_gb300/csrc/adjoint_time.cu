@@ -321,8 +321,7 @@ __global__ void relax_kernel(const SimConst sc, const RolloutArgs a, float* __re
 
 // The coefficients of particle i at substep t from the tape, one thread per (i, t).
 __global__ void __launch_bounds__(128) jac_kernel(const SimConst sc, const RolloutArgs a,
-                                                  const float* __restrict__ rel,
-                                                  float* __restrict__ coef) {
+                                                  const float* rel, float* __restrict__ coef) {
     after_previous();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int HT = sc.H * sc.T;
@@ -395,8 +394,7 @@ struct ScanSmem {
 };
 
 __global__ void __launch_bounds__(32) scan_kernel(const SimConst sc, const RolloutArgs a,
-                                                  const float* __restrict__ rel,
-                                                  const float* __restrict__ coef,
+                                                  const float* rel, const float* coef,
                                                   int* __restrict__ flag) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ScanSmem& sm = *reinterpret_cast<ScanSmem*>(smem_raw);

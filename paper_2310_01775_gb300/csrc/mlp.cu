@@ -220,8 +220,8 @@ __global__ void unpack_output_kernel(const float* __restrict__ ypad, int rows, i
 // dz_m (BF16 tiles) go to dzsave slot (m, tile_base + tile) for the weight
 // gradients; zsave holds the forward's pre-activations.
 __global__ void __launch_bounds__(kThreads, 1)
-mlp_bwd_kernel(const float* __restrict__ dy, int rows, int out_dim, int n_tiles,
-               const unsigned char* __restrict__ wt_tiled, const unsigned char* __restrict__ zsave,
+mlp_bwd_kernel(const float* dy, int rows, int out_dim, int n_tiles,
+               const unsigned char* wt_tiled, const unsigned char* zsave,
                unsigned char* __restrict__ dzsave, int tile_base, int tile_cap,
                float* __restrict__ dx, int in_dim, int* __restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -256,8 +256,11 @@ mlp_bwd_kernel(const float* __restrict__ dy, int rows, int out_dim, int n_tiles,
         const size_t slot = (size_t)tile_base + tile;
         if (half == 0) {   // dz_3 = dy as a BF16 K-major tile of 16 columns
             float d[kOut];
+            const float* dr = dy + (size_t)min(r, rows - 1) * out_dim;
 #pragma unroll
-            for (int c = 0; c < kOut; ++c) d[c] = (r < rows && c < out_dim) ? dy[(size_t)r * out_dim + c] : 0.f;
+            for (int c = 0; c < kOut; ++c) d[c] = dr[c < out_dim ? c : 0];   // no branch: all in flight
+#pragma unroll
+            for (int c = 0; c < kOut; ++c) d[c] = (r < rows && c < out_dim) ? d[c] : 0.f;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 uint4 pk;
@@ -307,13 +310,17 @@ mlp_bwd_kernel(const float* __restrict__ dy, int rows, int out_dim, int n_tiles,
                 const unsigned char* zt = zsave + ((size_t)(m - 1) * tile_cap + slot) * kActBytes;
                 unsigned char* dzt = dzsave + ((size_t)(m - 1) * tile_cap + slot) * kActBytes;
                 for (int c0 = half * (kHidden / kParts); c0 < (half + 1) * (kHidden / kParts); c0 += 32) {
+                    uint4 zq[4];   // before the read of tensor memory, which they may not pass
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        zq[q] = *reinterpret_cast<const uint4*>(zt + tile_off(row, c0 + q * 8, kHidden));
                     float v[32];
                     tmem_ld32(lane_base + c0, v);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const unsigned off = tile_off(row, c0 + q * 8, kHidden);
-                        const uint4 zq = *reinterpret_cast<const uint4*>(zt + off);
-                        const unsigned zw[4] = {zq.x, zq.y, zq.z, zq.w};
+                        const uint4 zv = zq[q];
+                        const unsigned zw[4] = {zv.x, zv.y, zv.z, zv.w};
                         uint4 pk;
                         unsigned* pw = reinterpret_cast<unsigned*>(&pk);
 #pragma unroll

@@ -135,7 +135,9 @@ cudaError_t launch_adjoint_time(const SimConst& sc, const RolloutArgs& a, float*
 // (programmatic stream serialisation): about 2 us less between two short
 // kernels (GB300: the Stein step of 2048 particles, five kernels, 95 -> 86 us).
 // The kernel must call after_previous() before it touches global memory; that
-// waits until everything before it is complete and visible.
+// waits until everything before it is complete and visible.  What it reads then it
+// reads with ordinary loads: its const arguments are not __restrict__, and it uses no
+// __ldg (the read-only path is for data that nothing writes while the kernel runs).
 template <class... P, class... A>
 cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                          const A&... args) {

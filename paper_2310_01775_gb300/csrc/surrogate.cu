@@ -75,8 +75,8 @@ features_kernel(const SimConst sc, const float* __restrict__ theta, int N, int k
 // + w_push sum_k dist_k^2 and, when apose is given, dC/dq_H.
 template <int NB>
 __global__ void __launch_bounds__(128)
-cost_kernel(const SimConst sc, int N, const float* __restrict__ src, const float* __restrict__ delta,
-            const float* __restrict__ relax, float* __restrict__ cost, float* __restrict__ apose,
+cost_kernel(const SimConst sc, int N, const float* src, const float* delta,
+            const float* relax, float* __restrict__ cost, float* __restrict__ apose,
             unsigned* __restrict__ stats_min) {
     after_previous();
     constexpr int M = rollout::Dims<NB>::M, P = M + 2;
@@ -191,7 +191,7 @@ __device__ __forceinline__ unsigned cost_key(float cost) {   // a negative or Na
     const unsigned cb = __float_as_uint(cost);
     return cb >= 0x7F800001u ? 0xFFFFFFFFu : cb;
 }
-__global__ void __launch_bounds__(256) select_pass_kernel(const float* __restrict__ cost, int n, int N,
+__global__ void __launch_bounds__(256) select_pass_kernel(const float* cost, int n, int N,
                                                           int p, Select s) {
     __shared__ unsigned h[kSelBins], st[24];
     after_previous();
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(256) select_pass_kernel(const float* __restric
         }
     }
 }
-__global__ void __launch_bounds__(256) select_gather_kernel(const float* __restrict__ cost, int n, Select s,
+__global__ void __launch_bounds__(256) select_gather_kernel(const float* cost, int n, Select s,
                                                             unsigned long long* __restrict__ out) {
     after_previous();
     const unsigned* st = s.state;
@@ -232,8 +232,8 @@ __global__ void __launch_bounds__(256) select_gather_kernel(const float* __restr
     if (key <= last) out[atomicAdd(s.state + 5, 1u)] = key;
 }
 // Places of 8 of the N pairs per CTA (a warp each), and their candidates' copies.
-__global__ void __launch_bounds__(256) select_place_kernel(const unsigned long long* __restrict__ keys,
-                                                           int N, int D, const float* __restrict__ cand,
+__global__ void __launch_bounds__(256) select_place_kernel(const unsigned long long* keys,
+                                                           int N, int D, const float* cand,
                                                            float* __restrict__ theta,
                                                            int* __restrict__ index) {
     after_previous();

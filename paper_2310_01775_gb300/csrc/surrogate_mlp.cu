@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(kThreads, 1) sur_fwd_cluster_kernel(const SimC
     }
     float bias[3];
 #pragma unroll
-    for (int l = 0; l < 3; ++l) bias[l] = __ldg(a.bias + l * kHidden + s.rank * kUnits + s.unit);
+    for (int l = 0; l < 3; ++l) bias[l] = a.bias[l * kHidden + s.rank * kUnits + s.unit];
     float q[S3];
 #pragma unroll
     for (int t = 0; t < S3; ++t) q[t] = sc.init[t / 3][t % 3];
@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(kThreads, 1) sur_fwd_cluster_kernel(const SimC
             const float* bl = a.bias + 3 * kHidden;
             float d[S3];
 #pragma unroll
-            for (int t = 0; t < S3; ++t) d[t] = v[t] + __ldg(bl + t);
+            for (int t = 0; t < S3; ++t) d[t] = v[t] + bl[t];
             if (k + 1 == sc.H) {   // the cost adds the last pose change itself
                 if (on && first)
 #pragma unroll

@@ -169,12 +169,10 @@ __global__ void __launch_bounds__(256) median_digit_batch_kernel(const SvgdInst*
 // the bound, N = 4096, D = 144: 392 -> 383).
 constexpr int phi_resident(int DP) { return DP <= 3 ? 4 : DP <= 4 ? 3 : 2; }
 template <int DP>
-__global__ void __launch_bounds__(kW * 32, phi_resident(DP)) phi_kernel(const float* __restrict__ theta,
-                                                      const float* __restrict__ grad, int N, int D,
-                                                      const float* __restrict__ d2,
-                                                      const float* __restrict__ h_dev,
+__global__ void __launch_bounds__(kW * 32, phi_resident(DP)) phi_kernel(const float* theta, const float* grad,
+                                                      int N, int D, const float* d2, const float* h_dev,
                                                       float* __restrict__ part, int shares,
-                                                      int* err, const float* __restrict__ wn,
+                                                      int* err, const float* wn,
                                                       unsigned wait_limit, int skip_first, int row0,
                                                       int rows) {
     after_previous();
@@ -198,7 +196,7 @@ __global__ void __launch_bounds__(kW * 32) phi_batch_kernel(const SvgdInst* __re
 // Adam (Kingma & Ba 2015) with gradient -phi, phi the in-order sum of the
 // `shares` partial directions (stride n); optionally stores phi.  Flags
 // non-finite inputs/results.
-__global__ void adam_kernel(float* __restrict__ theta, const float* __restrict__ part, int shares,
+__global__ void adam_kernel(float* __restrict__ theta, const float* part, int shares,
                             float* __restrict__ phi_out, float* __restrict__ m,
                             float* __restrict__ v, int n, float lr, float bc1, float bc2,
                             int* flag) {

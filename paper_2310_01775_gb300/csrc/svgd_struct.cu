@@ -60,10 +60,9 @@ constexpr int kCtaRows = kWarps / kSplit * (32 / HP) * kRows;
 
 template <int M, int HP>
 __global__ void __launch_bounds__(kWarps * 32)
-struct_phi_kernel(const float* __restrict__ theta, const float* __restrict__ grad,
-                  const float* __restrict__ S, int N, int H,
-                  const float* __restrict__ hc_dev, const float* __restrict__ hz_dev,
-                  const float* __restrict__ wn, float* __restrict__ phi, int j_chunk) {
+struct_phi_kernel(const float* theta, const float* grad, const float* S, int N, int H,
+                  const float* hc_dev, const float* hz_dev, const float* wn, float* __restrict__ phi,
+                  int j_chunk) {
     extern __shared__ float ssm[];
     constexpr int P = M + 2, kGroups = 32 / HP;
     const int D = H * P;
@@ -75,7 +74,7 @@ struct_phi_kernel(const float* __restrict__ theta, const float* __restrict__ gra
     const int row0 = (warp / kSplit * kGroups + lane / HP) * kRows, i0 = blockIdx.x * kCtaRows<HP>;
     after_previous();
     const float Hf = (float)H;
-    const float inv_hc = Hf / __ldg(hc_dev), inv_hz = Hf / __ldg(hz_dev);   // h = h_plain / H
+    const float inv_hc = Hf / *hc_dev, inv_hz = Hf / *hz_dev;   // h = h_plain / H
     const float alpha = 0.5f / Hf, ac = alpha * (2.f * inv_hc), az = alpha * (2.f * inv_hz);
     float xi[kRows][P], acc[kRows][P];
 #pragma unroll
