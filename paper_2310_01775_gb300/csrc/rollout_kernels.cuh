@@ -161,7 +161,8 @@ cudaError_t launch_batch(const SimConst& sc, const BatchArgs& b, int cta, bool a
     return cudaGetLastError();
 }
 
-// By lanes per particle (every count lanes_supported accepts): 1, 2 or 4 per block.
+// By lanes per particle: 1, 2 or 4 per block.  Four blocks never run on one
+// (lanes_supported, default_lanes), and three do only alone, from some count on.
 constexpr int lanes_per_block(int nb, int lanes) {
     const int q = lanes / team_groups(nb);
     return q < 4 ? q : 4;
@@ -170,7 +171,9 @@ template <int NB>
 cudaError_t launch_lanes(const SimConst& sc, RolloutArgs a, int lanes, bool adjoint, cudaStream_t st) {
     a.lanes = lanes;
     switch (lanes_per_block(NB, lanes)) {
-        case 1: return launch<NB, 1>(sc, a, adjoint, st);
+        case 1:
+            if constexpr (NB < 4) return launch<NB, 1>(sc, a, adjoint, st);
+            break;
         case 2: return launch<NB, 2>(sc, a, adjoint, st);
         case 4: return launch<NB, 4>(sc, a, adjoint, st);
     }
@@ -181,7 +184,9 @@ cudaError_t launch_batch_lanes(const SimConst& sc, BatchArgs b, int lanes, int c
                                cudaStream_t st) {
     b.lanes = lanes;
     switch (lanes_per_block(NB, lanes)) {
-        case 1: return launch_batch<NB, 1>(sc, b, cta, adjoint, st);
+        case 1:
+            if constexpr (NB < 3) return launch_batch<NB, 1>(sc, b, cta, adjoint, st);
+            break;
         case 2: return launch_batch<NB, 2>(sc, b, cta, adjoint, st);
         case 4: return launch_batch<NB, 4>(sc, b, cta, adjoint, st);
     }

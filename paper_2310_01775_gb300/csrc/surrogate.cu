@@ -31,29 +31,19 @@ constexpr int kChunk = 4096;         // transitions per chunk (one key each)
 constexpr int kTrainRows = 16384;    // largest training minibatch
 constexpr int kAttempts = 32;        // rejection-sampling attempts per start scene
 
-// Features of push k (and the stored relaxation).  Pose source: the scene's
-// start poses (src NULL), else src (+ delta when given); the pose used is
-// written to pose_out when given.
+// Features of N one-push plans from given start poses (N x 3 n_blocks).
 template <int NB>
 __global__ void __launch_bounds__(128)
-features_kernel(const SimConst sc, const float* __restrict__ theta, int N, int k, uint64_t seed,
-                int iter, const float* __restrict__ src, const float* __restrict__ delta,
-                float* __restrict__ pose_out, float* __restrict__ x, float* __restrict__ relax) {
-    constexpr int M = rollout::Dims<NB>::M, P = M + 2, IN = 8 * NB + 2;
+features_kernel(const SimConst sc, const float* __restrict__ theta, int N, uint64_t seed, int iter,
+                const float* __restrict__ start, float* __restrict__ x) {
+    constexpr int M = rollout::Dims<NB>::M, IN = 8 * NB + 2;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    float q[3 * NB];
-#pragma unroll
-    for (int t = 0; t < 3 * NB; ++t) {
-        q[t] = src ? src[(size_t)i * 3 * NB + t] : sc.init[t / 3][t % 3];
-        if (delta) q[t] += delta[(size_t)i * 3 * NB + t];
-        if (pose_out) pose_out[(size_t)i * 3 * NB + t] = q[t];
-    }
     const bool noise = iter >= 0;
     const uint64_t gkey = noise ? sm64(sm64(seed, kStreamGumbel), (uint64_t)iter) : 0ull;
     float z[M], uu, vv;
-    rollout::relax_action<NB>(sc, theta + (size_t)i * sc.D, k, i, gkey, noise, false, z, uu, vv);
-    const float tu = tanhf(uu), sv = rollout::sigmoidf_(vv);
+    rollout::relax_action<NB>(sc, theta + (size_t)i * sc.D, 0, i, gkey, noise, false, z, uu, vv);
+    const float* q = start + (size_t)i * 3 * NB;
     float* xi = x + (size_t)i * IN;
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
@@ -64,11 +54,10 @@ features_kernel(const SimConst sc, const float* __restrict__ theta, int N, int k
         xi[4 * b + 2] = cs;
         xi[4 * b + 3] = sn;
     }
-    float* ri = relax + ((size_t)i * sc.H + k) * P;
 #pragma unroll
-    for (int c = 0; c < M; ++c) xi[4 * NB + c] = ri[c] = z[c];
-    xi[4 * NB + M] = ri[M] = tu;
-    xi[4 * NB + M + 1] = ri[M + 1] = sv;
+    for (int c = 0; c < M; ++c) xi[4 * NB + c] = z[c];
+    xi[4 * NB + M] = tanhf(uu);
+    xi[4 * NB + M + 1] = rollout::sigmoidf_(vv);
 }
 
 // q_H = q_{H-1} + delta; C = sum_b |p_b - g_b|^2 + w_yaw wrap(phi_b - phi_gb)^2
@@ -356,11 +345,9 @@ __global__ void head_scale_kernel(const float* __restrict__ src, float* __restri
 }
 
 template <int NB>
-cudaError_t features(const SimConst& sc, const float* theta, int N, int k, uint64_t seed, int iter,
-                     const float* src, const float* delta, float* pose_out, float* x, float* relax,
-                     cudaStream_t st) {
-    features_kernel<NB><<<(N + 127) / 128, 128, 0, st>>>(sc, theta, N, k, seed, iter, src, delta,
-                                                         pose_out, x, relax);
+cudaError_t features(const SimConst& sc, const float* theta, int N, uint64_t seed, int iter,
+                     const float* start, float* x, cudaStream_t st) {
+    features_kernel<NB><<<(N + 127) / 128, 128, 0, st>>>(sc, theta, N, seed, iter, start, x);
     return cudaGetLastError();
 }
 template <int NB>
@@ -368,13 +355,12 @@ cudaError_t cost(const SimConst& sc, int N, const float* src, const float* delta
                  float* c, float* apose, unsigned* stats, cudaStream_t st) {
     return launch_after(cost_kernel<NB>, dim3((N + 127) / 128), 128, 0, st, sc, N, src, delta, relax, c, apose, stats);
 }
-cudaError_t features_nb(const SimConst& sc, const float* theta, int N, int k, uint64_t seed, int iter,
-                        const float* src, const float* delta, float* pose_out, float* x, float* relax,
-                        cudaStream_t st) {
+cudaError_t features_nb(const SimConst& sc, const float* theta, int N, uint64_t seed, int iter,
+                        const float* start, float* x, cudaStream_t st) {
     switch (sc.nb) {
-        case 1: return features<1>(sc, theta, N, k, seed, iter, src, delta, pose_out, x, relax, st);
-        case 2: return features<2>(sc, theta, N, k, seed, iter, src, delta, pose_out, x, relax, st);
-        case 3: return features<3>(sc, theta, N, k, seed, iter, src, delta, pose_out, x, relax, st);
+        case 1: return features<1>(sc, theta, N, seed, iter, start, x, st);
+        case 2: return features<2>(sc, theta, N, seed, iter, start, x, st);
+        case 3: return features<3>(sc, theta, N, seed, iter, start, x, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -613,8 +599,8 @@ stamp_status stamp_surrogate_transitions(stamp_surrogate* s, int n, unsigned lon
         stamp::surrogate::sample_actions_kernel<<<(m * P + 255) / 256, 256, 0, s->stream>>>(m, s->M, cs, s->taction);
         SUR_CUDA(cudaGetLastError(), "sampling launch failed");
         SUR_TRY(stamp::rollout_from(s->trans, s->taction, s->tstart, m, cs, 0, s->tcost, s->tfinal));
-        SUR_CUDA(stamp::surrogate::features_nb(sc1, s->taction, m, 0, cs, 0, s->tstart, nullptr, nullptr,
-                                               x_out + (size_t)c0 * s->in_dim, s->relax, s->stream),
+        SUR_CUDA(stamp::surrogate::features_nb(sc1, s->taction, m, cs, 0, s->tstart, x_out + (size_t)c0 * s->in_dim,
+                                               s->stream),
                  "feature launch failed");
         stamp::surrogate::delta_kernel<<<(m * S3 + 255) / 256, 256, 0, s->stream>>>(
             m, nb, s->tstart, s->tfinal, y_out + (size_t)c0 * S3);

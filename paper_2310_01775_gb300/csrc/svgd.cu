@@ -1,4 +1,3 @@
-#include <climits>
 // Stein update of Algorithm 1 (Eq. svgd with unit weights), its median
 // bandwidth, Adam, the initial particles and the final distinct-plan top-k.
 //
@@ -10,6 +9,8 @@
 // in L2 (4 MB at N = 1024).  Each pass histograms one digit; the last CTA of
 // the pass to finish (a device-scope counter, no waiting) picks the digit for
 // the next pass, and the last pass writes h.
+#include <climits>
+
 #include "svgd_bodies.cuh"
 
 namespace stamp {
