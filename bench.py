@@ -289,6 +289,7 @@ def small_requests(stream, n=512, N=32, iters=40):
         insts.append({"n_blocks": nb, "H": H, "N": N, "seed": 50021 + g, "init": init, "goal": goal})
     b = S.Batch(dict(W.PHYSICS, T=100), insts, stream)
     b.autotune(2)
+    cfg = {str(nb): dict(zip(("lanes", "cta", "ckpt_every"), b.get_config(nb))) for nb in range(1, 5)}
     persistent, _, _ = b.persistent()
     ms = {}
     for name, flag in (("per_class", False), ("persistent", True)):
@@ -299,7 +300,7 @@ def small_requests(stream, n=512, N=32, iters=40):
     units = sum(d["N"] * d["H"] * 100 for d in insts)
     b.close()
     return {"instances": n, "particles_each": N, "launch_mode": "persistent" if persistent else "per-class",
-            "ms_per_iteration_all_active": ms,
+            "config_per_block_count": cfg, "ms_per_iteration_all_active": ms,
             "value": units / (min(ms.values()) / 1e3), "unit": UNIT,
             "over": f"{iters} graph-replayed iterations, solve wall time incl. initialisation and "
                     f"final evaluation / {iters}"}
