@@ -40,7 +40,8 @@ FP32_LANES = 128                    # FP32 lanes per SM; 1 FMA = 2 FLOP
 # DRAM bytes (read + write) per launch of a rollout kernel, from one cold-cache ncu
 # capture of the workload, valid while the kernel sources are unchanged
 # (sha256 prefix over the rollout sources at capture time).
-TRAFFIC = {}
+TRAFFIC = {("pusher3_h6", "rollout_adj"): ("e21688d2934713fc", 89.4e6),
+           ("pusher3_h6", "rollout_fwd"): ("e21688d2934713fc", 33.5e6)}
 ROLLOUT_SOURCES = ("rollout.cuh", "block_team.cuh", "rollout_kernels.cuh", "adjoint_time.cu")
 
 

@@ -23,9 +23,9 @@
 //
 // Measured on GB300, three blocks, N = 2048, H = 6, T = 100, C = 25, softer
 // contact (us, forward + reverse sweep): 512 + 815 with every state on every
-// lane and all pairs dealt round-robin over 8 lanes; 161 + 279 here with QL = 2
-// (173 + 306 with QL = 4).  Four blocks, N = 613, H = 5: 539 + 901 against 255 + 355
-// (QL = 4).
+// lane and all pairs dealt round-robin over 8 lanes; 155 + 279 here with QL = 2.
+// Four blocks, N = 613, H = 5, both together: 1184 on scenes whose blocks stay apart,
+// up to 1464 where they meet, against 278 and up to 726 (QL = 4).
 //
 // The results' bits do not depend on QL, nor on the number of particles that a
 // width is picked by: every value that belongs to a side of a block (a contact's
